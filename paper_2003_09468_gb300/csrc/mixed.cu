@@ -206,12 +206,26 @@ static cudaError_t map5_pair(CUtensorMap* m, void* base, uint64_t d0, uint64_t d
 // ---------------------------------------------------------------------------
 // GEMM policies
 // ---------------------------------------------------------------------------
+// The epilogues (store_tile) run on 256 threads beside the next tile's MMAs.  With 128 threads
+// and per-element index arithmetic they were the longest part of a tile of few k chunks (3x3x3
+// system, 64 walkers: Green's function 130 us per launch against 39 with the stores left out,
+// vHS 499 / 172, exchange 780 / 426), so a thread keeps one column (or row) of the tile, all
+// divisions and scale factors are formed once per tile, before the tile is waited for, and
+// whatever the tile is combined with is loaded before that wait too.
+constexpr int ST = tcg::STORE_THREADS;
+// scales are powers of two: the reciprocal is exact, and a product with it is the quotient
+__device__ __forceinline__ float rcp2(float s) { return __frcp_rn(s); }
+// x * s of two neighbours as fp16 hi and lo pairs (split_val on both, packed conversions)
+__device__ __forceinline__ void split_pair(float x0, float x1, __half2& hi, __half2& lo) {
+  hi = __floats2half2_rn(x0, x1);
+  const float2 h = __half22float2(hi);
+  lo = __floats2half2_rn(x0 - h.x, x1 - h.y);
+}
 
 // Gh[ws] = B^T + S^-T phi_perp^T : rows i = (k1, a), cols (k2, p); written to g32 in tile
 // layout.  B = A (A^dag A)^-1 and phi_perp = phi - B S (see green()).
 struct GreenP {
   static constexpr bool kConjA = false;
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES;
   int tiles, kchunks;
   int mt_n, nt_n, N, NM, n, M, Mp, nk, WS;
@@ -228,13 +242,19 @@ struct GreenP {
     tcg::Coords c = {{kc * 32, mt * 128, 0, b, 0}, {kc * 32, nt * BN, 0, 0, b}};
     return c;
   }
-  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, int) const {
-    const float st = 1.f / (s_sinv[b] * s_phi[b]);
-    for (int e = tid; e < 128 * BN; e += 128) {
-      const int r = e / BN, c = e % BN;
-      const int i = mt * 128 + r, col = nt * BN + c;
-      if (i >= N || col >= NM) continue;
-      const int k1 = i / n, a = i % n, k2 = col / M, p = col % M;
+  template <class R>
+  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, R ready) const {
+    const int c = tid % BN, col = nt * BN + c, k2 = col / M, p = col - k2 * M;
+    const float st = rcp2(s_sinv[b] * s_phi[b]), inv_n = 1.f / (float)n;
+    const size_t blk = (size_t)WS * n * Mp;
+    float2* o = g32 + (size_t)k2 * blk + (size_t)b * n * Mp + p;
+    if (!ready() || col >= NM) return;
+#pragma unroll 4
+    for (int r = tid / BN; r < 128; r += ST / BN) {
+      const int i = mt * 128 + r;
+      if (i >= N) break;
+      // i / n: (i + 1/2) / n is at least 1 / 2n from the next integer, far more than its rounding
+      const int k1 = __float2int_rz(((float)i + 0.5f) * inv_n), a = i - k1 * n;
       const float2 v = tile[r * tcg::STAGE_LD + c];
       float gr = v.x * st, gi = v.y * st;
       if (k1 == k2) {
@@ -242,7 +262,7 @@ struct GreenP {
         gr += bp.x;
         gi += bp.y;
       }
-      g32[((((size_t)k1 * nk + k2) * WS + b) * n + a) * Mp + p] = make_float2(gr, gi);
+      o[(size_t)k1 * nk * blk + (size_t)a * Mp] = make_float2(gr, gi);
     }
   }
 };
@@ -255,7 +275,6 @@ struct GreenP {
 // walker), so the blocks of a group add in one fp32 running sum.
 struct ForceBiasP {
   static constexpr bool kConjA = false;
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES_LIGHT;
   int tiles, kchunks;
   int mt_n, nt_n, W, G, nk, ng, kg, kcb;   // ng groups of kg k blocks, kcb chunks per block
@@ -274,16 +293,21 @@ struct ForceBiasP {
     tcg::Coords c = {{c0, mt * 128, 0, k, Q}, {c0, nt * BN, 0, 0, k * nk + kminus[k * nk + Q]}};
     return c;
   }
-  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, int) const {
+  // down the rows: consecutive threads write consecutive g of one walker
+  template <class R>
+  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, R ready) const {
     const int Q = b / ng, grp = b % ng;
-    // down the rows: consecutive threads write consecutive g of one walker
-    for (int e = tid; e < 128 * BN; e += 128) {
-      const int r = e % 128, c = e / 128;
-      const int g = mt * 128 + r, w = nt * BN + c;
-      if (w >= W || g >= G) continue;
-      const float f = inv_s_lh[Q * G + g] / s_gsum[w];
+    const int r = tid % 128, g = mt * 128 + r;
+    const float fg = g < G ? inv_s_lh[Q * G + g] : 0.f;
+    double2* o = Xk + (((size_t)grp * W + nt * BN) * nk + Q) * G + g;
+    if (!ready() || g >= G) return;
+#pragma unroll 4
+    for (int c = tid / 128; c < BN; c += ST / 128) {
+      const int w = nt * BN + c;
+      if (w >= W) break;
+      const float f = fg * rcp2(s_gsum[w]);
       const float2 v = tile[r * tcg::STAGE_LD + c];
-      Xk[(((size_t)grp * W + w) * nk + Q) * G + g] = make_double2((double)(v.x * f), (double)(v.y * f));
+      o[(size_t)c * nk * G] = make_double2((double)(v.x * f), (double)(v.y * f));
     }
   }
 };
@@ -304,7 +328,6 @@ __global__ void xsum_kernel(const double2* Xk, zc* X, int ng, size_t per) {
 // V[w][(k,p)][(k-Q,r)] = sum_g y[w,Q,g] L[Q,k,g,p,r]  -> split planes with a fixed scale
 struct VhsP {
   static constexpr bool kConjA = false;
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES;
   int tiles, kchunks;
   int mt_n, nt_n, W, M, nk, NM, NMp;
@@ -323,45 +346,48 @@ struct VhsP {
     tcg::Coords c = {{kc * 32, mt * 128, 0, k, Q}, {kc * 32, nt * BN, 0, 0, Q}};
     return c;
   }
-  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, int) const {
+  template <class R>
+  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, R ready) const {
     const int Q = b / nk, k = b % nk, kq = kminus[k * nk + Q];
     const size_t ps = (size_t)NM * NMp;
+    const float* sy = s_y + Q * W + nt * BN;
+    const int wn = min(BN, W - nt * BN);
     bool bad = false;
     if ((M & 1) == 0) {
       // M even: rows 2i, 2i+1 of a tile are r, r+1 of one (p, r) run and land on one
-      // 4-byte aligned pair of the output row, so each plane takes one 32-bit store
-      for (int e = tid; e < 64 * BN; e += 128) {
-        const int rp = e % 64, c = e / 64;
-        const int pr = mt * 128 + 2 * rp, w = nt * BN + c;
-        if (w >= W || pr >= M * M) continue;
-        const float st = V_SCALE / s_y[Q * W + w];
+      // 4-byte aligned pair of the output row, so each plane takes one 32-bit store; a thread
+      // keeps one row pair and walks over the walkers
+      const int rp = tid % 64, pr = mt * 128 + 2 * rp, pp = pr / M, rr = pr - pp * M;
+      __half* o = v_sp + (size_t)nt * BN * 4 * ps + (size_t)(k * M + pp) * NMp + kq * M + rr;
+      if (!ready() || pr >= M * M) return;
+#pragma unroll 4
+      for (int c = tid / 64; c < wn; c += ST / 64) {
+        const float st = V_SCALE * rcp2(sy[c]);
         const float2 v0 = tile[(2 * rp) * tcg::STAGE_LD + c], v1 = tile[(2 * rp + 1) * tcg::STAGE_LD + c];
         const float r0 = v0.x * st, i0 = v0.y * st, r1 = v1.x * st, i1 = v1.y * st;
         bad |= !(fmaxf(fmaxf(fabsf(r0), fabsf(i0)), fmaxf(fabsf(r1), fabsf(i1))) < 60000.f);
-        const int pp = pr / M, rr = pr % M;
-        __half* base = v_sp + (size_t)w * 4 * ps + (size_t)(k * M + pp) * NMp + kq * M + rr;
-        __half h0, l0, h1, l1;
-        split_val(r0, h0, l0);
-        split_val(r1, h1, l1);
-        *reinterpret_cast<__half2*>(base) = __halves2half2(h0, h1);
-        *reinterpret_cast<__half2*>(base + ps) = __halves2half2(l0, l1);
-        split_val(i0, h0, l0);
-        split_val(i1, h1, l1);
-        *reinterpret_cast<__half2*>(base + 2 * ps) = __halves2half2(h0, h1);
-        *reinterpret_cast<__half2*>(base + 3 * ps) = __halves2half2(l0, l1);
+        __half* base = o + (size_t)c * 4 * ps;
+        __half2 hi, lo;
+        split_pair(r0, r1, hi, lo);
+        *reinterpret_cast<__half2*>(base) = hi;
+        *reinterpret_cast<__half2*>(base + ps) = lo;
+        split_pair(i0, i1, hi, lo);
+        *reinterpret_cast<__half2*>(base + 2 * ps) = hi;
+        *reinterpret_cast<__half2*>(base + 3 * ps) = lo;
       }
     } else {
       // down the rows: consecutive threads write consecutive r of one (walker, p)
-      for (int e = tid; e < 128 * BN; e += 128) {
-        const int r = e % 128, c = e / 128;
-        const int pr = mt * 128 + r, w = nt * BN + c;
-        if (w >= W || pr >= M * M) continue;
-        const float st = V_SCALE / s_y[Q * W + w];
+      const int r = tid % 128, pr = mt * 128 + r, pp = pr / M, rr = pr - pp * M;
+      __half* o = v_sp + (size_t)nt * BN * 4 * ps;
+      const size_t at = (size_t)(k * M + pp) * NMp + kq * M + rr;
+      if (!ready() || pr >= M * M) return;
+#pragma unroll 4
+      for (int c = tid / 128; c < wn; c += ST / 128) {
+        const float st = V_SCALE * rcp2(sy[c]);
         const float2 v = tile[r * tcg::STAGE_LD + c];
         const float vr = v.x * st, vi = v.y * st;
         bad |= !(fabsf(vr) < 60000.f && fabsf(vi) < 60000.f);
-        const int pp = pr / M, rr = pr % M;
-        put4f(v_sp + (size_t)w * 4 * ps, ps, (size_t)(k * M + pp) * NMp + kq * M + rr, vr, vi);
+        put4f(o + (size_t)c * 4 * ps, ps, at, vr, vi);
       }
     }
     if (bad) atomicExch(overflow, 1);
@@ -378,7 +404,6 @@ struct VhsP {
 //   last step:   acc = phi' (FP64) + V u, the identity part exact.
 struct TaylorP {
   static constexpr bool kConjA = false;
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES;
   int tiles, kchunks;
   int mt_n, nt_n, R, NM, NMp;
@@ -397,85 +422,97 @@ struct TaylorP {
     tcg::Coords c = {{kc * 32, mt * 128, 0, b, 0}, {kc * 32, nt * BN, 0, 0, b}};
     return c;
   }
-  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, int) const {
+  // Elements are taken in batches of U per thread, the next batch's loads issued before this
+  // one's stores (the first batch's before the tile is waited for).
+  template <int COUNT, class V, class L, class S, class R>
+  static __device__ __forceinline__ void batches(int tid, L load, S store, R ready) {
+    constexpr int U = 8, NB = COUNT / (ST * U);
+    static_assert(NB * ST * U == COUNT, "whole batches");
+    V cur[U], nxt[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) cur[u] = load(tid + ST * u);
+    if (!ready()) return;
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      if (n + 1 < NB) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) nxt[u] = load(tid + ST * (U * (n + 1) + u));
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) store(tid + ST * (U * n + u), cur[u]);
+      if (n + 1 < NB) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) cur[u] = nxt[u];
+      }
+    }
+  }
+  template <class RD>
+  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, RD ready) const {
     const float st = inv_j / V_SCALE, sc = s_t[b];
-    // all U reads of a batch are issued before its writes, so they overlap
     if (last) {
-      constexpr int U = 8;
-      const float inv_s = 1.f / sc;   // power of two: exact
+      const float inv_s = rcp2(sc);
       float4* cb = corr + (size_t)b * R * NM;
       const float2* pb = p32 + (size_t)b * R * NM;
-      for (int e0 = tid; e0 < 128 * BN; e0 += 128 * U) {
-        float2 dv[U], pv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = e0 + 128 * u, j = mt * 128 + e / BN, i = nt * BN + e % BN;
-          if (j < R && i < NM) {
+      batches<128 * BN, float4>(
+          tid,
+          [&](int e) {
+            const int j = mt * 128 + e / BN, i = nt * BN + e % BN;
+            if (j >= R || i >= NM) return make_float4(0.f, 0.f, 0.f, 0.f);
             const size_t o = (size_t)j * NM + i;
-            dv[u] = reinterpret_cast<const float2*>(cb)[2 * o];
-            pv[u] = pb[o];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = e0 + 128 * u, r = e / BN, c = e % BN, j = mt * 128 + r, i = nt * BN + c;
-          if (j >= R || i >= NM) continue;
-          const float2 v = tile[r * tcg::STAGE_LD + c];
-          const float vr = v.x * st * inv_s, vi = v.y * st * inv_s;   // V u
-          cb[(size_t)j * NM + i] = make_float4(dv[u].x + vr, dv[u].y + vi, pv[u].x + vr, pv[u].y + vi);
-        }
-      }
+            const float2 d = reinterpret_cast<const float2*>(cb)[2 * o], q = pb[o];
+            return make_float4(d.x, d.y, q.x, q.y);
+          },
+          [&](int e, const float4& x) {
+            const int r = e / BN, c = e % BN, j = mt * 128 + r, i = nt * BN + c;
+            if (j >= R || i >= NM) return;
+            const float2 v = tile[r * tcg::STAGE_LD + c];
+            const float vr = v.x * st * inv_s, vi = v.y * st * inv_s;   // V u
+            cb[(size_t)j * NM + i] = make_float4(x.x + vr, x.y + vi, x.z + vr, x.w + vi);
+          },
+          ready);
     } else if ((NM & 1) == 0) {
       // even NM: a thread takes two adjacent columns, one 16-byte load of phi' and one
       // 32-bit store per plane
-      constexpr int U = 8;
       const size_t ps = (size_t)R * NMp;
       __half* tb = t_next + (size_t)b * 4 * ps;
       const float4* pb = reinterpret_cast<const float4*>(p32 + (size_t)b * R * NM);
-      for (int e0 = tid; e0 < 128 * (BN / 2); e0 += 128 * U) {
-        float4 pv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = e0 + 128 * u, j = mt * 128 + e / (BN / 2), i = nt * BN + 2 * (e % (BN / 2));
-          if (j < R && i < NM) pv[u] = pb[((size_t)j * NM + i) / 2];
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = e0 + 128 * u, r = e / (BN / 2), c = 2 * (e % (BN / 2)), j = mt * 128 + r, i = nt * BN + c;
-          if (j >= R || i >= NM) continue;
-          const float2 v0 = tile[r * tcg::STAGE_LD + c], v1 = tile[r * tcg::STAGE_LD + c + 1];
-          __half h0, l0, h1, l1;
-          __half* o = tb + (size_t)j * NMp + i;
-          split_val(fmaf(pv[u].x, sc, v0.x * st), h0, l0);
-          split_val(fmaf(pv[u].z, sc, v1.x * st), h1, l1);
-          *reinterpret_cast<__half2*>(o) = __halves2half2(h0, h1);
-          *reinterpret_cast<__half2*>(o + ps) = __halves2half2(l0, l1);
-          split_val(fmaf(pv[u].y, sc, v0.y * st), h0, l0);
-          split_val(fmaf(pv[u].w, sc, v1.y * st), h1, l1);
-          *reinterpret_cast<__half2*>(o + 2 * ps) = __halves2half2(h0, h1);
-          *reinterpret_cast<__half2*>(o + 3 * ps) = __halves2half2(l0, l1);
-        }
-      }
+      batches<128 * (BN / 2), float4>(
+          tid,
+          [&](int e) {
+            const int j = mt * 128 + e / (BN / 2), i = nt * BN + 2 * (e % (BN / 2));
+            return j < R && i < NM ? pb[((size_t)j * NM + i) / 2] : make_float4(0.f, 0.f, 0.f, 0.f);
+          },
+          [&](int e, const float4& x) {
+            const int r = e / (BN / 2), c = 2 * (e % (BN / 2)), j = mt * 128 + r, i = nt * BN + c;
+            if (j >= R || i >= NM) return;
+            const float2 v0 = tile[r * tcg::STAGE_LD + c], v1 = tile[r * tcg::STAGE_LD + c + 1];
+            __half* o = tb + (size_t)j * NMp + i;
+            __half2 hi, lo;
+            split_pair(fmaf(x.x, sc, v0.x * st), fmaf(x.z, sc, v1.x * st), hi, lo);
+            *reinterpret_cast<__half2*>(o) = hi;
+            *reinterpret_cast<__half2*>(o + ps) = lo;
+            split_pair(fmaf(x.y, sc, v0.y * st), fmaf(x.w, sc, v1.y * st), hi, lo);
+            *reinterpret_cast<__half2*>(o + 2 * ps) = hi;
+            *reinterpret_cast<__half2*>(o + 3 * ps) = lo;
+          },
+          ready);
     } else {
-      constexpr int U = 8;
       const size_t ps = (size_t)R * NMp;
       __half* tb = t_next + (size_t)b * 4 * ps;
       const float2* pb = p32 + (size_t)b * R * NM;
-      for (int e0 = tid; e0 < 128 * BN; e0 += 128 * U) {
-        float2 pv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = e0 + 128 * u, j = mt * 128 + e / BN, i = nt * BN + e % BN;
-          if (j < R && i < NM) pv[u] = pb[(size_t)j * NM + i];
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = e0 + 128 * u, r = e / BN, c = e % BN, j = mt * 128 + r, i = nt * BN + c;
-          if (j >= R || i >= NM) continue;
-          const float2 v = tile[r * tcg::STAGE_LD + c];
-          put4f(tb, ps, (size_t)j * NMp + i, fmaf(pv[u].x, sc, v.x * st), fmaf(pv[u].y, sc, v.y * st));
-        }
-      }
+      batches<128 * BN, float2>(
+          tid,
+          [&](int e) {
+            const int j = mt * 128 + e / BN, i = nt * BN + e % BN;
+            return j < R && i < NM ? pb[(size_t)j * NM + i] : make_float2(0.f, 0.f);
+          },
+          [&](int e, const float2& x) {
+            const int r = e / BN, c = e % BN, j = mt * 128 + r, i = nt * BN + c;
+            if (j >= R || i >= NM) return;
+            const float2 v = tile[r * tcg::STAGE_LD + c];
+            put4f(tb, ps, (size_t)j * NMp + i, fmaf(x.x, sc, v.x * st), fmaf(x.y, sc, v.y * st));
+          },
+          ready);
     }
   }
 };
@@ -487,7 +524,6 @@ struct TaylorP {
 struct ExchangeP {
   static constexpr bool kConjA = false;
   static constexpr bool kStreamB = true;   // Z streams through L2 once per launch when mt_n == 1
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES_LIGHT;
   int tiles, kchunks;
   int mt_n, nt_n, WS, nk, nMp;
@@ -510,17 +546,18 @@ struct ExchangeP {
     tcg::Coords c = {{kc * 32, mt * 128, 0, kminus[q.y * nk + q.x], q.z}, {kc * 32, nt * BN, 0, 0, t}};
     return c;
   }
-  // Each store warp takes 32 rows of the tile, four at a time: eight lanes per row, each
-  // reading four 16-byte pieces of the row's partner run, so that one warp load covers four
-  // whole 128-byte lines.  Every load of the tile is issued before the first product.
-  __device__ void store_tile(int t, int mt, int nt, const float2* tile, int tid, int, int lane) const {
+  // Each store warp takes 128 / (store warps) rows of the tile, four at a time: eight lanes per
+  // row, each reading four 16-byte pieces of the row's partner run, so that one warp load covers
+  // four whole 128-byte lines.  Every load of the tile is issued before the tile is waited for.
+  template <class R>
+  __device__ void store_tile(int t, int mt, int nt, const float2* tile, int tid, int lane, R ready) const {
     const int4 q = tri[t];
     const int kxq = kminus[q.z * nk + minus[q.x]];  // kx + Q
     const float2* gb = g32 + ((size_t)q.y * nk + kxq) * WS * nMp + nt * BN;
     // padding columns (s >= M) of Z_t are zero, so every column below n*Mp takes part
     const int pairs = min(BN, nMp - nt * BN) / 2;
-    const int ri = lane >> 3, cl = lane & 7, r0 = (tid >> 5) * 32;
-    constexpr int IT = 8, UJ = BN / 16;   // rows per lane, 16-byte pieces per lane and row
+    constexpr int ROWS = 128 * 32 / ST, IT = ROWS / 4, UJ = BN / 16;   // rows per warp and lane, pieces per lane
+    const int ri = lane >> 3, cl = lane & 7, r0 = (tid >> 5) * ROWS;
     float4 gv[IT][UJ];
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
@@ -532,6 +569,7 @@ struct ExchangeP {
         gv[it][u] = (ws < WS && j < pairs) ? g4[j] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
+    if (!ready()) return;
     const float inv_z = 1.f / s_z[t];
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
@@ -573,7 +611,6 @@ struct AdjointP {
   static constexpr bool kConjA = false;
   static constexpr bool kStreamB = true;   // Z streams through L2 once per launch when mt_n == 1
   static constexpr bool kChunkScale = true;
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES_LIGHT;
   int tiles, kchunks;  // kchunks = nk * kcb
   int kcb, mt_n, nt_n, WS, nk, nMp;
@@ -608,15 +645,18 @@ struct AdjointP {
     split_k(b, kc, tf, km, kx, kk);
     return 1.f / s_z[tf];   // a power of two: exact
   }
-  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, int) const {
-    const int cols = min(BN, nMp - nt * BN);
-    for (int e = tid; e < 128 * BN; e += 128) {
-      const int r = e / BN, c = e % BN;
+  template <class R>
+  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, R ready) const {
+    const int c = tid % BN, cols = min(BN, nMp - nt * BN);
+    float2* o = gam32 + ((size_t)b * WS + mt * 128) * nMp + nt * BN + c;
+    if (!ready() || c >= cols) return;
+#pragma unroll 4
+    for (int r = tid / BN; r < 128; r += ST / BN) {
       const int ws = mt * 128 + r;
-      if (ws >= WS || c >= cols) continue;
-      const float inv = 1.f / s_g[ws];
+      if (ws >= WS) break;
+      const float inv = rcp2(s_g[ws]);
       const float2 v = tile[r * tcg::STAGE_LD + c];
-      gam32[((size_t)b * WS + ws) * nMp + nt * BN + c] = make_float2(v.x * inv, v.y * inv);
+      o[(size_t)r * nMp] = make_float2(v.x * inv, v.y * inv);
     }
   }
 };
@@ -624,7 +664,6 @@ struct AdjointP {
 // Gram[ws] = phi_ws^dag phi_ws from the transposed split planes (rows = columns of phi).
 struct GramP {
   static constexpr bool kConjA = true;
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES;
   int tiles, kchunks;
   int mt_n, nt_n, N;
@@ -640,13 +679,16 @@ struct GramP {
     tcg::Coords c = {{kc * 32, sp * N + mt * 128, 0, w, 0}, {kc * 32, sp * N + nt * BN, 0, 0, w}};
     return c;
   }
-  __device__ void store_tile(int ws, int mt, int nt, const float2* tile, int tid, int, int) const {
+  template <class R>
+  __device__ void store_tile(int ws, int mt, int nt, const float2* tile, int tid, int, R ready) const {
     const float sc = s_t[ws >> 1];
-    const float st = 1.f / (sc * sc);
-    for (int e = tid; e < 128 * BN; e += 128) {
-      const int r = e / BN, c = e % BN;
-      const int i = mt * 128 + r, j = nt * BN + c;
-      if (i >= N || j >= N) continue;
+    const float st = rcp2(sc * sc);
+    const int c = tid % BN, j = nt * BN + c;
+    if (!ready() || j >= N) return;
+#pragma unroll 4
+    for (int r = tid / BN; r < 128; r += ST / BN) {
+      const int i = mt * 128 + r;
+      if (i >= N) break;
       const float2 v = tile[r * tcg::STAGE_LD + c];
       gram[((size_t)ws * N + i) * N + j] = make_float2(v.x * st, v.y * st);
     }
@@ -656,7 +698,6 @@ struct GramP {
 // phi[ws] <- phi[ws] R^-1 : rows r = (k,p), columns j; B = (R^-1)^T split planes.
 struct ApplyRP {
   static constexpr bool kConjA = false;
-  static constexpr bool kPairB = true;
   static constexpr int kStages = STAGES;
   int tiles, kchunks;
   int mt_n, nt_n, NM, N;
@@ -672,12 +713,15 @@ struct ApplyRP {
     tcg::Coords c = {{kc * 32, mt * 128, 0, ws, 0}, {kc * 32, nt * BN, 0, 0, ws}};
     return c;
   }
-  __device__ void store_tile(int ws, int mt, int nt, const float2* tile, int tid, int, int) const {
-    const float st = 1.f / (s_phi[ws] * s_r[ws]);
-    for (int e = tid; e < 128 * BN; e += 128) {
-      const int r = e / BN, c = e % BN;
-      const int row = mt * 128 + r, j = nt * BN + c;
-      if (row >= NM || j >= N) continue;
+  template <class R>
+  __device__ void store_tile(int ws, int mt, int nt, const float2* tile, int tid, int, R ready) const {
+    const float st = rcp2(s_phi[ws] * s_r[ws]);
+    const int c = tid % BN, j = nt * BN + c;
+    if (!ready() || j >= N) return;
+#pragma unroll 4
+    for (int r = tid / BN; r < 128; r += ST / BN) {
+      const int row = mt * 128 + r;
+      if (row >= NM) break;
       const float2 v = tile[r * tcg::STAGE_LD + c];
       phi[((size_t)ws * NM + row) * N + j] = make_double2((double)(v.x * st), (double)(v.y * st));
     }

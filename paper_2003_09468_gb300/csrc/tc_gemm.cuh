@@ -9,16 +9,20 @@
 // that |x*s| stays well inside the fp16 range.  Each real product is formed
 // from three fp16 products (hi*hi + hi*lo + lo*hi), accumulated in fp32 in
 // tensor memory, which keeps about 22 significant bits per operand.  The real
-// and imaginary parts of D use two accumulators:
-//   D_re = Ar Br - Ai Bi,   D_im = Ar Bi + Ai Br   (negation via the MMA's B-negate bit)
+// and imaginary parts of D come from four real accumulators (below):
+//   D_re = Ar Br - Ai Bi,   D_im = Ar Bi + Ai Br
 //
-// Persistent kernel, one CTA per SM over a contiguous range of 128 x 64 output tiles:
-// warp 0 issues TMA loads (one 5-D box per operand per 32-wide k chunk, all four planes
-// at once, 64-byte swizzle) into a STAGES-deep ring; warp 1 allocates tensor memory and
-// one of its threads issues the tcgen05.mma chain; warps 2-5 read the accumulators back
-// with tcgen05.ld and hand the finished tile to the policy's epilogue.  Every mbarrier
-// wait is bounded; on time-out the kernel records an error, drains its own copies and
-// MMAs, frees tensor memory and returns.
+// Persistent kernel, one CTA per SM over 128 x 64 output tiles, 512 threads in four warp
+// groups with their own register budgets:
+//   group 0  warp 0 issues TMA loads (one 5-D box per operand per 32-wide k chunk, all four
+//            planes at once, 64-byte swizzle) into a STAGES-deep ring; one thread of each of
+//            warps 1 and 2 issues the tcgen05.mma chains, warp 1 the even chunks into
+//            accumulator set 0, warp 2 the odd ones into set 1; warp 3 owns the tensor
+//            memory allocation;
+//   group 1  reads the accumulators back with tcgen05.ld into fp32 running sums;
+//   groups 2, 3  hand the finished tile to the policy's epilogue.
+// Every mbarrier wait is bounded; on time-out the kernel records an error, drains its own
+// copies and MMAs, frees tensor memory and returns.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -31,25 +35,40 @@ namespace tcg {
 constexpr int BM = 128;      // tile rows = TMEM lanes
 constexpr int BK = 32;       // complex k per stage: 64-byte fp16 rows
 constexpr int NPLANE = 4;
-// warp 0 TMA, warp 1 MMA, warps 2-5 drain the accumulators, warps 6-9 store the drained
-// tiles (so that the stores of one tile overlap the MMAs of the next)
-constexpr int THREADS = 320;
+constexpr int DRAIN_THREADS = 128;
+constexpr int STORE_THREADS = 256;
+constexpr int THREADS = 128 + DRAIN_THREADS + STORE_THREADS;
+constexpr int TILE_BAR_THREADS = DRAIN_THREADS + STORE_THREADS;   // the tile hand-over barriers
+// Registers per thread of the four groups: the drain holds 128 running sums and two TMEM load
+// buffers, the store groups their epilogue's loads in flight.  The shares add up to what the
+// launch gets (4 x 128 at 512 threads per SM), so every setmaxnreg.inc is served.
+constexpr int REGS_ISSUE = 64, REGS_DRAIN = 208, REGS_STORE = 120;
+static_assert(REGS_ISSUE + REGS_DRAIN + 2 * REGS_STORE <= 4 * (65536 / THREADS), "register shares");
+static_assert(THREADS == 512, "four warp groups");
 
 struct Coords {
   int a[5];
   int b[5];
 };
 
+// B is staged with its planes in the order (re_hi, im_hi, re_lo, im_lo) (a tensor map whose
+// plane dimensions are (re/im, hi/lo)), so that [B_re; B_im] is one 128-row operand: one
+// N = 128 MMA gives [A_x B_re | A_x B_im], twelve MMAs per chunk.
+//
 // Policy P provides:
 //   static constexpr bool kConjA;     D = sum conj(A) B instead of sum A B
 //   int tiles;                        number of output tiles
 //   int kchunks;                      k chunks of BK per tile
 //   __device__ void tile(int t, int& b, int& mt, int& nt) const;
 //   __device__ Coords coords(int b, int mt, int nt, int kc) const;
-//   __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int ewarp, int lane) const;
-//       the finished 128 x 64 tile in shared memory, tile[r * STAGE_LD + c] = (re, im);
-//       called by the 128 store threads (tid 0..127, ewarp 0..3) while the drain warps
-//       already accumulate the next tile
+//   template <class R> __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int lane,
+//                                                 R ready) const;
+//       called by the STORE_THREADS store threads (tid 0..STORE_THREADS-1) while the drain warps
+//       already accumulate the next tile.  Every thread calls ready() exactly once: it waits
+//       until the finished 128 x 64 tile is in shared memory, tile[r * STAGE_LD + c] = (re, im),
+//       and returns false when the kernel is giving up (nothing may be stored then).  Loads
+//       that do not depend on the tile go before it, so that they are in flight while the
+//       tile is still being accumulated.
 // and optionally
 //   static constexpr bool kChunkScale = true;
 //   __device__ float chunk_scale(int b, int kc) const;
@@ -63,33 +82,6 @@ template <class P>
 struct ChunkScaled<P, decltype((void)P::kChunkScale)> {
   static constexpr bool value = P::kChunkScale;
 };
-//   static constexpr bool kPairB = true;
-//       B is staged with its planes in the order (re_hi, im_hi, re_lo, im_lo) (a tensor map
-//       whose plane dimensions are (re/im, hi/lo)), so that [B_re; B_im] is one 128-row
-//       operand: one N = 128 MMA then gives [A_x B_re | A_x B_im], twelve MMAs per chunk
-//       instead of twenty-four, and each A plane is read half as often
-template <class P, class = void>
-struct PairB {
-  static constexpr bool value = false;
-};
-template <class P>
-struct PairB<P, decltype((void)P::kPairB)> {
-  static constexpr bool value = P::kPairB;
-};
-
-//   static constexpr int kDrainChunks = D;
-//       the accumulators run over D consecutive k chunks before they are drained (default 1):
-//       the drain work per MMA falls by D, each fp32 partial carries D times as many
-//       truncating additions.  Not with kChunkScale (one factor per drained partial).
-template <class P, class = void>
-struct DrainChunks {
-  static constexpr int value = 1;
-};
-template <class P>
-struct DrainChunks<P, decltype((void)P::kDrainChunks)> {
-  static constexpr int value = P::kDrainChunks;
-};
-
 //   static constexpr bool kStreamB = true;  __device__ bool stream_b() const;
 //       when stream_b() is true, B is read once per launch (a large static tensor streamed
 //       through, one row tile): its TMA loads carry the L2 evict-first policy, so that the
@@ -147,16 +139,15 @@ __device__ __forceinline__ float chunk_factor(const P& p, int b, int kc) {
 // ---------------------------------------------------------------- precise variant
 // The tensor-core accumulator adds each MMA's partial sum with truncation, so a
 // long chain of MMAs into one accumulator loses accuracy in proportion to its
-// length.  This variant keeps four real accumulators per k-step,
+// length.  This variant keeps four real accumulators per k chunk,
 //   P_rr = Ar Br, P_ii = Ai Bi, P_ri = Ar Bi, P_ir = Ai Br   (each hi*hi + hi*lo + lo*hi),
-// restarts them on every 16-wide k step (two TMEM sets in ping-pong), and the
-// epilogue warps fold each step into fp32 register sums with round-to-nearest:
+// restarts them on every 32-wide k chunk (two TMEM sets in ping-pong), and the
+// drain warps fold each chunk into fp32 register sums with round-to-nearest:
 //   re += P_rr - P_ii,  im += P_ri + P_ir.
 // Tile 128 x BNP (BNP = 64): 4 x 64 columns per set, 2 sets = all 512 TMEM columns.
 constexpr int BNP = 64;
 
-// Accumulator columns per tcgen05.ld in the drain (8 or 16): fewer round trips against more
-// registers beyond the 128 running sums.
+// Accumulator columns per tcgen05.ld in the drain.
 constexpr int DRAIN_COLS = 8;
 
 // Epilogue staging: the finished 128 x 64 tile as (re, im) fp32 pairs, rows padded to 65
@@ -181,11 +172,18 @@ struct LayoutP {
 // of the two), so the pair reads each B element from shared memory once where two CTAs would
 // read it twice.  Tile t of the policy is then a pair of row tiles: CTA r takes row tile
 // 2 mt + r.  Each CTA drains and stores its own rows as in the single form.
+//
+// What bounds it.  A chunk is twelve 128x128x16 MMAs, 64 clocks each at the tensor peak, but the
+// tensor pipe queues hardly more than one MMA ahead of the issuing thread: any clock that
+// thread spends on a barrier, a commit or a descriptor is a clock without MMAs (a chain with one
+// wait and one commit per chunk runs at 1030 clocks per chunk against 770 without).  So two threads
+// issue: while one's chunk runs, the other waits for its stage and its accumulator set.
 template <int STAGES, class P, bool PAIR = false>
 __global__ void __launch_bounds__(THREADS, 1)
     cgemm_precise_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ P p, int* err) {
-  static_assert(!PAIR || (PairB<P>::value && !Grouped<P>::value), "pair form: paired B, one problem");
+  static_assert(!PAIR || !Grouped<P>::value, "pair form: one problem");
+  static_assert(STAGES >= 2 && STAGES <= 4, "the issuing threads' barrier phases (see their waits)");
   static_assert(LayoutP<STAGES, PAIR>::SMEM <= 232448, "shared memory per CTA");
   // Persistent: CTA i handles tiles i, i + grid, i + 2 grid, ...  The TMA ring and the
   // two TMEM accumulator sets run continuously across tile boundaries.  One drain per 32-wide k
@@ -197,8 +195,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   float2* tile_buf = reinterpret_cast<float2*>(smem + STAGES * Lay::STAGE_BYTES);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * Lay::STAGE_BYTES + Lay::TILE_BYTES);
   uint64_t* empty = full + STAGES;
-  uint64_t* accf = empty + STAGES;   // [2] MMA -> epilogue: set holds a finished chunk
-  uint64_t* acce = accf + 2;         // [2] epilogue -> MMA: set drained
+  uint64_t* accf = empty + STAGES;   // [2] MMA -> drain: set holds a finished chunk
+  uint64_t* acce = accf + 2;         // [2] drain -> MMA: set drained
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -217,7 +215,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     *abort = 0;
     tc::fence_mbar_init();
   }
-  if (warp == 1) {
+  if (warp == 3) {
     if constexpr (PAIR) {
       tc::tmem_alloc_pair(tmem_slot, Lay::TMEM_COLS);
       tc::tmem_relinquish_pair();
@@ -237,11 +235,10 @@ __global__ void __launch_bounds__(THREADS, 1)
   // are read from HBM once and served from L2 to the others
   const int t0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int tstep = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-  constexpr int DC = DrainChunks<P>::value;
-  static_assert(DC >= 1 && (DC == 1 || !ChunkScaled<P>::value), "one chunk factor per drained partial");
 
-  if (warp == 0) {
-    if (lane == 0) {
+  if (warp < 4) {
+    tc::setmaxnreg_dec<REGS_ISSUE>();
+    if (warp == 0 && lane == 0) {
       if constexpr (!Grouped<P>::value) {
         tc::tma_prefetch(&tmA);
         tc::tma_prefetch(&tmB);
@@ -296,132 +293,91 @@ __global__ void __launch_bounds__(THREADS, 1)
         int zero = 0;
         if (!tc::mbar_wait(&full[s], ph, &zero)) atomicCAS(err, 0, tc::ERR_TIMEOUT_DRAIN);
       }
-    }
-  } else if (warp == 1) {
-    if (lane == 0 && leader) {   // the pair form's MMAs are issued by the even CTA alone
-      constexpr uint32_t id = tc::idesc_f16(BM, BNP, false);
-      long g = 0;   // k chunks (TMA ring)
-      long a = 0;   // drained partials (accumulator sets), one per D chunks
+    } else if ((warp == 1 || warp == 2) && lane == 0 && leader) {
+      // The chunks alternate between the two issuing threads: chunk g goes to set g & 1, whose
+      // thread waits for the chunk's stage and for its own set while the other's MMAs run.  In
+      // the pair form the even CTA issues for both.
+      const int set = warp - 1;
+      const uint32_t d = tmem + set * 4 * BNP;
+      const uint64_t desc0 = tc::desc_kmajor_sw64(tc::smem_u32(smem));   // offsets add in 16-byte units
+      long g = 0;
+      uint32_t use = 0;   // chunks this thread has issued
       bool failed = false;
       for (int t = t0; t < p.tiles && !failed; t += tstep) {
         int b, mt, nt;
         p.tile(t, b, mt, nt);
         const int KC = kchunks_of(p, b);
         for (int kc = 0; kc < KC; ++kc, ++g) {
+          if ((int)(g & 1) != set) continue;
           const int s = (int)(g % STAGES);
           const uint32_t ph = (uint32_t)((g / STAGES) & 1);
+          // The accumulator set first: chunk g - 2 drained means that chunk g - 3, the previous
+          // one in this stage of a three-deep ring and the other thread's, has been consumed, so
+          // the stage's barrier is in this chunk's phase and its parity cannot be mistaken for
+          // an older phase's.
+          if (!tc::mbar_wait(&acce[set], (use & 1) ^ 1, abort)) {
+            atomicCAS(err, 0, tc::ERR_TIMEOUT_ACC);
+            *abort = 1;
+            failed = true;
+            break;
+          }
           if (!tc::mbar_wait(&full[s], ph, abort)) {
             atomicCAS(err, 0, tc::ERR_TIMEOUT_FULL);
             *abort = 1;
             failed = true;
             break;
           }
-          const bool open = (kc % DC) == 0;                      // first chunk of a partial
-          const bool close = (kc % DC) == DC - 1 || kc == KC - 1;  // last chunk of a partial
-          const int set = (int)(a & 1);
-          const uint32_t use = (uint32_t)(a >> 1);
-          if (open && !tc::mbar_wait(&acce[set], (use & 1) ^ 1, abort)) {
-            atomicCAS(err, 0, tc::ERR_TIMEOUT_ACC);
-            *abort = 1;
-            failed = true;
-            break;
-          }
-          const uint32_t acc0 = open ? 0u : 1u;   // the partial's first MMA overwrites the set
           tc::fence_after_sync();
-          const uint32_t sa = tc::smem_u32(smem + s * Lay::STAGE_BYTES);
-          const uint32_t sb = sa + Lay::A_BYTES;
-          const uint32_t d = tmem + set * 4 * BNP;
-          uint64_t A[4][2];  // [plane][k16 half]; A planes: 0 re_hi, 1 re_lo, 2 im_hi, 3 im_lo
-#pragma unroll
-          for (int pl = 0; pl < 4; ++pl)
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk) A[pl][kk] = tc::desc_kmajor_sw64(sa + pl * BM * 64 + kk * 32);
+          const uint64_t da = desc0 + (uint64_t)((s * Lay::STAGE_BYTES) >> 4);   // A planes: re_hi, re_lo, im_hi, im_lo
+          const uint64_t db = da + (uint64_t)(Lay::A_BYTES >> 4);
+          constexpr uint64_t PL = (BM * 64) >> 4, KK = 32 >> 4;   // next A plane, next 16-wide k half
           if constexpr (PAIR) {
             // Each CTA holds [B_hi; B_lo] of its half (re in the even CTA, im in the odd one),
             // 64 rows each: the pair's B operand rows 0..127 are [Br_hi; Bi_hi] (or _lo).
             constexpr uint32_t idp = tc::idesc_f16(2 * BM, 2 * BNP, false);
-            uint64_t Bh[2], Bl[2];
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk) {
-              Bh[kk] = tc::desc_kmajor_sw64(sb + kk * 32);
-              Bl[kk] = tc::desc_kmajor_sw64(sb + BNP * 64 + kk * 32);
-            }
+            constexpr uint64_t LO = (BNP * 64) >> 4;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               const uint32_t dq = d + q * 2 * BNP;
-              const int ah = 2 * q;
-              tc::mma_f16_pair(dq, A[ah + 1][0], Bh[0], idp, acc0);
-              tc::mma_f16_pair(dq, A[ah][0], Bl[0], idp, 1);
-              tc::mma_f16_pair(dq, A[ah + 1][1], Bh[1], idp, 1);
-              tc::mma_f16_pair(dq, A[ah][1], Bl[1], idp, 1);
-              tc::mma_f16_pair(dq, A[ah][0], Bh[0], idp, 1);
-              tc::mma_f16_pair(dq, A[ah][1], Bh[1], idp, 1);
+              const uint64_t hi = da + 2 * q * PL, lo = hi + PL;
+              tc::mma_f16_pair(dq, lo, db, idp, 0);   // the chunk's first MMA overwrites the set
+              tc::mma_f16_pair(dq, hi, db + LO, idp, 1);
+              tc::mma_f16_pair(dq, lo + KK, db + KK, idp, 1);
+              tc::mma_f16_pair(dq, hi + KK, db + LO + KK, idp, 1);
+              tc::mma_f16_pair(dq, hi, db, idp, 1);
+              tc::mma_f16_pair(dq, hi + KK, db + KK, idp, 1);
             }
-          } else if constexpr (PairB<P>::value) {
+            tc::mma_commit_pair(&accf[set]);
+            tc::mma_commit_pair(&empty[s]);
+          } else {
             // B rows 0..127 = [Br_hi; Bi_hi], rows 128..255 = [Br_lo; Bi_lo].  Accumulators:
             // Ar [Br | Bi] -> P_rr (0), P_ri (64); Ai [Br | Bi] -> P_ir (128), P_ii (192).
             constexpr uint32_t id2 = tc::idesc_f16(BM, 2 * BNP, false);
-            uint64_t Bh[2], Bl[2];
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk) {
-              Bh[kk] = tc::desc_kmajor_sw64(sb + kk * 32);
-              Bl[kk] = tc::desc_kmajor_sw64(sb + 2 * BNP * 64 + kk * 32);
-            }
+            constexpr uint64_t LO = (2 * BNP * 64) >> 4;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               const uint32_t dq = d + q * 2 * BNP;
-              const int ah = 2 * q;
-              tc::mma_f16(dq, A[ah + 1][0], Bh[0], id2, acc0);
-              tc::mma_f16(dq, A[ah][0], Bl[0], id2, 1);
-              tc::mma_f16(dq, A[ah + 1][1], Bh[1], id2, 1);
-              tc::mma_f16(dq, A[ah][1], Bl[1], id2, 1);
-              tc::mma_f16(dq, A[ah][0], Bh[0], id2, 1);
-              tc::mma_f16(dq, A[ah][1], Bh[1], id2, 1);
+              const uint64_t hi = da + 2 * q * PL, lo = hi + PL;
+              tc::mma_f16(dq, lo, db, id2, 0);
+              tc::mma_f16(dq, hi, db + LO, id2, 1);
+              tc::mma_f16(dq, lo + KK, db + KK, id2, 1);
+              tc::mma_f16(dq, hi + KK, db + LO + KK, id2, 1);
+              tc::mma_f16(dq, hi, db, id2, 1);
+              tc::mma_f16(dq, hi + KK, db + KK, id2, 1);
             }
-          } else {
-            uint64_t B[4][2];
-#pragma unroll
-            for (int pl = 0; pl < 4; ++pl)
-#pragma unroll
-              for (int kk = 0; kk < 2; ++kk) B[pl][kk] = tc::desc_kmajor_sw64(sb + pl * BNP * 64 + kk * 32);
-            // Accumulators (column offsets):
-            // P_rr = Ar Br (0), P_ii = Ai Bi (64), P_ri = Ar Bi (128), P_ir = Ai Br (192).
-            const int ap[4] = {0, 2, 0, 2}, bp[4] = {0, 2, 2, 0};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const uint32_t dq = d + q * BNP;
-              const int ah = ap[q], bh = bp[q];
-              tc::mma_f16(dq, A[ah + 1][0], B[bh][0], id, acc0);
-              tc::mma_f16(dq, A[ah][0], B[bh + 1][0], id, 1);
-              tc::mma_f16(dq, A[ah + 1][1], B[bh][1], id, 1);
-              tc::mma_f16(dq, A[ah][1], B[bh + 1][1], id, 1);
-              tc::mma_f16(dq, A[ah][0], B[bh][0], id, 1);
-              tc::mma_f16(dq, A[ah][1], B[bh][1], id, 1);
-            }
-          }
-          if constexpr (PAIR) {
-            if (close) {
-              tc::mma_commit_pair(&accf[set]);
-              ++a;
-            }
-            tc::mma_commit_pair(&empty[s]);
-          } else {
-            if (close) {
-              tc::mma_commit(&accf[set]);
-              ++a;
-            }
+            tc::mma_commit(&accf[set]);
             tc::mma_commit(&empty[s]);
           }
+          ++use;
         }
       }
-      if (a > 0) {  // our own MMAs must complete before TMEM is freed
-        const long last = a - 1;
+      if (use > 0) {  // our own MMAs must complete before TMEM is freed
         int zero = 0;
-        if (!tc::mbar_wait(&accf[last & 1], (uint32_t)((last >> 1) & 1), &zero))
-          atomicCAS(err, 0, tc::ERR_TIMEOUT_DRAIN);
+        if (!tc::mbar_wait(&accf[set], (use - 1) & 1, &zero)) atomicCAS(err, 0, tc::ERR_TIMEOUT_DRAIN);
       }
     }
-  } else if (warp < 6) {
+  } else if (warp < 8) {
+    tc::setmaxnreg_inc<REGS_DRAIN>();
     // Drain warps.  All four run the same sequence of named barriers for every tile, so a
     // failed (timed-out) wait never leaves a warp behind at a barrier: failure is sticky,
     // skips the work, and raises the abort flag that ends every later wait at once.
@@ -431,7 +387,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int q = warp & 3;
     const int r = q * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
-    long g = 0;   // drained partials, in the MMA warp's order
+    long g = 0;   // k chunks, in the MMA warps' order
     bool ok = true;
     int ntile = 0;
     for (int t = t0; t < p.tiles; t += tstep, ++ntile) {
@@ -441,7 +397,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
       for (int c = 0; c < BNP; ++c) { sre[c] = 0.f; sim[c] = 0.f; }
       const int KC = kchunks_of(p, b);
-      for (int kc = 0; kc < KC; kc += DC, ++g) {
+      for (int kc = 0; kc < KC; ++kc, ++g) {
         const int set = (int)(g & 1);
         const uint32_t use = (uint32_t)(g >> 1);
         if (ok && !tc::mbar_wait(&accf[set], use & 1, abort)) {
@@ -449,66 +405,82 @@ __global__ void __launch_bounds__(THREADS, 1)
           *abort = 1;
           ok = false;
         }
+        __syncwarp();   // the TMEM loads are warp-wide: the lanes leave the wait together
+        ok = __all_sync(0xffffffffu, ok);
         if (!ok) continue;
         tc::fence_after_sync();
         const uint32_t d = tmem + lane_off + set * 4 * BNP;
         const float cf = chunk_factor(p, b, kc);
-        // column blocks of P_rr, P_ii, P_ri, P_ir in the set
-        constexpr int o_ii = PairB<P>::value ? 3 : 1, o_ri = PairB<P>::value ? 1 : 2, o_ir = PairB<P>::value ? 2 : 3;
-        // DRAIN_COLS columns of two accumulators per load round
+        // column blocks of P_rr, P_ri, P_ir, P_ii in the set; the loads of one pair of
+        // accumulators are in flight while the other pair's columns are added
+        constexpr int o_ri = BNP, o_ir = 2 * BNP, o_ii = 3 * BNP, DCOL = DRAIN_COLS;
+        float xr[DCOL], yr[DCOL], xi[DCOL], yi[DCOL];
+        tc::tmem_ld8(d, xr);
+        tc::tmem_ld8(d + o_ii, yr);
 #pragma unroll
-        for (int gq = 0; gq < BNP / DRAIN_COLS; ++gq) {
-          float x[DRAIN_COLS], y[DRAIN_COLS];
-          tc::tmem_ld<DRAIN_COLS>(d + 0 * BNP + gq * DRAIN_COLS, x);      // P_rr
-          tc::tmem_ld<DRAIN_COLS>(d + o_ii * BNP + gq * DRAIN_COLS, y);   // P_ii
-          tc::tmem_ld_wait();
+        for (int gq = 0; gq < BNP / DCOL; ++gq) {
+          tc::tmem_ld_wait(xr, yr);
+          tc::tmem_ld8(d + o_ri + gq * DCOL, xi);
+          tc::tmem_ld8(d + o_ir + gq * DCOL, yi);
 #pragma unroll
-          for (int c = 0; c < DRAIN_COLS; ++c) {
-            const float v = P::kConjA ? x[c] + y[c] : x[c] - y[c];
+          for (int c = 0; c < DCOL; ++c) {
+            const float v = P::kConjA ? xr[c] + yr[c] : xr[c] - yr[c];
             if constexpr (ChunkScaled<P>::value)
-              sre[gq * DRAIN_COLS + c] = fmaf(cf, v, sre[gq * DRAIN_COLS + c]);
+              sre[gq * DCOL + c] = fmaf(cf, v, sre[gq * DCOL + c]);
             else
-              sre[gq * DRAIN_COLS + c] += v;
+              sre[gq * DCOL + c] += v;
           }
-          tc::tmem_ld<DRAIN_COLS>(d + o_ri * BNP + gq * DRAIN_COLS, x);   // P_ri
-          tc::tmem_ld<DRAIN_COLS>(d + o_ir * BNP + gq * DRAIN_COLS, y);   // P_ir
-          tc::tmem_ld_wait();
+          tc::tmem_ld_wait(xi, yi);
+          if (gq + 1 < BNP / DCOL) {
+            tc::tmem_ld8(d + (gq + 1) * DCOL, xr);
+            tc::tmem_ld8(d + o_ii + (gq + 1) * DCOL, yr);
+          } else {
+            // the set's last loads have landed: hand it back before the last additions
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) {
+              if (PAIR && !leader)
+                tc::mbar_arrive_remote(tc::mapa_shared(tc::smem_u32(&acce[set]), 0));
+              else
+                tc::mbar_arrive(&acce[set]);
+            }
+          }
           // conj(a) b = (ar br + ai bi) + i (ar bi - ai br)
 #pragma unroll
-          for (int c = 0; c < DRAIN_COLS; ++c) {
-            const float v = P::kConjA ? x[c] - y[c] : x[c] + y[c];
+          for (int c = 0; c < DCOL; ++c) {
+            const float v = P::kConjA ? xi[c] - yi[c] : xi[c] + yi[c];
             if constexpr (ChunkScaled<P>::value)
-              sim[gq * DRAIN_COLS + c] = fmaf(cf, v, sim[gq * DRAIN_COLS + c]);
+              sim[gq * DCOL + c] = fmaf(cf, v, sim[gq * DCOL + c]);
             else
-              sim[gq * DRAIN_COLS + c] += v;
+              sim[gq * DCOL + c] += v;
           }
         }
-        tc::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) {
-          if (PAIR && !leader)
-            tc::mbar_arrive_remote(tc::mapa_shared(tc::smem_u32(&acce[set]), 0));
-          else
-            tc::mbar_arrive(&acce[set]);
-        }
       }
-      if (ntile > 0) asm volatile("bar.sync 3, 256;" ::: "memory");   // previous tile stored
+      __syncwarp();
+      if (ntile > 0) tc::named_sync<3, TILE_BAR_THREADS>();   // previous tile stored
 #pragma unroll
       for (int c = 0; c < BNP; ++c) tile_buf[r * STAGE_LD + c] = make_float2(sre[c], sim[c]);
       __threadfence_block();
-      asm volatile("bar.arrive 2, 256;" ::: "memory");
+      __syncwarp();
+      tc::named_arrive<2, TILE_BAR_THREADS>();
     }
-    if (ntile > 0) asm volatile("bar.sync 3, 256;" ::: "memory");
+    if (ntile > 0) tc::named_sync<3, TILE_BAR_THREADS>();
   } else {
+    tc::setmaxnreg_dec<REGS_STORE>();
     // Store warps: write each staged tile with the policy's own (coalesced) mapping.
-    const int tid = threadIdx.x - 192, ew = warp - 6;
+    const int tid = threadIdx.x - 128 - DRAIN_THREADS;
     for (int t = t0; t < p.tiles; t += tstep) {
       int b, mt, nt;
       p.tile(t, b, mt, nt);
-      asm volatile("bar.sync 2, 256;" ::: "memory");
-      if (!*abort) p.store_tile(b, PAIR ? 2 * mt + (int)rank : mt, nt, tile_buf, tid, ew, lane);
+      // the named barriers are warp-wide instructions: the warp reconverges before each
+      p.store_tile(b, PAIR ? 2 * mt + (int)rank : mt, nt, tile_buf, tid, lane, [&]() {
+        __syncwarp();
+        tc::named_sync<2, TILE_BAR_THREADS>();
+        return *abort == 0;
+      });
       __threadfence_block();
-      asm volatile("bar.arrive 3, 256;" ::: "memory");
+      __syncwarp();
+      tc::named_arrive<3, TILE_BAR_THREADS>();
     }
   }
   tc::fence_before_sync();
@@ -516,7 +488,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   // pair form: the peer's copies, MMAs and remote arrivals are all done before either CTA
   // frees its tensor memory or exits
   if constexpr (PAIR) tc::cluster_sync();
-  if (warp == 1) {
+  if (warp == 3) {
     tc::fence_after_sync();
     if constexpr (PAIR)
       tc::tmem_dealloc_pair(tmem, Lay::TMEM_COLS);
@@ -534,11 +506,10 @@ __global__ void __launch_bounds__(THREADS, 1)
 template <class P, int NMAX = 8>
 struct GroupP {
   static constexpr bool kConjA = P::kConjA;
-  static constexpr bool kPairB = PairB<P>::value;
   static constexpr bool kGrouped = true;
   static constexpr bool kStreamB = StreamB<P>::value;
   static constexpr int kStages = P::kStages;
-  static_assert(!ChunkScaled<P>::value && DrainChunks<P>::value == 1, "plain policies only");
+  static_assert(!ChunkScaled<P>::value, "plain policies only");
   int tiles, kchunks;   // kchunks unused: per member
   int n;
   int start[NMAX + 1];
@@ -552,8 +523,9 @@ struct GroupP {
     b = (i << 20) | bl;
   }
   __device__ Coords coords(int b, int mt, int nt, int kc) const { return m[b >> 20].coords(b & 0xFFFFF, mt, nt, kc); }
-  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int ew, int lane) const {
-    m[b >> 20].store_tile(b & 0xFFFFF, mt, nt, tile, tid, ew, lane);
+  template <class R>
+  __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int lane, R ready) const {
+    m[b >> 20].store_tile(b & 0xFFFFF, mt, nt, tile, tid, lane, ready);
   }
   __device__ int kchunks_of(int b) const { return m[b >> 20].kchunks; }
   __device__ bool stream_b_of(int b) const {
