@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(OV_THREADS)
 //   log det S = sum_j log a_jj + i pi (number of swaps mod 2).
 // A zero or non-finite pivot marks the matrix singular: logdet = (-inf, 0), sing = 1,
 // flags[0] counts it, and the inverse written is zero.
-// INV output: the split planes of S^-T, out[b][4][N][Np] with scale s_out[b].
+// INV output: the split planes of S^-T, out[b][N][Np] (split.cuh) with scale s_out[b].
 template <bool SMEM, bool INV>
 __global__ void __launch_bounds__(GJ_THREADS)
     gj_ff_kernel(float4* Sff, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out) {
@@ -269,10 +269,9 @@ __global__ void __launch_bounds__(GJ_THREADS)
     }
   }
   if (!INV) return;
-  const size_t ps = (size_t)N * Np;
-  __half* o = out + (size_t)b * 4 * ps;
+  __half* o = out + (size_t)b * 4 * N * Np;
   if (singular) {
-    for (int e = tid; e < N * N; e += GJ_THREADS) mixed::put4f(o, ps, (size_t)(e / N) * Np + e % N, 0.f, 0.f);
+    for (int e = tid; e < N * N; e += GJ_THREADS) mixed::put4f(o + mixed::sp_at(e / N, Np, e % N), 0.f, 0.f);
     if (tid == 0) s_out[b] = 1.f;
     return;
   }
@@ -289,7 +288,7 @@ __global__ void __launch_bounds__(GJ_THREADS)
   for (int e = tid; e < N * N; e += GJ_THREADS) {
     const int i = e / N, c = e % N;
     const float4 v = a[(size_t)c * N + iperm[i]];
-    mixed::put4f(o, ps, (size_t)i * Np + c, v.x * s, v.z * s);
+    mixed::put4f(o + mixed::sp_at(i, Np, c), v.x * s, v.z * s);
   }
 }
 
@@ -503,10 +502,9 @@ __global__ void __launch_bounds__(GJB_THREADS)
       sing[b] = 0;
     }
   }
-  const size_t ps = (size_t)N * Np;
-  __half* o = out + (size_t)b * 4 * ps;
+  __half* o = out + (size_t)b * 4 * N * Np;
   if (singular) {
-    for (int e = tid; e < N * N; e += GJB_THREADS) mixed::put4f(o, ps, (size_t)(e / N) * Np + e % N, 0.f, 0.f);
+    for (int e = tid; e < N * N; e += GJB_THREADS) mixed::put4f(o + mixed::sp_at(e / N, Np, e % N), 0.f, 0.f);
     if (tid == 0) s_out[b] = 1.f;
     return;
   }
@@ -522,7 +520,7 @@ __global__ void __launch_bounds__(GJB_THREADS)
   for (int e = tid; e < N * N; e += GJB_THREADS) {
     const int i = e / N, c = e % N;
     const float4 v = a[(size_t)c * N + iperm[i]];
-    mixed::put4f(o, ps, (size_t)i * Np + c, v.x * sc, v.z * sc);
+    mixed::put4f(o + mixed::sp_at(i, Np, c), v.x * sc, v.z * sc);
   }
 }
 

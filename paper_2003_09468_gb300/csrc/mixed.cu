@@ -39,15 +39,15 @@
 
 struct MixedState {
   int Np, NMp, Mp, Gp, nMp, nM, WS, T;
-  // walker-dependent operands (split planes, fp16) and their scales
-  __half* phi_sp = nullptr;   float* s_phi = nullptr;   // [WS][4][NM][Np]
-  __half* sinvt_sp = nullptr; float* s_sinv = nullptr;  // [WS][4][N][Np]
+  // walker-dependent operands (split planes in the blocked layout of split.cuh) and their scales
+  __half* phi_sp = nullptr;   float* s_phi = nullptr;   // [WS][NM][Np]
+  __half* sinvt_sp = nullptr; float* s_sinv = nullptr;  // [WS][N][Np]
   float2* g32 = nullptr;                                 // [Nk][Nk][WS][n][Mp]
-  __half* g_sp = nullptr;     float* s_g = nullptr;     // [4][Nk][Nk][WS][n][Mp]
-  __half* gsum_sp = nullptr;  float* s_gsum = nullptr;  // [4][Nk][Nk][W][n][Mp]
-  __half* y_sp = nullptr;     float* s_y = nullptr;     // [4][Nk][W][Gp], s_y[Q][W]
-  __half* v_sp = nullptr;                                // [W][4][NM][NMp]
-  __half* t_sp[2] = {nullptr, nullptr}; float* s_t = nullptr;  // [W][4][2N][NMp]
+  __half* g_sp = nullptr;     float* s_g = nullptr;     // [Nk][Nk][WS][n Mp]
+  __half* gsum_sp = nullptr;  float* s_gsum = nullptr;  // [Nk][Nk][W][n Mp]
+  __half* y_sp = nullptr;     float* s_y = nullptr;     // [Nk][W][Gp], s_y[Q][W]
+  __half* v_sp = nullptr;                                // [W][NM][NMp]
+  __half* t_sp[2] = {nullptr, nullptr}; float* s_t = nullptr;  // [W][2N][NMp]
   double2* acc = nullptr;                                // [W][2N][NM] (scratch: float4 Taylor corrections, phi_perp)
   float2* p32 = nullptr;                                 // [W][2N][NM] phi' in fp32 (Taylor series)
   double2* xpart = nullptr;                              // [T][ntile][WS]
@@ -55,12 +55,13 @@ struct MixedState {
   int fb_groups = 1;                                     // groups of k blocks in the force-bias GEMM
   unsigned long long* mx = nullptr;                      // max |.| bit patterns: phi[WS], sinv[WS], g[3W], acc[W]
   // static operands
-  __half* lh_sp = nullptr;    float* s_lh = nullptr;    // [4][Nk][Nk][G][n][Mp], s_lh[Q][G]
-  __half* lt_sp = nullptr;    float* s_l = nullptr;     // [4][Nk][Nk][M*M][Gp], s_l[Q][G]
+  __half* lh_sp = nullptr;    float* s_lh = nullptr;    // [Nk][Nk][G][n Mp], s_lh[Q][G]
+  __half* lt_sp = nullptr;    float* s_l = nullptr;     // [Nk][Nk][M*M][Gp], s_l[Q][G]
   // Z of every triple in one array: rows 0 .. T-1 the canonical triples (exchange order),
   // rows T .. Nk^3-1 the transposes for their partners (the adjoint's operands)
-  __half* z_sp = nullptr;     float* s_z = nullptr;     // [4][Nk^3][n*Mp][n*Mp], s_z[Nk^3]
+  __half* z_sp = nullptr;     float* s_z = nullptr;     // [Nk^3][n*Mp][n*Mp], s_z[Nk^3]
   int4* tri = nullptr;                                   // [T] (Q, k, kx, weight)
+  int2* tri_blocks = nullptr;                            // [T] Green's-function blocks (kx, k-Q), (k, kx+Q)
   // adjoint of the exchange: the row of z_sp that holds Z of triple t = (Q nk + k) nk + kx,
   // and dEX/dGh per block
   int* zrow = nullptr;                                   // [Nk^3]
@@ -103,12 +104,12 @@ constexpr int ZCTAS = 304;
 // ---------------------------------------------------------------------------
 // FP64 input of moderate range: rounded once to fp32 (24 bits, of which the split keeps
 // 22), then scaled (per-step operands: walkers, inverses, Green's functions)
-__device__ __forceinline__ void put4(__half* base, size_t plane_stride, size_t idx, double re, double im, float s) {
-  put4f(base, plane_stride, idx, (float)re * s, (float)im * s);
+__device__ __forceinline__ void put4(__half* o, double re, double im, float s) {
+  put4f(o, (float)re * s, (float)im * s);
 }
 // FP64 input of any range: scaled in FP64 first (set-up data only)
-__device__ __forceinline__ void put4d(__half* base, size_t plane_stride, size_t idx, double re, double im, float s) {
-  put4f(base, plane_stride, idx, (float)(re * (double)s), (float)(im * (double)s));
+__device__ __forceinline__ void put4d(__half* o, double re, double im, float s) {
+  put4f(o, (float)(re * (double)s), (float)(im * (double)s));
 }
 
 __device__ __forceinline__ double block_max(double v, double* red) {
@@ -169,37 +170,29 @@ cudaError_t make_map(CUtensorMap* map, void* base, const MapSpec& s) {
 
 namespace mixed {
 
-// Build a map for an array of fp16 elements with logical dims d[0..4] (d[0]
-// contiguous) and element strides e[1..4].
-static cudaError_t map5(CUtensorMap* m, void* base, std::initializer_list<uint64_t> d,
-                        std::initializer_list<uint64_t> estride, uint32_t rows) {
+// Map of a split array of `batch` matrices of rows x ld (split.cuh), staged box_rows rows of one
+// 32-wide k chunk at a time, the four planes one after another: dimensions (k in the chunk, row,
+// plane, chunk, matrix).
+static cudaError_t map_split(CUtensorMap* m, void* base, int ld, size_t rows, size_t batch, uint32_t box_rows) {
   tcg::MapSpec s;
-  auto di = d.begin();
-  auto ei = estride.begin();
-  for (int i = 0; i < 5; ++i) s.dims[i] = di[i];
-  for (int i = 0; i < 4; ++i) s.strides[i] = ei[i] * sizeof(__half);
-  s.box[0] = 32;
-  s.box[1] = rows;
-  s.box[2] = 4;
-  s.box[3] = 1;
-  s.box[4] = 1;
+  s.dims[0] = 32; s.dims[1] = rows; s.dims[2] = 4; s.dims[3] = ld / 32; s.dims[4] = batch;
+  s.strides[0] = (uint64_t)4 * ld * sizeof(__half);
+  s.strides[1] = SP_PLANE * sizeof(__half);
+  s.strides[2] = 4 * SP_PLANE * sizeof(__half);
+  s.strides[3] = (uint64_t)4 * ld * rows * sizeof(__half);
+  s.box[0] = 32; s.box[1] = box_rows; s.box[2] = 4; s.box[3] = 1; s.box[4] = 1;
   return tcg::make_map(m, base, s);
 }
-
-// The same for a B operand of a kPairB policy: the four planes (stride ps elements, order
-// re_hi, re_lo, im_hi, im_lo in memory) are addressed as the two dimensions (re/im, hi/lo),
-// so the staged box holds them as re_hi, im_hi, re_lo, im_lo; d0, d1 and the batch dimension
-// keep their element strides e0 (rows) and eb.
-// halves = 1: the box holds one of re / im (the CTA-pair form, each CTA staging its half).
-static cudaError_t map5_pair(CUtensorMap* m, void* base, uint64_t d0, uint64_t d1, uint64_t batch, uint64_t e0,
-                             uint64_t ps, uint64_t eb, uint32_t rows, uint32_t halves = 2) {
+// The same array for the CTA-pair form, whose CTAs each stage one of the re / im halves: x runs
+// over a row's blocks (chunk * 128 + 32 for the im planes), the third dimension over hi / lo.
+static cudaError_t map_split_half(CUtensorMap* m, void* base, int ld, size_t rows, size_t batch, uint32_t box_rows) {
   tcg::MapSpec s;
-  s.dims[0] = d0; s.dims[1] = d1; s.dims[2] = 2; s.dims[3] = 2; s.dims[4] = batch;
-  s.strides[0] = e0 * sizeof(__half);
-  s.strides[1] = 2 * ps * sizeof(__half);   // re -> im
-  s.strides[2] = ps * sizeof(__half);       // hi -> lo
-  s.strides[3] = eb * sizeof(__half);
-  s.box[0] = 32; s.box[1] = rows; s.box[2] = halves; s.box[3] = 2; s.box[4] = 1;
+  s.dims[0] = (uint64_t)4 * ld; s.dims[1] = rows; s.dims[2] = 2; s.dims[3] = batch; s.dims[4] = 1;
+  s.strides[0] = (uint64_t)4 * ld * sizeof(__half);
+  s.strides[1] = 2 * SP_PLANE * sizeof(__half);
+  s.strides[2] = (uint64_t)4 * ld * rows * sizeof(__half);
+  s.strides[3] = (uint64_t)4 * ld * rows * batch * sizeof(__half);
+  s.box[0] = 32; s.box[1] = box_rows; s.box[2] = 2; s.box[3] = 1; s.box[4] = 1;
   return tcg::make_map(m, base, s);
 }
 
@@ -215,12 +208,6 @@ static cudaError_t map5_pair(CUtensorMap* m, void* base, uint64_t d0, uint64_t d
 constexpr int ST = tcg::STORE_THREADS;
 // scales are powers of two: the reciprocal is exact, and a product with it is the quotient
 __device__ __forceinline__ float rcp2(float s) { return __frcp_rn(s); }
-// x * s of two neighbours as fp16 hi and lo pairs (split_val on both, packed conversions)
-__device__ __forceinline__ void split_pair(float x0, float x1, __half2& hi, __half2& lo) {
-  hi = __floats2half2_rn(x0, x1);
-  const float2 h = __half22float2(hi);
-  lo = __floats2half2_rn(x0 - h.x, x1 - h.y);
-}
 
 // Gh[ws] = B^T + S^-T phi_perp^T : rows i = (k1, a), cols (k2, p); written to g32 in tile
 // layout.  B = A (A^dag A)^-1 and phi_perp = phi - B S (see green()).
@@ -239,7 +226,7 @@ struct GreenP {
     b = t / (nt_n * mt_n);
   }
   __device__ tcg::Coords coords(int b, int mt, int nt, int kc) const {
-    tcg::Coords c = {{kc * 32, mt * 128, 0, b, 0}, {kc * 32, nt * BN, 0, 0, b}};
+    tcg::Coords c = {{0, mt * 128, 0, kc, b}, {0, nt * BN, 0, kc, b}};
     return c;
   }
   template <class R>
@@ -289,8 +276,8 @@ struct ForceBiasP {
   }
   // rows = Cholesky index g of LH[Q][k] (A), columns = walkers (B = spin-summed Gh)
   __device__ tcg::Coords coords(int b, int mt, int nt, int kc) const {
-    const int Q = b / ng, k = (b % ng) * kg + kc / kcb, c0 = (kc % kcb) * 32;
-    tcg::Coords c = {{c0, mt * 128, 0, k, Q}, {c0, nt * BN, 0, 0, k * nk + kminus[k * nk + Q]}};
+    const int Q = b / ng, k = (b % ng) * kg + kc / kcb, ch = kc % kcb;
+    tcg::Coords c = {{0, mt * 128, 0, ch, Q * nk + k}, {0, nt * BN, 0, ch, k * nk + kminus[k * nk + Q]}};
     return c;
   }
   // down the rows: consecutive threads write consecutive g of one walker
@@ -342,14 +329,13 @@ struct VhsP {
   }
   // rows (p, r) of L[Q][k] (A), columns = walkers (B = y[Q])
   __device__ tcg::Coords coords(int b, int mt, int nt, int kc) const {
-    const int Q = b / nk, k = b % nk;
-    tcg::Coords c = {{kc * 32, mt * 128, 0, k, Q}, {kc * 32, nt * BN, 0, 0, Q}};
+    tcg::Coords c = {{0, mt * 128, 0, kc, b}, {0, nt * BN, 0, kc, b / nk}};
     return c;
   }
   template <class R>
   __device__ void store_tile(int b, int mt, int nt, const float2* tile, int tid, int, R ready) const {
     const int Q = b / nk, k = b % nk, kq = kminus[k * nk + Q];
-    const size_t ps = (size_t)NM * NMp;
+    const size_t pw = (size_t)4 * NM * NMp;   // one walker's V
     const float* sy = s_y + Q * W + nt * BN;
     const int wn = min(BN, W - nt * BN);
     bool bad = false;
@@ -358,7 +344,7 @@ struct VhsP {
       // 4-byte aligned pair of the output row, so each plane takes one 32-bit store; a thread
       // keeps one row pair and walks over the walkers
       const int rp = tid % 64, pr = mt * 128 + 2 * rp, pp = pr / M, rr = pr - pp * M;
-      __half* o = v_sp + (size_t)nt * BN * 4 * ps + (size_t)(k * M + pp) * NMp + kq * M + rr;
+      __half* o = v_sp + (size_t)nt * BN * pw + sp_at(k * M + pp, NMp, kq * M + rr);
       if (!ready() || pr >= M * M) return;
 #pragma unroll 4
       for (int c = tid / 64; c < wn; c += ST / 64) {
@@ -366,20 +352,12 @@ struct VhsP {
         const float2 v0 = tile[(2 * rp) * tcg::STAGE_LD + c], v1 = tile[(2 * rp + 1) * tcg::STAGE_LD + c];
         const float r0 = v0.x * st, i0 = v0.y * st, r1 = v1.x * st, i1 = v1.y * st;
         bad |= !(fmaxf(fmaxf(fabsf(r0), fabsf(i0)), fmaxf(fabsf(r1), fabsf(i1))) < 60000.f);
-        __half* base = o + (size_t)c * 4 * ps;
-        __half2 hi, lo;
-        split_pair(r0, r1, hi, lo);
-        *reinterpret_cast<__half2*>(base) = hi;
-        *reinterpret_cast<__half2*>(base + ps) = lo;
-        split_pair(i0, i1, hi, lo);
-        *reinterpret_cast<__half2*>(base + 2 * ps) = hi;
-        *reinterpret_cast<__half2*>(base + 3 * ps) = lo;
+        put4f_pair(o + (size_t)c * pw, r0, i0, r1, i1);
       }
     } else {
       // down the rows: consecutive threads write consecutive r of one (walker, p)
       const int r = tid % 128, pr = mt * 128 + r, pp = pr / M, rr = pr - pp * M;
-      __half* o = v_sp + (size_t)nt * BN * 4 * ps;
-      const size_t at = (size_t)(k * M + pp) * NMp + kq * M + rr;
+      __half* o = v_sp + (size_t)nt * BN * pw + sp_at(k * M + pp, NMp, kq * M + rr);
       if (!ready() || pr >= M * M) return;
 #pragma unroll 4
       for (int c = tid / 128; c < wn; c += ST / 128) {
@@ -387,7 +365,7 @@ struct VhsP {
         const float2 v = tile[r * tcg::STAGE_LD + c];
         const float vr = v.x * st, vi = v.y * st;
         bad |= !(fabsf(vr) < 60000.f && fabsf(vi) < 60000.f);
-        put4f(o + (size_t)c * 4 * ps, ps, at, vr, vi);
+        put4f(o + (size_t)c * pw, vr, vi);
       }
     }
     if (bad) atomicExch(overflow, 1);
@@ -412,14 +390,14 @@ struct TaylorP {
   const float* s_t;
   const float2* p32;  // [W][R][NM] phi' in fp32
   float4* corr;       // [W][R][NM] (d, .) with d = phi' - phi on entry; (phi'' - phi, phi'') after the last step
-  __half* t_next;     // [W][4][R][NMp]
+  __half* t_next;     // [W][R][NMp]
   __device__ void tile(int t, int& b, int& mt, int& nt) const {
     nt = t % nt_n;
     mt = (t / nt_n) % mt_n;
     b = t / (nt_n * mt_n);
   }
   __device__ tcg::Coords coords(int b, int mt, int nt, int kc) const {
-    tcg::Coords c = {{kc * 32, mt * 128, 0, b, 0}, {kc * 32, nt * BN, 0, 0, b}};
+    tcg::Coords c = {{0, mt * 128, 0, kc, b}, {0, nt * BN, 0, kc, b}};
     return c;
   }
   // Elements are taken in batches of U per thread, the next batch's loads issued before this
@@ -473,8 +451,7 @@ struct TaylorP {
     } else if ((NM & 1) == 0) {
       // even NM: a thread takes two adjacent columns, one 16-byte load of phi' and one
       // 32-bit store per plane
-      const size_t ps = (size_t)R * NMp;
-      __half* tb = t_next + (size_t)b * 4 * ps;
+      __half* tb = t_next + (size_t)b * 4 * R * NMp;
       const float4* pb = reinterpret_cast<const float4*>(p32 + (size_t)b * R * NM);
       batches<128 * (BN / 2), float4>(
           tid,
@@ -486,19 +463,12 @@ struct TaylorP {
             const int r = e / (BN / 2), c = 2 * (e % (BN / 2)), j = mt * 128 + r, i = nt * BN + c;
             if (j >= R || i >= NM) return;
             const float2 v0 = tile[r * tcg::STAGE_LD + c], v1 = tile[r * tcg::STAGE_LD + c + 1];
-            __half* o = tb + (size_t)j * NMp + i;
-            __half2 hi, lo;
-            split_pair(fmaf(x.x, sc, v0.x * st), fmaf(x.z, sc, v1.x * st), hi, lo);
-            *reinterpret_cast<__half2*>(o) = hi;
-            *reinterpret_cast<__half2*>(o + ps) = lo;
-            split_pair(fmaf(x.y, sc, v0.y * st), fmaf(x.w, sc, v1.y * st), hi, lo);
-            *reinterpret_cast<__half2*>(o + 2 * ps) = hi;
-            *reinterpret_cast<__half2*>(o + 3 * ps) = lo;
+            put4f_pair(tb + sp_at(j, NMp, i), fmaf(x.x, sc, v0.x * st), fmaf(x.y, sc, v0.y * st),
+                       fmaf(x.z, sc, v1.x * st), fmaf(x.w, sc, v1.y * st));
           },
           ready);
     } else {
-      const size_t ps = (size_t)R * NMp;
-      __half* tb = t_next + (size_t)b * 4 * ps;
+      __half* tb = t_next + (size_t)b * 4 * R * NMp;
       const float2* pb = p32 + (size_t)b * R * NM;
       batches<128 * BN, float2>(
           tid,
@@ -510,7 +480,7 @@ struct TaylorP {
             const int r = e / BN, c = e % BN, j = mt * 128 + r, i = nt * BN + c;
             if (j >= R || i >= NM) return;
             const float2 v = tile[r * tcg::STAGE_LD + c];
-            put4f(tb, ps, (size_t)j * NMp + i, fmaf(x.x, sc, v.x * st), fmaf(x.y, sc, v.y * st));
+            put4f(tb + sp_at(j, NMp, i), fmaf(x.x, sc, v.x * st), fmaf(x.y, sc, v.y * st));
           },
           ready);
     }
@@ -526,10 +496,8 @@ struct ExchangeP {
   static constexpr bool kStreamB = true;   // Z streams through L2 once per launch when mt_n == 1
   static constexpr int kStages = STAGES_LIGHT;
   int tiles, kchunks;
-  int mt_n, nt_n, WS, nk, nMp;
-  const int* kminus;
-  const int* minus;
-  const int4* tri;
+  int mt_n, nt_n, WS, nMp;
+  const int2* blocks;  // [T] Green's-function blocks of a triple: the A operand's, the partner's
   const float* s_g;
   const float* s_z;
   const float2* g32;  // [Nk][Nk][WS][n*Mp]
@@ -542,8 +510,7 @@ struct ExchangeP {
     b = t / (nt_n * mt_n);
   }
   __device__ tcg::Coords coords(int t, int mt, int nt, int kc) const {
-    const int4 q = tri[t];  // (Q, k, kx, weight)
-    tcg::Coords c = {{kc * 32, mt * 128, 0, kminus[q.y * nk + q.x], q.z}, {kc * 32, nt * BN, 0, 0, t}};
+    tcg::Coords c = {{0, mt * 128, 0, kc, blocks[t].x}, {0, nt * BN, 0, kc, t}};
     return c;
   }
   // Each store warp takes 128 / (store warps) rows of the tile, four at a time: eight lanes per
@@ -551,17 +518,18 @@ struct ExchangeP {
   // four whole 128-byte lines.  Every load of the tile is issued before the tile is waited for.
   template <class R>
   __device__ void store_tile(int t, int mt, int nt, const float2* tile, int tid, int lane, R ready) const {
-    const int4 q = tri[t];
-    const int kxq = kminus[q.z * nk + minus[q.x]];  // kx + Q
-    const float2* gb = g32 + ((size_t)q.y * nk + kxq) * WS * nMp + nt * BN;
+    const float2* gb = g32 + (size_t)blocks[t].y * WS * nMp + nt * BN;
     // padding columns (s >= M) of Z_t are zero, so every column below n*Mp takes part
     const int pairs = min(BN, nMp - nt * BN) / 2;
     constexpr int ROWS = 128 * 32 / ST, IT = ROWS / 4, UJ = BN / 16;   // rows per warp and lane, pieces per lane
     const int ri = lane >> 3, cl = lane & 7, r0 = (tid >> 5) * ROWS;
+    const float inv_z = rcp2(s_z[t]);
     float4 gv[IT][UJ];
+    float inv[IT];
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
       const int ws = mt * 128 + r0 + 4 * it + ri;
+      inv[it] = ws < WS ? s_g[ws] : 1.f;
       const float4* g4 = reinterpret_cast<const float4*>(gb + (size_t)ws * nMp);
 #pragma unroll
       for (int u = 0; u < UJ; ++u) {
@@ -570,7 +538,6 @@ struct ExchangeP {
       }
     }
     if (!ready()) return;
-    const float inv_z = 1.f / s_z[t];
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
       const int r = r0 + 4 * it + ri, ws = mt * 128 + r;
@@ -592,8 +559,8 @@ struct ExchangeP {
         pi += __shfl_xor_sync(0xffffffffu, pi, o);
       }
       if (cl == 0 && ws < WS) {
-        const float inv = inv_z / s_g[ws];   // powers of two: exact after the sum
-        xpart[((size_t)t * nt_n + nt) * WS + ws] = make_double2((double)(pr * inv), (double)(pi * inv));
+        const float f = inv_z * rcp2(inv[it]);   // powers of two: exact after the sum
+        xpart[((size_t)t * nt_n + nt) * WS + ws] = make_double2((double)(pr * f), (double)(pi * f));
       }
     }
   }
@@ -637,7 +604,7 @@ struct AdjointP {
   __device__ tcg::Coords coords(int b, int mt, int nt, int kc) const {
     int tf, km, kx, kk;
     split_k(b, kc, tf, km, kx, kk);
-    tcg::Coords c = {{kk * 32, mt * 128, 0, km, kx}, {kk * 32, nt * BN, 0, 0, tf}};
+    tcg::Coords c = {{0, mt * 128, 0, kk, kx * nk + km}, {0, nt * BN, 0, kk, tf}};
     return c;
   }
   __device__ float chunk_scale(int b, int kc) const {
@@ -676,7 +643,7 @@ struct GramP {
   }
   __device__ tcg::Coords coords(int ws, int mt, int nt, int kc) const {
     const int w = ws >> 1, sp = ws & 1;
-    tcg::Coords c = {{kc * 32, sp * N + mt * 128, 0, w, 0}, {kc * 32, sp * N + nt * BN, 0, 0, w}};
+    tcg::Coords c = {{0, sp * N + mt * 128, 0, kc, w}, {0, sp * N + nt * BN, 0, kc, w}};
     return c;
   }
   template <class R>
@@ -710,7 +677,7 @@ struct ApplyRP {
     b = t / (nt_n * mt_n);
   }
   __device__ tcg::Coords coords(int ws, int mt, int nt, int kc) const {
-    tcg::Coords c = {{kc * 32, mt * 128, 0, ws, 0}, {kc * 32, nt * BN, 0, 0, ws}};
+    tcg::Coords c = {{0, mt * 128, 0, kc, ws}, {0, nt * BN, 0, kc, ws}};
     return c;
   }
   template <class R>
@@ -765,7 +732,7 @@ __global__ void maxabs_kernel(const zc* src, size_t per, unsigned long long* out
   }
 }
 
-// src[m][rows][cols] (FP64) -> dst[m][4][rows][ldd] with the per-matrix scale; grid (nmat, chunks)
+// src[m][rows][cols] (FP64) -> dst[m][rows][ldd] with the per-matrix scale; grid (nmat, chunks)
 __global__ void split_rows_kernel(const zc* src, int rows, int cols, int ldd, const unsigned long long* mx,
                                   float* scale, __half* dst) {
   const int mI = blockIdx.x;
@@ -774,24 +741,22 @@ __global__ void split_rows_kernel(const zc* src, int rows, int cols, int ldd, co
   const size_t per = (size_t)rows * cols, chunk = (per + gridDim.y - 1) / gridDim.y;
   const size_t b = blockIdx.y * chunk, e_end = min(per, b + chunk);
   const zc* p = src + (size_t)mI * per;
-  const size_t ps = (size_t)rows * ldd;
-  __half* o = dst + (size_t)mI * 4 * ps;
+  __half* o = dst + (size_t)mI * 4 * rows * ldd;
   for (size_t e = b + threadIdx.x; e < e_end; e += blockDim.x) {
     const size_t i = e / cols, j = e % cols;
-    put4(o, ps, i * ldd + j, p[e].x, p[e].y, s);
+    put4(o + sp_at(i, ldd, (int)j), p[e].x, p[e].y, s);
   }
 }
 
-// src[m][rows][cols] (fp32) -> dst[m][4][rows][ldd] with the per-matrix scale; grid (nmat, chunks)
+// src[m][rows][cols] (fp32) -> dst[m][rows][ldd] with the per-matrix scale; grid (nmat, chunks)
 __global__ void split_rows32_kernel(const float2* src, int rows, int cols, int ldd, const unsigned long long* mx,
                                     float* scale, __half* dst) {
   const int mI = blockIdx.x;
   const float s = scale_from_bits(mx + mI);
   if (blockIdx.y == 0 && threadIdx.x == 0) scale[mI] = s;
   const float2* p = src + (size_t)mI * rows * cols;
-  const size_t ps = (size_t)rows * ldd;
-  __half* o = dst + (size_t)mI * 4 * ps;
-  if ((cols & 1) == 0 && (ldd & 1) == 0) {
+  __half* o = dst + (size_t)mI * 4 * rows * ldd;
+  if ((cols & 1) == 0) {
     // column pairs: one 16-byte load and one 32-bit store per plane
     const size_t per = (size_t)rows * (cols / 2), chunk = (per + gridDim.y - 1) / gridDim.y;
     const size_t b = blockIdx.y * chunk, e_end = min(per, b + chunk);
@@ -799,16 +764,7 @@ __global__ void split_rows32_kernel(const float2* src, int rows, int cols, int l
     for (size_t e = b + threadIdx.x; e < e_end; e += blockDim.x) {
       const size_t i = e / (cols / 2), j = 2 * (e % (cols / 2));
       const float4 v = p4[(i * cols + j) / 2];
-      __half h0, l0, h1, l1;
-      __half* q = o + i * ldd + j;
-      split_val(v.x * s, h0, l0);
-      split_val(v.z * s, h1, l1);
-      *reinterpret_cast<__half2*>(q) = __halves2half2(h0, h1);
-      *reinterpret_cast<__half2*>(q + ps) = __halves2half2(l0, l1);
-      split_val(v.y * s, h0, l0);
-      split_val(v.w * s, h1, l1);
-      *reinterpret_cast<__half2*>(q + 2 * ps) = __halves2half2(h0, h1);
-      *reinterpret_cast<__half2*>(q + 3 * ps) = __halves2half2(l0, l1);
+      put4f_pair(o + sp_at(i, ldd, (int)j), v.x * s, v.y * s, v.z * s, v.w * s);
     }
     return;
   }
@@ -816,7 +772,7 @@ __global__ void split_rows32_kernel(const float2* src, int rows, int cols, int l
   const size_t b = blockIdx.y * chunk, e_end = min(per, b + chunk);
   for (size_t e = b + threadIdx.x; e < e_end; e += blockDim.x) {
     const size_t i = e / cols, j = e % cols;
-    put4f(o, ps, i * ldd + j, p[e].x * s, p[e].y * s);
+    put4f(o + sp_at(i, ldd, (int)j), p[e].x * s, p[e].y * s);
   }
 }
 
@@ -870,19 +826,19 @@ __global__ void split_green_kernel(const float2* g32, const unsigned long long* 
   }
   const unsigned per = (unsigned)(nk * nk * nMp), chunk = (per + gridDim.y - 1) / gridDim.y;
   const unsigned b = blockIdx.y * chunk, e_end = min(per, b + chunk);
-  const size_t psg = (size_t)nk * nk * WS * nMp, pss = (size_t)nk * nk * W * nMp;
   for (unsigned e = b + threadIdx.x; e < e_end; e += blockDim.x) {
     const unsigned blk = e / nMp, off = e % nMp;
     const size_t i0 = ((size_t)blk * WS + 2 * w) * nMp + off;
     const float2 a = g32[i0];
     const float2 c = g32[i0 + nMp];
-    put4f(gsp, psg, i0, a.x * s0, a.y * s0);
-    put4f(gsp, psg, i0 + nMp, c.x * s1, c.y * s1);
-    put4f(gsum, pss, ((size_t)blk * W + w) * nMp + off, (a.x + c.x) * ss, (a.y + c.y) * ss);
+    const size_t row = (size_t)blk * WS + 2 * w;
+    put4f(gsp + sp_at(row, nMp, off), a.x * s0, a.y * s0);
+    put4f(gsp + sp_at(row + 1, nMp, off), c.x * s1, c.y * s1);
+    put4f(gsum + sp_at((size_t)blk * W + w, nMp, off), (a.x + c.x) * ss, (a.y + c.y) * ss);
   }
 }
 
-// y [W][Nk][G] (zc, carries sqrt(dt)) -> y_sp [4][Nk][W][Gp] of y / s_l[Q][g], scale s_y[Q][W]
+// y [W][Nk][G] (zc, carries sqrt(dt)) -> y_sp [Nk][W][Gp] of y / s_l[Q][g], scale s_y[Q][W]
 __global__ void split_y_kernel(const zc* y, const float* s_l, __half* out, float* s_y, int nk, int W, int G, int Gp) {
   const int Q = blockIdx.x, w = blockIdx.y;
   __shared__ double red[32];
@@ -895,10 +851,9 @@ __global__ void split_y_kernel(const zc* y, const float* s_l, __half* out, float
   m = block_max(m, red);
   const float s = pow2_scale(m);
   if (threadIdx.x == 0) s_y[Q * W + w] = s;
-  const size_t ps = (size_t)nk * W * Gp;
   for (int g = threadIdx.x; g < G; g += blockDim.x) {
     const double f = 1.0 / (double)s_l[Q * G + g];
-    put4(out, ps, ((size_t)Q * W + w) * Gp + g, yp[g].x * f, yp[g].y * f, s);
+    put4(out + sp_at((size_t)Q * W + w, Gp, g), yp[g].x * f, yp[g].y * f, s);
   }
 }
 
@@ -1060,7 +1015,7 @@ __global__ void trial_projector_kernel(const zc* A, zc* B, zc* scratch, int M, i
   }
 }
 
-// phi [W][2][NM][N] (FP64) -> transposed split planes [W][4][2N][NMp] (rows = (spin, column)),
+// phi [W][2][NM][N] (FP64) -> transposed split planes [W][2N][NMp] (rows = (spin, column)),
 // per-walker scale; grid (W, chunks)
 __global__ void split_T_kernel(const zc* phi, const unsigned long long* mx, float* scale, __half* out, int NM, int N,
                                int NMp) {
@@ -1082,17 +1037,16 @@ __global__ void split_T_kernel(const zc* phi, const unsigned long long* mx, floa
     t[rr][jj] = v;
   }
   __syncthreads();
-  const size_t ps = (size_t)2 * N * NMp;
-  __half* o = out + (size_t)w * 4 * ps;
+  __half* o = out + (size_t)w * 4 * 2 * N * NMp;
   for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
     const int jj = e / 32, rr = e % 32, r = r0 + rr, j = j0 + jj;
-    if (r < NM && j < N) put4f(o, ps, ((size_t)sp * N + j) * NMp + r, t[rr][jj].x, t[rr][jj].y);
+    if (r < NM && j < N) put4f(o + sp_at(sp * N + j, NMp, r), t[rr][jj].x, t[rr][jj].y);
   }
 }
 
 // Gram = R^dag R (Cholesky, upper R in place) and X = R^-1, both in fp32 (the Gram
 // comes from the split GEMM, about 22 bits, so FP64 would add nothing), then the split
-// planes of X^T [WS][4][N][Np] with a per-ws scale.  One block per walker-spin, the
+// planes of X^T [WS][N][Np] with a per-ws scale.  One block per walker-spin, the
 // matrix in shared memory when it fits (SMEM), else in place in global memory.
 // R^-1 is formed by Gauss-Jordan elimination on the upper triangle: step j scales row j
 // by 1/r_jj and clears column j from the rows above it, N^3/6 complex multiply-adds with
@@ -1205,8 +1159,7 @@ __global__ void __launch_bounds__(CI_THREADS) chol_inv_kernel(float2* gram, __ha
   for (int w = 0; w < NW; ++w) m = fmaxf(m, s_red[w]);
   const float sc = pow2_scale((double)m);
   if (tid == 0) scale[ws] = sc;
-  const size_t ps = (size_t)N * Np;
-  __half* o = out + (size_t)ws * 4 * ps;
+  __half* o = out + (size_t)ws * 4 * N * Np;
   for (int e = tid; e < N * N; e += CI_THREADS) {
     const int jr = e / N, i = e % N;
     float2 v = make_float2(0.f, 0.f);
@@ -1214,7 +1167,7 @@ __global__ void __launch_bounds__(CI_THREADS) chol_inv_kernel(float2* gram, __ha
       v.x = (i == jr) ? 1.f : 0.f;
     else if (i <= jr)
       v = a[(size_t)i * N + jr];
-    put4f(o, ps, (size_t)jr * Np + i, v.x * sc, v.y * sc);
+    put4f(o + sp_at(jr, Np, i), v.x * sc, v.y * sc);
   }
 }
 
@@ -1330,33 +1283,31 @@ __global__ void static_scales_kernel(const zc* L, const zc* LH, float* s_l, floa
   }
 }
 
-// lh_sp[4][Q][k][g][a][Mp] and lt_sp[4][Q][k][(p,r)][Gp]; grid (Q*nk + k)
+// lh_sp[Q][k][g][a Mp] and lt_sp[Q][k][(p,r)][Gp]; grid (Q*nk + k)
 __global__ void static_split_kernel(const zc* L, const zc* LH, const float* s_l, const float* s_lh, __half* lh_sp,
                                     __half* lt_sp, int nk, int G, int Gp, int M, int Mp, int n) {
   const int b = blockIdx.x, Q = b / nk;
-  const size_t lh_ps = (size_t)nk * nk * G * n * Mp, lt_ps = (size_t)nk * nk * M * M * Gp;
   const zc* hp = LH + (size_t)b * G * n * M;
   for (int e = threadIdx.x; e < G * n * M; e += blockDim.x) {
     const int g = e / (n * M), a = (e / M) % n, r = e % M;
-    put4d(lh_sp, lh_ps, (((size_t)b * G + g) * n + a) * Mp + r, hp[e].x, hp[e].y, s_lh[Q * G + g]);
+    put4d(lh_sp + sp_at((size_t)b * G + g, n * Mp, a * Mp + r), hp[e].x, hp[e].y, s_lh[Q * G + g]);
   }
   const zc* lp = L + (size_t)b * G * M * M;
   for (int e = threadIdx.x; e < G * M * M; e += blockDim.x) {
     const int pr = e / G, g = e % G;  // g fastest in the output
     const zc v = lp[(size_t)g * M * M + pr];
-    put4d(lt_sp, lt_ps, ((size_t)b * M * M + pr) * Gp + g, v.x, v.y, s_l[Q * G + g]);
+    put4d(lt_sp + sp_at((size_t)b * M * M + pr, Gp, g), v.x, v.y, s_l[Q * G + g]);
   }
 }
 
 // Z_t[(a,s)][(b,r)] = sum_g LH[Q,k,g,a,r] LH[-Q,kx,g,b,s] in FP64, split per triple.
 __global__ void z_build_kernel(const zc* LH, const int4* tri, const int* minus, zc* scratch, __half* z_sp,
-                               float* s_z, int T, int rows, int nk, int G, int M, int n, int Mp) {
+                               float* s_z, int T, int nk, int G, int M, int n, int Mp) {
   const int nM = n * M;
   const size_t per = (size_t)nM * nM;
   zc* buf = scratch + (size_t)blockIdx.x * per;
   __shared__ double red[32];
   const int nMp = n * Mp;
-  const size_t ps = (size_t)rows * nMp * nMp;   // plane stride: z_sp holds `rows` matrices per plane
   for (int t = blockIdx.x; t < T; t += gridDim.x) {
     const int4 q = tri[t];
     const zc* L1 = LH + ((size_t)q.x * nk + q.y) * G * nM;            // LH[Q][k]
@@ -1378,26 +1329,25 @@ __global__ void z_build_kernel(const zc* LH, const int4* tri, const int* minus, 
     for (size_t e = threadIdx.x; e < per; e += blockDim.x) {
       const int r = (int)(e % M), b = (int)((e / M) % n), s = (int)((e / ((size_t)M * n)) % M),
                 a = (int)(e / ((size_t)M * n * M));
-      const size_t idx = ((size_t)t * nMp + a * Mp + s) * nMp + b * Mp + r;   // rows s >= M stay zero
-      put4d(z_sp, ps, idx, buf[e].x, buf[e].y, sc);
+      put4d(z_sp + sp_at((size_t)t * nMp + a * Mp + s, nMp, b * Mp + r), buf[e].x, buf[e].y, sc);   // rows s >= M stay zero
     }
     __syncthreads();
   }
 }
 
 // The partners' rows of z_sp: row T + j holds the transpose of canonical row pmap[j].
-__global__ void z_partner_kernel(__half* z_sp, float* s_z, const int* pmap, int T, int P, int rows, int nMp) {
-  const size_t per = (size_t)nMp * nMp, ps = (size_t)rows * per;
+__global__ void z_partner_kernel(__half* z_sp, float* s_z, const int* pmap, int T, int P, int nMp) {
+  const size_t per = (size_t)nMp * nMp;
   for (int j = blockIdx.x; j < P; j += gridDim.x) {
     const int i = pmap[j];
     if (threadIdx.x == 0) s_z[T + j] = s_z[i];
-    for (int pl = 0; pl < 4; ++pl) {
-      const __half* src = z_sp + pl * ps + (size_t)i * per;
-      __half* dst = z_sp + pl * ps + (size_t)(T + j) * per;
-      for (size_t e = threadIdx.x; e < per; e += blockDim.x) {
-        const size_t row = e / nMp, col = e % nMp;
-        dst[e] = src[col * nMp + row];
-      }
+    const __half* src = z_sp + (size_t)i * 4 * per;
+    __half* dst = z_sp + (size_t)(T + j) * 4 * per;
+    for (size_t e = threadIdx.x; e < per; e += blockDim.x) {
+      const int row = (int)(e / nMp), col = (int)(e % nMp);
+      const size_t a = sp_at(row, nMp, col), b = sp_at(col, nMp, row);
+#pragma unroll
+      for (int pl = 0; pl < 4; ++pl) dst[a + pl * SP_PLANE] = src[b + pl * SP_PLANE];
     }
   }
 }
@@ -1553,8 +1503,8 @@ static ExchangeP exchange_params(const afqmc_kp* h) {
   p.nt_n = cdiv(m->nMp, BN);
   p.tiles = m->T * p.mt_n * p.nt_n;
   p.kchunks = m->nMp / 32;
-  p.WS = m->WS; p.nk = h->nk; p.nMp = m->nMp;
-  p.kminus = h->kminus; p.minus = h->minus; p.tri = m->tri; p.s_g = m->s_g; p.s_z = m->s_z; p.g32 = m->g32;
+  p.WS = m->WS; p.nMp = m->nMp;
+  p.blocks = m->tri_blocks; p.s_g = m->s_g; p.s_z = m->s_z; p.g32 = m->g32;
   p.xpart = m->xpart;
   return p;
 }
@@ -1740,18 +1690,25 @@ static cudaError_t create_impl(afqmc_kp* h, cudaStream_t st) {
   MTRY(dalloc(h, &m->s_z, Tf, true, st));
   MTRY(dalloc(h, &m->tri, T, false, st));
   MTRY(dalloc(h, &m->zrow, Tf, false, st));
+  MTRY(dalloc(h, &m->tri_blocks, T, false, st));
+  std::vector<int2> blocks_h(T);
+  for (int i = 0; i < T; ++i) {
+    const int4 q = tri[i];
+    const int kmq = h->h_kminus[(size_t)q.y * nk + q.x], kxq = h->h_kminus[(size_t)q.z * nk + h->h_minus[q.x]];
+    blocks_h[i] = make_int2(q.z * nk + kmq, q.y * nk + kxq);
+  }
   int* pmap = nullptr;
   MTRY(dalloc(h, &pmap, std::max(P, 1), false, st));
   const int zctas = std::min(T, ZCTAS);
   MTRY(dalloc(h, &m->zscratch, std::max((size_t)zctas * nM * nM, (size_t)nk * n * 2 * n), false, st));
   MTRY(cudaMemcpyAsync(m->tri, tri.data(), sizeof(int4) * T, cudaMemcpyHostToDevice, st));
   MTRY(cudaMemcpyAsync(m->zrow, zrow_h.data(), sizeof(int) * Tf, cudaMemcpyHostToDevice, st));
+  MTRY(cudaMemcpyAsync(m->tri_blocks, blocks_h.data(), sizeof(int2) * T, cudaMemcpyHostToDevice, st));
   if (P) MTRY(cudaMemcpyAsync(pmap, pmap_h.data(), sizeof(int) * P, cudaMemcpyHostToDevice, st));
-  z_build_kernel<<<zctas, 256, 0, st>>>(h->LH, m->tri, h->minus, m->zscratch, m->z_sp, m->s_z, T, Tf, nk, G, M, n,
-                                        Mp);
+  z_build_kernel<<<zctas, 256, 0, st>>>(h->LH, m->tri, h->minus, m->zscratch, m->z_sp, m->s_z, T, nk, G, M, n, Mp);
   AFQMC_LAUNCHED(h);
   if (P) {
-    z_partner_kernel<<<std::min(P, 4096), 256, 0, st>>>(m->z_sp, m->s_z, pmap, T, P, Tf, nMp);
+    z_partner_kernel<<<std::min(P, 4096), 256, 0, st>>>(m->z_sp, m->s_z, pmap, T, P, nMp);
     AFQMC_LAUNCHED(h);
   }
   MTRY(cudaGetLastError());
@@ -1808,39 +1765,23 @@ static cudaError_t create_impl(afqmc_kp* h, cudaStream_t st) {
   MTRY(set_one_body(h, st));
 
   // tensor maps
-  MTRY(map5(&m->m_sinvt, m->sinvt_sp, {(uint64_t)Np, (uint64_t)N, 4, (uint64_t)WS, 1},
-            {(uint64_t)Np, (uint64_t)N * Np, (uint64_t)4 * N * Np, (uint64_t)WS * 4 * N * Np}, 128));
-  MTRY(map5_pair(&m->m_phi, m->phi_sp, (uint64_t)Np, (uint64_t)NM, (uint64_t)WS, (uint64_t)Np, (uint64_t)NM * Np,
-                 (uint64_t)4 * NM * Np, BN));
-  // blocks (k1, k2) of gsum addressed by the one index k1 Nk + k2 (stride W nMp)
-  MTRY(map5_pair(&m->m_gsum, m->gsum_sp, (uint64_t)nMp, (uint64_t)W, (uint64_t)nk * nk, (uint64_t)nMp,
-                 (uint64_t)nk * nk * W * nMp, (uint64_t)W * nMp, BN));
-  MTRY(map5(&m->m_lh, m->lh_sp, {(uint64_t)nMp, (uint64_t)G, 4, (uint64_t)nk, (uint64_t)nk},
-            {(uint64_t)nMp, (uint64_t)nk * nk * G * nMp, (uint64_t)G * nMp, (uint64_t)nk * G * nMp}, 128));
-  MTRY(map5_pair(&m->m_y, m->y_sp, (uint64_t)Gp, (uint64_t)W, (uint64_t)nk, (uint64_t)Gp, (uint64_t)nk * W * Gp,
-                 (uint64_t)W * Gp, BN));
-  MTRY(map5(&m->m_lt, m->lt_sp, {(uint64_t)Gp, (uint64_t)M * M, 4, (uint64_t)nk, (uint64_t)nk},
-            {(uint64_t)Gp, (uint64_t)nk * nk * M * M * Gp, (uint64_t)M * M * Gp, (uint64_t)nk * M * M * Gp}, 128));
-  for (int i = 0; i < 2; ++i)
-    MTRY(map5(&m->m_t[i], m->t_sp[i], {(uint64_t)NMp, (uint64_t)2 * N, 4, (uint64_t)W, 1},
-              {(uint64_t)NMp, (uint64_t)2 * N * NMp, (uint64_t)4 * 2 * N * NMp, (uint64_t)W * 4 * 2 * N * NMp}, 128));
-  MTRY(map5_pair(&m->m_v, m->v_sp, (uint64_t)NMp, (uint64_t)NM, (uint64_t)W, (uint64_t)NMp, (uint64_t)NM * NMp,
-                 (uint64_t)4 * NM * NMp, BN));
-  MTRY(map5_pair(&m->m_vp, m->v_sp, (uint64_t)NMp, (uint64_t)NM, (uint64_t)W, (uint64_t)NMp, (uint64_t)NM * NMp,
-                 (uint64_t)4 * NM * NMp, BN, 1));
-  MTRY(map5(&m->m_g, m->g_sp, {(uint64_t)nMp, (uint64_t)WS, 4, (uint64_t)nk, (uint64_t)nk},
-            {(uint64_t)nMp, (uint64_t)nk * nk * WS * nMp, (uint64_t)WS * nMp, (uint64_t)nk * WS * nMp}, 128));
+  const size_t nk2 = (size_t)nk * nk;
+  MTRY(map_split(&m->m_sinvt, m->sinvt_sp, Np, N, WS, 128));
+  MTRY(map_split(&m->m_phi, m->phi_sp, Np, NM, WS, BN));
+  MTRY(map_split(&m->m_gsum, m->gsum_sp, nMp, W, nk2, BN));   // block k1 Nk + k2
+  MTRY(map_split(&m->m_lh, m->lh_sp, nMp, G, nk2, 128));      // Q Nk + k
+  MTRY(map_split(&m->m_y, m->y_sp, Gp, W, nk, BN));
+  MTRY(map_split(&m->m_lt, m->lt_sp, Gp, (size_t)M * M, nk2, 128));   // Q Nk + k
+  for (int i = 0; i < 2; ++i) MTRY(map_split(&m->m_t[i], m->t_sp[i], NMp, (size_t)2 * N, W, 128));
+  MTRY(map_split(&m->m_v, m->v_sp, NMp, NM, W, BN));
+  MTRY(map_split_half(&m->m_vp, m->v_sp, NMp, NM, W, BN));
+  MTRY(map_split(&m->m_g, m->g_sp, nMp, WS, nk2, 128));   // block k1 Nk + k2
   // the exchange reads the canonical rows, the adjoint every row
-  MTRY(map5_pair(&m->m_z, m->z_sp, (uint64_t)nMp, (uint64_t)nMp, (uint64_t)T, (uint64_t)nMp,
-                 (uint64_t)Tf * nMp * nMp, (uint64_t)nMp * nMp, BN));
-  MTRY(map5_pair(&m->m_zall, m->z_sp, (uint64_t)nMp, (uint64_t)nMp, (uint64_t)Tf, (uint64_t)nMp,
-                 (uint64_t)Tf * nMp * nMp, (uint64_t)nMp * nMp, BN));
-  MTRY(map5(&m->m_phi_a, m->phi_sp, {(uint64_t)Np, (uint64_t)NM, 4, (uint64_t)WS, 1},
-            {(uint64_t)Np, (uint64_t)NM * Np, (uint64_t)4 * NM * Np, (uint64_t)WS * 4 * NM * Np}, 128));
-  MTRY(map5_pair(&m->m_sinvt_b, m->sinvt_sp, (uint64_t)Np, (uint64_t)N, (uint64_t)WS, (uint64_t)Np, (uint64_t)N * Np,
-                 (uint64_t)4 * N * Np, BN));
-  MTRY(map5_pair(&m->m_t0_b, m->t_sp[0], (uint64_t)NMp, (uint64_t)2 * N, (uint64_t)W, (uint64_t)NMp,
-                 (uint64_t)2 * N * NMp, (uint64_t)4 * 2 * N * NMp, BN));
+  MTRY(map_split(&m->m_z, m->z_sp, nMp, nMp, T, BN));
+  MTRY(map_split(&m->m_zall, m->z_sp, nMp, nMp, Tf, BN));
+  MTRY(map_split(&m->m_phi_a, m->phi_sp, Np, NM, WS, 128));
+  MTRY(map_split(&m->m_sinvt_b, m->sinvt_sp, Np, N, WS, BN));
+  MTRY(map_split(&m->m_t0_b, m->t_sp[0], NMp, (size_t)2 * N, W, BN));
   MTRY(set_smem_attr((const void*)gamma_assemble_kernel, sizeof(float2) * GA_W * G));
   MTRY(set_smem_attr((const void*)onebody_in_kernel, onebody_smem(h)));
   if (onebody_out_staged(h))

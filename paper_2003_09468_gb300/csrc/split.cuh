@@ -1,7 +1,6 @@
 // fp16 hi/lo operand split shared by the tensor-core GEMM operands (tc_gemm.cuh).
 //
-// A matrix enters a GEMM as four fp16 planes (hi, lo of the real part, hi, lo of the
-// imaginary part) of x*s, with s a power of two chosen per matrix so that the
+// A matrix enters a GEMM as four fp16 planes (hi and lo of the real and imaginary parts) of x*s, with s a power of two chosen per matrix so that the
 // largest |x*s| sits near SCALE_TARGET: far from the fp16 overflow, and high enough
 // that lo keeps its full 11 bits.
 #pragma once
@@ -30,13 +29,42 @@ __device__ __forceinline__ void split_val(float xs, __half& hi, __half& lo) {
   hi = __float2half_rn(xs);
   lo = __float2half_rn(xs - __half2float(hi));
 }
-__device__ __forceinline__ void put4f(__half* base, size_t plane_stride, size_t idx, float re, float im) {
+// Layout of a split matrix of `rows` rows (all matrices of a batch one after another) and `ld`
+// columns, ld a multiple of 32: every row in blocks of 32 columns, a block holding its four
+// planes one after another (re hi, im hi, re lo, im lo; 64 bytes each), so that the four planes
+// of an element lie in one 256-byte block: a producer's stores of a run of columns and a TMA
+// box's rows stay in neighbouring lines and in one memory page, where planes of whole matrices
+// would be scattered over four.
+constexpr int SP_PLANE = 32;
+enum : int { SP_RE_HI = 0, SP_IM_HI = SP_PLANE, SP_RE_LO = 2 * SP_PLANE, SP_IM_LO = 3 * SP_PLANE };
+// index of (row, col) in the re hi plane
+__host__ __device__ __forceinline__ size_t sp_at(size_t row, int ld, int col) {
+  return row * (size_t)(4 * ld) + (size_t)((col >> 5) * 128 + (col & 31));
+}
+// one element at `o` = base + sp_at(row, ld, col), already scaled
+__device__ __forceinline__ void put4f(__half* o, float re, float im) {
   __half h, l;
   split_val(re, h, l);
-  base[idx] = h;
-  base[plane_stride + idx] = l;
+  o[SP_RE_HI] = h;
+  o[SP_RE_LO] = l;
   split_val(im, h, l);
-  base[2 * plane_stride + idx] = h;
-  base[3 * plane_stride + idx] = l;
+  o[SP_IM_HI] = h;
+  o[SP_IM_LO] = l;
+}
+// x * s of two neighbours as fp16 hi and lo pairs (split_val on both, packed conversions)
+__device__ __forceinline__ void split_pair(float x0, float x1, __half2& hi, __half2& lo) {
+  hi = __floats2half2_rn(x0, x1);
+  const float2 h = __half22float2(hi);
+  lo = __floats2half2_rn(x0 - h.x, x1 - h.y);
+}
+// two elements of one row at even column: one 32-bit store per plane
+__device__ __forceinline__ void put4f_pair(__half* o, float re0, float im0, float re1, float im1) {
+  __half2 hi, lo;
+  split_pair(re0, re1, hi, lo);
+  *reinterpret_cast<__half2*>(o + SP_RE_HI) = hi;
+  *reinterpret_cast<__half2*>(o + SP_RE_LO) = lo;
+  split_pair(im0, im1, hi, lo);
+  *reinterpret_cast<__half2*>(o + SP_IM_HI) = hi;
+  *reinterpret_cast<__half2*>(o + SP_IM_LO) = lo;
 }
 }  // namespace mixed

@@ -2,9 +2,9 @@
 //
 //   D[m][n] = sum_k A[m][k] * B[n][k]          (complex, no conjugation)
 //
-// Operands live in global memory as four fp16 "planes" of the same shape,
-// K-major (k contiguous), padded to a multiple of 32 complex elements in k:
-//   plane 0 = hi(Re x*s), 1 = lo(Re x*s), 2 = hi(Im x*s), 3 = lo(Im x*s)
+// Operands live in global memory as four fp16 "planes", K-major and padded to a multiple of
+// 32 complex elements in k, in 256-byte blocks of 32 k by four planes (split.cuh):
+//   plane 0 = hi(Re x*s), 1 = hi(Im x*s), 2 = lo(Re x*s), 3 = lo(Im x*s)
 // with hi = fp16(x*s), lo = fp16(x*s - hi) and s a power-of-two scale chosen so
 // that |x*s| stays well inside the fp16 range.  Each real product is formed
 // from three fp16 products (hi*hi + hi*lo + lo*hi), accumulated in fp32 in
@@ -42,18 +42,18 @@ constexpr int TILE_BAR_THREADS = DRAIN_THREADS + STORE_THREADS;   // the tile ha
 // Registers per thread of the four groups: the drain holds 128 running sums and two TMEM load
 // buffers, the store groups their epilogue's loads in flight.  The shares add up to what the
 // launch gets (4 x 128 at 512 threads per SM), so every setmaxnreg.inc is served.
-constexpr int REGS_ISSUE = 64, REGS_DRAIN = 208, REGS_STORE = 120;
+constexpr int REGS_ISSUE = 48, REGS_DRAIN = 224, REGS_STORE = 120;
 static_assert(REGS_ISSUE + REGS_DRAIN + 2 * REGS_STORE <= 4 * (65536 / THREADS), "register shares");
 static_assert(THREADS == 512, "four warp groups");
 
+// TMA coordinates of a chunk's operands: (0, first row, 0, k chunk, matrix of the batch).
 struct Coords {
   int a[5];
   int b[5];
 };
 
-// B is staged with its planes in the order (re_hi, im_hi, re_lo, im_lo) (a tensor map whose
-// plane dimensions are (re/im, hi/lo)), so that [B_re; B_im] is one 128-row operand: one
-// N = 128 MMA gives [A_x B_re | A_x B_im], twelve MMAs per chunk.
+// With the planes staged in that order [B_re; B_im] is one 128-row operand: one N = 128 MMA
+// gives [A_x B_re | A_x B_im], twelve MMAs per chunk.
 //
 // Policy P provides:
 //   static constexpr bool kConjA;     D = sum conj(A) B instead of sum A B
@@ -147,8 +147,9 @@ __device__ __forceinline__ float chunk_factor(const P& p, int b, int kc) {
 // Tile 128 x BNP (BNP = 64): 4 x 64 columns per set, 2 sets = all 512 TMEM columns.
 constexpr int BNP = 64;
 
-// Accumulator columns per tcgen05.ld in the drain.
-constexpr int DRAIN_COLS = 8;
+// Accumulator columns per tcgen05.ld in the drain: every wait exposes the load's latency, so
+// few wide loads (with 8 columns a chunk's drain took 1250 clocks, longer than its MMAs).
+constexpr int DRAIN_COLS = 16;
 
 // Epilogue staging: the finished 128 x 64 tile as (re, im) fp32 pairs, rows padded to 65
 // entries so that row-per-thread and column-per-thread accesses both avoid bank conflicts.
@@ -268,11 +269,12 @@ __global__ void __launch_bounds__(THREADS, 1)
           if constexpr (PAIR) {
             // both CTAs' copies complete on the even CTA's full barrier
             if (leader) tc::mbar_arrive_expect_tx(&full[s], 2 * Lay::STAGE_BYTES);
-            Coords c = p.coords(b, 2 * mt + (int)rank, nt, kc);
-            c.b[2] += (int)rank;   // re planes in the even CTA, im planes in the odd one
+            const Coords c = p.coords(b, 2 * mt + (int)rank, nt, kc);
             const uint32_t fb = tc::mapa_shared(tc::smem_u32(&full[s]), 0);
             tc::tma_load_5d_pair(sa, ma, fb, c.a[0], c.a[1], c.a[2], c.a[3], c.a[4]);
-            tc::tma_load_5d_pair(sa + Lay::A_BYTES, mb, fb, c.b[0], c.b[1], c.b[2], c.b[3], c.b[4]);
+            // the pair's B map addresses a row's blocks through x: re planes in the even CTA, im
+            // planes in the odd one
+            tc::tma_load_5d_pair(sa + Lay::A_BYTES, mb, fb, c.b[3] * 128 + (int)rank * 32, c.b[1], 0, c.b[4], 0);
             continue;
           }
           tc::mbar_arrive_expect_tx(&full[s], Lay::STAGE_BYTES);
@@ -328,7 +330,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             break;
           }
           tc::fence_after_sync();
-          const uint64_t da = desc0 + (uint64_t)((s * Lay::STAGE_BYTES) >> 4);   // A planes: re_hi, re_lo, im_hi, im_lo
+          const uint64_t da = desc0 + (uint64_t)((s * Lay::STAGE_BYTES) >> 4);   // A planes: re_hi, im_hi, re_lo, im_lo
           const uint64_t db = da + (uint64_t)(Lay::A_BYTES >> 4);
           constexpr uint64_t PL = (BM * 64) >> 4, KK = 32 >> 4;   // next A plane, next 16-wide k half
           if constexpr (PAIR) {
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               const uint32_t dq = d + q * 2 * BNP;
-              const uint64_t hi = da + 2 * q * PL, lo = hi + PL;
+              const uint64_t hi = da + q * PL, lo = hi + 2 * PL;
               tc::mma_f16_pair(dq, lo, db, idp, 0);   // the chunk's first MMA overwrites the set
               tc::mma_f16_pair(dq, hi, db + LO, idp, 1);
               tc::mma_f16_pair(dq, lo + KK, db + KK, idp, 1);
@@ -357,7 +359,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               const uint32_t dq = d + q * 2 * BNP;
-              const uint64_t hi = da + 2 * q * PL, lo = hi + PL;
+              const uint64_t hi = da + q * PL, lo = hi + 2 * PL;
               tc::mma_f16(dq, lo, db, id2, 0);
               tc::mma_f16(dq, hi, db + LO, id2, 1);
               tc::mma_f16(dq, lo + KK, db + KK, id2, 1);
@@ -415,13 +417,13 @@ __global__ void __launch_bounds__(THREADS, 1)
         // accumulators are in flight while the other pair's columns are added
         constexpr int o_ri = BNP, o_ir = 2 * BNP, o_ii = 3 * BNP, DCOL = DRAIN_COLS;
         float xr[DCOL], yr[DCOL], xi[DCOL], yi[DCOL];
-        tc::tmem_ld8(d, xr);
-        tc::tmem_ld8(d + o_ii, yr);
+        tc::tmem_ld16(d, xr);
+        tc::tmem_ld16(d + o_ii, yr);
 #pragma unroll
         for (int gq = 0; gq < BNP / DCOL; ++gq) {
           tc::tmem_ld_wait(xr, yr);
-          tc::tmem_ld8(d + o_ri + gq * DCOL, xi);
-          tc::tmem_ld8(d + o_ir + gq * DCOL, yi);
+          tc::tmem_ld16(d + o_ri + gq * DCOL, xi);
+          tc::tmem_ld16(d + o_ir + gq * DCOL, yi);
 #pragma unroll
           for (int c = 0; c < DCOL; ++c) {
             const float v = P::kConjA ? xr[c] + yr[c] : xr[c] - yr[c];
@@ -432,8 +434,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           tc::tmem_ld_wait(xi, yi);
           if (gq + 1 < BNP / DCOL) {
-            tc::tmem_ld8(d + (gq + 1) * DCOL, xr);
-            tc::tmem_ld8(d + o_ii + (gq + 1) * DCOL, yr);
+            tc::tmem_ld16(d + (gq + 1) * DCOL, xr);
+            tc::tmem_ld16(d + o_ii + (gq + 1) * DCOL, yr);
           } else {
             // the set's last loads have landed: hand it back before the last additions
             tc::fence_before_sync();
