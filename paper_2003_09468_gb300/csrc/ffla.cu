@@ -10,6 +10,8 @@
 // bits at several times the speed.
 #include <cuda_fp16.h>
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 
@@ -27,9 +29,6 @@ constexpr int GJ_THREADS = 512;
 constexpr int GJ_WARPS = GJ_THREADS / 32;
 constexpr size_t OV_SMEM_TARGET = 96 * 1024;
 constexpr size_t SMEM_LIMIT = 220 * 1024;
-// largest N held in shared memory (N^2 float4 + per-row arrays within SMEM_LIMIT; < 128,
-// which the register-held pivot row of the shared-memory variant relies on)
-constexpr int GJ_SMEM_MAXN = 118;
 
 __device__ __forceinline__ float block_max_f(float v, float* red) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
@@ -112,7 +111,8 @@ __global__ void __launch_bounds__(OV_THREADS)
 // A zero or non-finite pivot marks the matrix singular: logdet = (-inf, 0), sing = 1,
 // flags[0] counts it, and the inverse written is zero.
 // INV output: the split planes of S^-T, out[b][N][Np] (split.cuh) with scale s_out[b].
-template <bool SMEM, bool INV>
+// For matrices too large for the cluster form below; the matrix stays in global memory (L2).
+template <bool INV>
 __global__ void __launch_bounds__(GJ_THREADS)
     gj_ff_kernel(float4* Sff, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out) {
   extern __shared__ __align__(16) unsigned char gj_smem[];
@@ -121,14 +121,11 @@ __global__ void __launch_bounds__(GJ_THREADS)
   __shared__ double s_red[GJ_WARPS];
   __shared__ float s_redf[GJ_WARPS];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float4* g = Sff + (size_t)b * N * N;
-  float4* a = SMEM ? reinterpret_cast<float4*>(gj_smem) : g;
-  float4* f = reinterpret_cast<float4*>(gj_smem + (SMEM ? (size_t)N * N * sizeof(float4) : 0));
+  float4* a = Sff + (size_t)b * N * N;
+  float4* f = reinterpret_cast<float4*>(gj_smem);
   double2* piv = reinterpret_cast<double2*>(f + N);
   int* perm = reinterpret_cast<int*>(piv + N);
   int* iperm = perm + N;
-  if (SMEM)
-    for (int e = tid; e < N * N; e += GJ_THREADS) a[e] = g[e];
   for (int i = tid; i < N; i += GJ_THREADS) perm[i] = i;
   if (tid == 0) {
     s_sing = 0;
@@ -201,31 +198,7 @@ __global__ void __launch_bounds__(GJ_THREADS)
     }
     __syncthreads();
     const float4* aj = a + (size_t)j * N;
-    if (SMEM) {
-      // N <= GJ_SMEM_MAXN < 128: each lane owns the columns lane + 32 h, h < 4, and keeps
-      // its part of row j in registers for all the rows it updates
-      float4 ajr[4];
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const int c = lane + 32 * h;
-        ajr[h] = (c < N) ? aj[c] : ffa::czero();
-      }
-      const int i0 = INV ? warp : j + 1 + warp;
-      for (int i = i0; i < N; i += GJ_WARPS) {
-        if (INV && i == j) continue;
-        const float4 fi = f[i];
-        float4* ai = a + (size_t)i * N;
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int c = lane + 32 * h;
-          if (c >= N || (!INV && c <= j)) continue;
-          if (INV && c == j)
-            ai[c] = ffa::cneg(ffa::cmul(fi, inv));
-          else
-            ai[c] = ffa::cfms(ai[c], fi, ajr[h]);
-        }
-      }
-    } else if (INV) {
+    if (INV) {
       for (int i = warp; i < N; i += GJ_WARPS) {
         if (i == j) continue;
         const float4 fi = f[i];
@@ -292,22 +265,17 @@ __global__ void __launch_bounds__(GJ_THREADS)
   }
 }
 
-// Blocked form of the same Gauss-Jordan inverse, matrix in shared memory.  Pivots are taken
-// in panels of GJB columns: within a panel every step updates only the panel's columns
-// (all rows), so that afterwards those columns hold the panel's accumulated transform T
-// (T - I has non-zeros only there); every other column c then receives the panel's row
-// swaps and one rank-GJB update c <- T c = c + (T - I)[:, panel] c[panel rows].  The
-// arithmetic per element is unchanged (N^3 double-float multiply-adds in all); the
-// rank-GJB update reads and writes each element once per panel instead of once per pivot,
-// with the panel's multipliers and rows reused from registers.
-// The matrix lives in shared memory when it fits (SMEM, N <= GJB_MAXN), else in place in
-// global memory (the overlap buffer, L2-resident while the CTA works on it): each panel then
-// reads and writes the matrix once, where the unblocked kernel does so once per pivot.
+// Blocked form of the same Gauss-Jordan inverse.  Pivots are taken in panels of GJB columns:
+// within a panel every step updates only the panel's columns (all rows), so that afterwards
+// those columns hold the panel's accumulated transform T (T - I has non-zeros only there); every
+// other column c then receives the panel's row swaps and one rank-GJB update
+// c <- T c = c + (T - I)[:, panel] c[panel rows].  The matrix lives in place in global memory
+// (the overlap buffer, L2-resident while the CTA works on it): each panel reads and writes the
+// matrix once, where the unblocked kernel does so once per pivot.
 constexpr int GJB = 8;
 static_assert(GJB == 8, "the panel's index arithmetic uses shifts by 3");
 constexpr int GJB_THREADS = 512;
 constexpr int GJB_WARPS = GJB_THREADS / 32;
-constexpr int GJB_MAXN = 112;   // N^2 + GJB N float4 + per-row arrays within SMEM_LIMIT
 constexpr int GJB_GLOBAL_MAXN = 1024;   // GJB N float4 + per-row arrays within SMEM_LIMIT
 
 // Pivot candidate key: larger |value| first, then the smaller row (m >= 0 and not NaN, so its
@@ -316,7 +284,6 @@ __device__ __forceinline__ unsigned long long pivot_key(float m, int i) {
   return ((unsigned long long)__float_as_uint(m) << 32) | (unsigned long long)(0xffffffffu - (unsigned)i);
 }
 
-template <bool SMEM>
 __global__ void __launch_bounds__(GJB_THREADS)
     gjb_ff_kernel(float4* Sff, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out) {
   extern __shared__ __align__(16) unsigned char gj_smem[];
@@ -326,15 +293,12 @@ __global__ void __launch_bounds__(GJB_THREADS)
   __shared__ float s_redf[GJB_WARPS];
   __shared__ int s_prow[GJB];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float4* g = Sff + (size_t)b * N * N;
-  float4* a = SMEM ? reinterpret_cast<float4*>(gj_smem) : g;   // [N][N]
-  float4* tmp = reinterpret_cast<float4*>(gj_smem) + (SMEM ? (size_t)N * N : 0);   // [GJB][N] panel rows
+  float4* a = Sff + (size_t)b * N * N;                    // [N][N]
+  float4* tmp = reinterpret_cast<float4*>(gj_smem);       // [GJB][N] panel rows
   float4* f = tmp + (size_t)GJB * N;                      // [N] multipliers
   double2* piv = reinterpret_cast<double2*>(f + N);
   int* perm = reinterpret_cast<int*>(piv + N);
   int* iperm = perm + N;
-  if (SMEM)
-    for (int e = tid; e < N * N; e += GJB_THREADS) a[e] = g[e];
   for (int i = tid; i < N; i += GJB_THREADS) perm[i] = i;
   if (tid == 0) s_swaps = 0;
   __syncthreads();
@@ -524,13 +488,488 @@ __global__ void __launch_bounds__(GJB_THREADS)
   }
 }
 
+// The same inverse (or log det alone) with the matrix in shared memory, its columns spread over
+// a cluster of C CTAs (C = 1 up to N = 110 here).  Per panel of GJB = 8 pivots:
+//   1. the CTA that owns the panel's columns eliminates them in registers, LPR lanes per row with
+//      8 / LPR of the row's entries each: per pivot a warp maximum and one more over the warps'
+//      candidates pick the row, the pivot row and the row it displaces go through shared memory,
+//      and every lane eliminates its own entries (INV: all rows, else the rows from the panel
+//      down), two barriers a pivot.  A pivot is a chain of about 250 dependent instructions
+//      (reciprocal, scaled row, update); several lanes per row keep the loop body short
+//      enough for the instruction cache (one lane with all eight entries took 3200 clocks a pivot);
+//   2. T - I (T the panel's accumulated transform) and the row moves go to every CTA of the cluster;
+//   3. each CTA moves the affected rows of its other columns and updates them,
+//      c += (T - I)[:, panel] c[panel rows]: a thread takes two rows of one column, consecutive
+//      threads consecutive columns, so that T is a broadcast.  INV: element by element the
+//      arithmetic of gjb_ff_kernel, so that both give the same bits; the log det alone, which is
+//      never rounded to a GEMM operand, uses biased accumulators (ff.cuh) of half the instructions.
+// The INV update is N^3 complex multiply-adds of 48 FP32 instructions, the panels 8 N^2 of 60: 230 us
+// at 128 instructions per clock and SM for one matrix of N = 108 per SM.
+constexpr size_t GC_SMEM_LIMIT = 228000;   // dynamic, beside 3.4 KB of static
+
+struct GcLayout {
+  int nloc, lda;   // columns per CTA (a multiple of GJB for C > 1), row stride in float4 (odd: columns and rows both conflict-free)
+  size_t T, tmp, piv, rmax, cs, perm, bytes;   // byte offsets
+};
+__host__ __device__ inline GcLayout gc_layout(int N, int C) {
+  GcLayout L;
+  L.nloc = C == 1 ? N : ((N + C - 1) / C + GJB - 1) / GJB * GJB;
+  L.lda = L.nloc | 1;
+  const int tb = C == 1 ? 1 : 2;   // the next panel's owner writes T while this panel's is still read
+  L.T = (size_t)N * L.lda * sizeof(float4);
+  L.tmp = L.T + (size_t)tb * N * GJB * sizeof(float4);
+  L.piv = L.tmp + (size_t)GJB * L.nloc * sizeof(float4);
+  L.rmax = L.piv + (size_t)L.nloc * sizeof(float4);
+  L.cs = L.rmax + (size_t)tb * N * sizeof(float);
+  L.perm = L.cs + (size_t)L.nloc * sizeof(float);
+  L.bytes = L.perm + (size_t)N * sizeof(int);
+  return L;
+}
+
+struct GcPanel {          // what the owner tells every CTA about one panel
+  int prow[GJB];          // pivot row of each step
+  int srcp[GJB];          // row (before the panel) that ends at pivot position j0 + l
+  int srcd[GJB];          // row that ends at position prow[l], where that lies below the panel
+  int singular;
+};
+
+template <int C, bool INV, int GC_THREADS, int LPR>
+__global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
+    gjc_ff_kernel(const float4* Sff, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out) {
+  namespace cg = cooperative_groups;
+  constexpr int GC_WARPS = GC_THREADS / 32, SLOTS = GJB / LPR;   // a lane's entries: columns sub + LPR k
+  extern __shared__ __align__(16) unsigned char gj_smem[];
+  __shared__ GcPanel s_panel[2];
+  __shared__ uint2 s_cand[2][GC_WARPS];   // a warp's pivot candidate: |value| bits, row
+  __shared__ float4 s_prow[2][GJB], s_jrow[2][GJB], s_scaled[GC_WARPS][GJB];
+  __shared__ int s_porig[2], s_jorig[2], s_next;
+  __shared__ double s_red[GC_WARPS];
+  __shared__ float s_redf[GC_WARPS];
+  __shared__ double s_ld[8][2];
+  __shared__ float s_max[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = C == 1 ? 0 : (int)(blockIdx.x % C), b = blockIdx.x / C;
+  const GcLayout L = gc_layout(N, C);
+  const int lda = L.lda, nloc = L.nloc, c0 = rank * nloc, nc = max(0, min(nloc, N - c0));
+  float4* a = reinterpret_cast<float4*>(gj_smem);
+  float4* Tbuf = reinterpret_cast<float4*>(gj_smem + L.T);
+  float4* tmp = reinterpret_cast<float4*>(gj_smem + L.tmp);
+  float4* piv = reinterpret_cast<float4*>(gj_smem + L.piv);
+  float* rmaxbuf = reinterpret_cast<float*>(gj_smem + L.rmax);
+  float* cs = reinterpret_cast<float*>(gj_smem + L.cs);
+  int* perm = reinterpret_cast<int*>(gj_smem + L.perm);
+  const float4* g = Sff + (size_t)b * N * N + c0;
+  if (nc > 0)
+    for (int e = tid; e < N * nc; e += GC_THREADS) {
+      const int i = e / nc, c = e - i * nc;
+      a[i * lda + c] = g[(size_t)i * N + c];
+    }
+  for (int i = tid; i < N; i += GC_THREADS) perm[i] = i;
+  int swaps = 0;   // thread 0's count
+  bool singular = false;
+  // the panel's row threads: LPR lanes per row
+  const int rows_threads = (N * LPR + 31) & ~31, row_warps = rows_threads >> 5;
+  const int ri = tid / LPR, sub = tid % LPR, group = lane & ~(LPR - 1);
+  const bool row_thread = tid < rows_threads;
+  float4 v[SLOTS];   // this lane's entries of the panel, kept until T may be written
+  if (C > 1) cg::this_cluster().sync();   // every CTA of the cluster runs before the first remote store
+  else __syncthreads();
+
+  // ---- 1. the panel at column j0 (local column jl), by the row threads of the CTA that owns it
+  auto factor = [&](int j0, int jl, int par) {
+    const int jb = min(GJB, N - j0), i = ri;
+    const bool active = i < N && (INV || i >= j0);
+#pragma unroll
+    for (int k = 0; k < SLOTS; ++k) {
+      const int l = sub + LPR * k;
+      v[k] = (active && l < jb) ? a[i * lda + jl + l] : ffa::czero();
+    }
+    int orig = i;
+    bool bad = false;   // the same for all row threads
+#pragma unroll 1
+    for (int jj = 0; jj < jb; ++jj) {
+      const int j = j0 + jj, q = jj & 1, slot = jj / LPR;
+      const bool holds = sub == jj % LPR;   // this lane has the row's entry of column j
+      float4 vj = v[0];
+#pragma unroll
+      for (int k = 1; k < SLOTS; ++k)
+        if (slot == k) vj = v[k];
+      const float m = fabsf(vj.x) + fabsf(vj.z);
+      const bool elig = holds && active && i >= j;
+      const unsigned key = (elig && !isnan(m)) ? __float_as_uint(m) : 0u;
+      const unsigned wk = __reduce_max_sync(FULL, key);
+      const unsigned who = __ballot_sync(FULL, elig && key == wk);   // the smallest row among equals
+      if (lane == 0) s_cand[q][warp] = make_uint2(wk, (unsigned)(tid + (who ? __ffs(who) - 1 : 0)) / LPR);
+      asm volatile("bar.sync 1, %0;" ::"r"(rows_threads) : "memory");
+      const uint2 cand = lane < row_warps ? s_cand[q][lane] : make_uint2(0u, 0u);
+      const unsigned best = __reduce_max_sync(FULL, cand.x);
+      const int p = (int)__shfl_sync(FULL, cand.y, __ffs(__ballot_sync(FULL, cand.x == best)) - 1);
+      if (best == 0u || best >= 0x7f800000u) {
+        bad = true;
+        break;
+      }
+      if (i == p) {
+#pragma unroll
+        for (int k = 0; k < SLOTS; ++k) s_prow[q][sub + LPR * k] = v[k];
+        s_porig[q] = orig;
+        if (holds) piv[jl + jj] = vj;
+      }
+      if (i == j && p != j) {
+#pragma unroll
+        for (int k = 0; k < SLOTS; ++k) s_jrow[q][sub + LPR * k] = v[k];
+        s_jorig[q] = orig;
+      }
+      if (tid == 0) s_panel[par].prow[jj] = p;
+      asm volatile("bar.sync 1, %0;" ::"r"(rows_threads) : "memory");
+      // every warp scales the pivot row for itself, one entry per lane
+      const float4 inv = ffa::crecip(s_prow[q][jj]);
+      if (lane < GJB) s_scaled[warp][lane] = lane == jj ? inv : ffa::cmul(s_prow[q][lane], inv);
+      if (p != j) {   // rows j and p trade places
+        if (i == p) {
+#pragma unroll
+          for (int k = 0; k < SLOTS; ++k) v[k] = s_jrow[q][sub + LPR * k];
+          orig = s_jorig[q];
+        }
+        if (i == j) orig = s_porig[q];
+      }
+      vj = v[0];
+#pragma unroll
+      for (int k = 1; k < SLOTS; ++k)
+        if (slot == k) vj = v[k];
+      const int from = group + jj % LPR;
+      float4 f = vj;
+      if (LPR > 1)
+        f = make_float4(__shfl_sync(FULL, vj.x, from), __shfl_sync(FULL, vj.y, from), __shfl_sync(FULL, vj.z, from),
+                        __shfl_sync(FULL, vj.w, from));
+      __syncwarp();
+      // row i -= f (row j / pivot); column j, whose entry of the scaled row is 1 / pivot, starts
+      // from zero (bit for bit -(f / pivot)), and the pivot row becomes the scaled row
+#pragma unroll
+      for (int k = 0; k < SLOTS; ++k) {
+        const float4 t = s_scaled[warp][sub + LPR * k];
+        const float4 from0 = (holds && slot == k) ? ffa::czero() : v[k];
+        const float4 e = ffa::cfms(from0, f, t);
+        v[k] = i == j ? t : e;
+      }
+      __syncwarp();
+    }
+    if (tid == 0) s_panel[par].singular = bad;
+    if (!bad && i < N) {
+#pragma unroll
+      for (int k = 0; k < SLOTS; ++k) {
+        const int l = sub + LPR * k;
+        if (active && l < jb) a[i * lda + jl + l] = v[k];
+        if (l >= jb || !active) v[k] = ffa::czero();
+        else if (i == j0 + l) v[k] = ffa::pack(ffa::add(ffa::re(v[k]), ffa::make(-1.f, 0.f)), ffa::im(v[k]));
+      }
+      if (sub == 0) {
+        if (i >= j0 && i < j0 + jb) s_panel[par].srcp[i - j0] = orig;
+        for (int l = 0; l < jb; ++l)
+          if (s_panel[par].prow[l] == i) s_panel[par].srcd[l] = orig;
+      }
+    }
+  };
+  // ---- T - I (v) to every CTA of the cluster; for C > 1 the row moves and the verdict too
+  auto publish = [&](int par) {
+    const int i = ri;
+    if (!s_panel[par].singular && i < N) {
+      float m = 0.f;
+      if constexpr (!INV) {   // the row's largest multiplier, for the biased accumulators
+#pragma unroll
+        for (int k = 0; k < SLOTS; ++k) m = fmaxf(m, fabsf(v[k].x) + fabsf(v[k].z));
+        const unsigned lanes = (LPR == 32 ? 0u : (1u << LPR)) - 1u;   // rows are whole groups of lanes
+#pragma unroll
+        for (int o = 1; o < LPR; o <<= 1) m = fmaxf(m, __shfl_xor_sync(lanes << group, m, o));
+      }
+#pragma unroll
+      for (int r = 0; r < C; ++r) {
+        float4* T = Tbuf + (size_t)par * N * GJB;
+        float* rm = rmaxbuf + (size_t)par * N;
+        if (C > 1) {
+          T = cg::this_cluster().map_shared_rank(T, r);
+          rm = cg::this_cluster().map_shared_rank(rm, r);
+        }
+#pragma unroll
+        for (int k = 0; k < SLOTS; ++k) T[i * GJB + sub + LPR * k] = v[k];
+        if (!INV && sub == 0) rm[i] = m;
+      }
+    }
+    if (C > 1 && tid < (int)(sizeof(GcPanel) / sizeof(int))) {
+      const int val = reinterpret_cast<const int*>(&s_panel[par])[tid];
+      for (int r = 0; r < C; ++r)
+        if (r != rank) reinterpret_cast<int*>(cg::this_cluster().map_shared_rank(&s_panel[par], r))[tid] = val;
+    }
+  };
+  // ---- 3. rows i0, i0 + 1 of local column c: += (T - I) tmp
+  auto update = [&](int j0, int par, int ip, int c) {
+    const int jb = min(GJB, N - j0), i0 = (INV ? 0 : j0 + jb) + 2 * ip;
+    const int i1 = min(i0 + 1, N - 1);   // an odd last row is done twice, stored once
+    const float4 a0 = a[i0 * lda + c], a1 = a[i1 * lda + c];
+    const float4* d0 = Tbuf + ((size_t)par * N + i0) * GJB;
+    const float4* d1 = Tbuf + ((size_t)par * N + i1) * GJB;
+    float4 v0, v1;
+    if constexpr (INV) {
+      ffa::cacc x0 = ffa::cacc_from(a0), x1 = ffa::cacc_from(a1);
+#pragma unroll 4
+      for (int l = 0; l < jb; ++l) {
+        const float4 t = tmp[l * nloc + c];
+        ffa::cacc_fma(x0, d0[l], t);
+        ffa::cacc_fma(x1, d1[l], t);
+      }
+      v0 = ffa::cacc_get(x0);
+      v1 = ffa::cacc_get(x1);
+    } else {
+      const float* rmax = rmaxbuf + (size_t)par * N;
+      const float cc = cs[c];
+      // a hair more than the exact sums: rmax and cs are sums of rounded leading parts
+      const float B0 = ffa::bias_of(fmaf(rmax[i0] * cc, 1.001f, 1.001f * fmaxf(fabsf(a0.x), fabsf(a0.z))));
+      const float B1 = ffa::bias_of(fmaf(rmax[i1] * cc, 1.001f, 1.001f * fmaxf(fabsf(a1.x), fabsf(a1.z))));
+      ffa::bacc r0 = ffa::bacc_from(ffa::re(a0), B0), m0 = ffa::bacc_from(ffa::im(a0), B0);
+      ffa::bacc r1 = ffa::bacc_from(ffa::re(a1), B1), m1 = ffa::bacc_from(ffa::im(a1), B1);
+#pragma unroll 4
+      for (int l = 0; l < GJB; ++l) {
+        const float4 t = tmp[l * nloc + c], x = d0[l], y = d1[l];
+        ffa::bacc_fma(r0, x.x, x.y, t.x, t.y);
+        ffa::bacc_fma(m0, x.x, x.y, t.z, t.w);
+        ffa::bacc_fma(r1, y.x, y.y, t.x, t.y);
+        ffa::bacc_fma(m1, y.x, y.y, t.z, t.w);
+        ffa::bacc_fma(r0, -x.z, -x.w, t.z, t.w);
+        ffa::bacc_fma(m0, x.z, x.w, t.x, t.y);
+        ffa::bacc_fma(r1, -y.z, -y.w, t.z, t.w);
+        ffa::bacc_fma(m1, y.z, y.w, t.x, t.y);
+      }
+      v0 = ffa::pack(ffa::bacc_get(r0, B0), ffa::bacc_get(m0, B0));
+      v1 = ffa::pack(ffa::bacc_get(r1, B1), ffa::bacc_get(m1, B1));
+    }
+    a[i0 * lda + c] = v0;
+    if (i0 + 1 < N) a[(i0 + 1) * lda + c] = v1;
+  };
+
+  if (rank == 0 && row_thread) {
+    factor(0, 0, 0);
+    asm volatile("bar.sync 1, %0;" ::"r"(rows_threads) : "memory");
+    if (C > 1) publish(0);
+  }
+  for (int j0 = 0, pan = 0; j0 < N; j0 += GJB, ++pan) {
+    const int jb = min(GJB, N - j0), par = C == 1 ? 0 : (pan & 1);
+    const int owner = C == 1 ? 0 : j0 / nloc, jl = j0 - owner * nloc;   // the panel's first local column
+    if (C > 1) {
+      cg::this_cluster().sync();
+    } else {
+      __syncthreads();   // the previous panel's T has been read for the last time
+      if (row_thread) publish(0);
+      __syncthreads();
+    }
+    if (s_panel[par].singular) {
+      singular = true;
+      break;
+    }
+    if (tid == 0) {
+      s_next = 0;
+      for (int l = 0; l < jb; ++l) {
+        const int p = s_panel[par].prow[l];
+        if (p != j0 + l) {
+          const int t = perm[j0 + l];
+          perm[j0 + l] = perm[p];
+          perm[p] = t;
+          ++swaps;
+        }
+      }
+    }
+    // ---- 2. the affected rows of the other columns (LU: those right of the panel): thread
+    // (column, half), half 0 the panel's rows (also kept in tmp), half 1 the rows they displaced
+    {
+      const int first = INV ? 0 : (rank < owner ? nc : (rank == owner ? jl + jb : 0));
+      const int x0 = INV && rank == owner ? jl : nc, own = INV && rank == owner ? jb : 0;
+      const int c1 = first + (tid >> 1), c = c1 + (c1 >= x0 ? own : 0), half = tid & 1;
+      const bool has = c < nc;
+      float4 x[GJB];
+#pragma unroll
+      for (int l = 0; l < GJB; ++l) {
+        const int src = half ? s_panel[par].srcd[l < jb ? l : 0] : s_panel[par].srcp[l < jb ? l : 0];
+        const bool need = has && l < jb && (!half || s_panel[par].prow[l] >= j0 + jb);
+        x[l] = need ? a[src * lda + c] : ffa::czero();
+      }
+      __syncthreads();
+      if (has && !half) {
+        float m = 0.f;
+#pragma unroll
+        for (int l = 0; l < GJB; ++l) {
+          tmp[l * nloc + c] = x[l];
+          if (l < jb) a[(j0 + l) * lda + c] = x[l];
+          m += fmaxf(fabsf(x[l].x), fabsf(x[l].z));
+        }
+        cs[c] = m;
+      } else if (has) {
+#pragma unroll
+        for (int l = 0; l < GJB; ++l)
+          if (l < jb && s_panel[par].prow[l] >= j0 + jb) a[s_panel[par].prow[l] * lda + c] = x[l];
+      }
+      __syncthreads();
+    }
+    // ---- 3. the rank-GJB update.  The next panel's columns first; then its row threads factor it
+    // while the other warps update the rest, and join them.
+    const int jn = j0 + GJB, jbn = min(GJB, N - jn);
+    const int nowner = jn >= N ? -1 : (C == 1 ? 0 : jn / nloc), nl = jn - nowner * nloc;
+    const int np = (N - (INV ? 0 : j0 + jb) + 1) / 2;
+    const bool mine = rank == nowner;
+    if (mine) {
+      for (int u = tid; u < np * GJB; u += GC_THREADS)
+        if ((u & (GJB - 1)) < jbn) update(j0, par, u / GJB, nl + (u & (GJB - 1)));
+      __syncthreads();
+      if (row_thread) {
+        const int parn = C == 1 ? 0 : ((pan + 1) & 1);
+        factor(jn, nl, parn);
+        if (C > 1) {
+          asm volatile("bar.sync 1, %0;" ::"r"(rows_threads) : "memory");
+          publish(parn);
+        }
+      }
+      __syncwarp();
+    }
+    // the rest: columns [first, nc) without [x0, x1)
+    const int first = INV ? 0 : (rank < owner ? nc : (rank == owner ? jl + jb + (mine ? jbn : 0) : (mine ? jbn : 0)));
+    const int x0 = !INV ? nc : (rank == owner ? jl : (mine ? nl : nc));
+    const int xn = !INV ? 0 : (rank == owner ? jb : 0) + (mine ? jbn : 0);
+    const int R = max(0, nc - first - xn), total = np * R;
+    for (;;) {
+      int u = 0;
+      if (lane == 0) u = atomicAdd(&s_next, 32);
+      u = __shfl_sync(FULL, u, 0) + lane;
+      if (u - lane >= total) break;
+      if (u < total) {
+        const int ip = u / R, c1 = first + u - ip * R;
+        update(j0, par, ip, c1 + (c1 >= x0 ? xn : 0));
+      }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  // ---- log det from the pivots (each CTA its own columns')
+  double lg = 0.0, an = 0.0;
+  if (!singular)
+    for (int c = tid; c < nc; c += GC_THREADS) {
+      const double2 v = make_double2(ffa::to_double(ffa::re(piv[c])), ffa::to_double(ffa::im(piv[c])));
+      lg += 0.5 * log(v.x * v.x + v.y * v.y);
+      an += atan2(v.y, v.x);
+    }
+  lg = block_sum_d(lg, s_red);
+  an = block_sum_d(an, s_red);
+  float m = 0.f;
+  if (INV && !singular) {
+    for (int e = tid; e < N * nc; e += GC_THREADS) {
+      const int i = e / nc, c = e - i * nc;
+      const float4 v = a[i * lda + c];
+      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.z)));
+    }
+    m = block_max_f(m, s_redf);
+  }
+  if (C > 1) {
+    if (tid < C) {
+      double(*ld)[2] = cg::this_cluster().map_shared_rank(s_ld, tid);
+      ld[rank][0] = lg;
+      ld[rank][1] = an;
+      cg::this_cluster().map_shared_rank(s_max, tid)[rank] = m;
+    }
+    cg::this_cluster().sync();
+    lg = an = 0.0;
+    m = 0.f;
+    for (int r = 0; r < C; ++r) {
+      lg += s_ld[r][0];
+      an += s_ld[r][1];
+      m = fmaxf(m, s_max[r]);
+    }
+  }
+  if (rank == 0 && tid == 0) {
+    if (singular) {
+      logdet[b] = make_double2(-INFINITY, 0.0);
+      sing[b] = 1;
+      atomicAdd(&flags[0], 1);
+    } else {
+      const double ang = remainder(an + ((swaps & 1) ? M_PI : 0.0), 2.0 * M_PI);
+      logdet[b] = make_double2(lg, ang);
+      sing[b] = 0;
+    }
+  }
+  if (!INV) return;
+  __half* o = out + (size_t)b * 4 * N * Np;
+  const float sc = singular ? 1.f : mixed::pow2_scale((double)m);
+  if (rank == 0 && tid == 0) s_out[b] = sc;
+  // out row i, column r = S^-T[i][r] = S^-1[r][i] = a[r][iperm[i]]: local column c is row perm[c0 + c]
+  for (int e = tid; e < N * nc; e += GC_THREADS) {
+    const int c = e / N, r = e - c * N;
+    const float4 v = singular ? ffa::czero() : a[r * lda + c];
+    const int i = singular ? c0 + c : perm[c0 + c];
+    mixed::put4f(o + mixed::sp_at(i, Np, r), v.x * sc, v.z * sc);
+  }
+}
+
 template <class K>
 cudaError_t set_smem(K kernel, size_t bytes) {
   return ensure_dyn_smem(reinterpret_cast<const void*>(kernel), bytes);
 }
 
-size_t gj_smem_bytes(int N, bool in_smem) {
-  return (in_smem ? (size_t)N * N * sizeof(float4) : 0) + (size_t)N * (sizeof(float4) + sizeof(double2) + 2 * sizeof(int));
+size_t gj_smem_bytes(int N) { return (size_t)N * (sizeof(float4) + sizeof(double2) + 2 * sizeof(int)); }
+
+struct GjcArgs {
+  const float4* Sff;
+  int WS, N;
+  zc* logdet;
+  int *sing, *flags;
+  __half* out;
+  int Np;
+  float* s_out;
+};
+
+template <int C, bool INV, int THREADS, int LPR>
+cudaError_t gjc_launch(const GjcArgs& g, cudaStream_t st) {
+  const size_t bytes = gc_layout(g.N, C).bytes;
+  auto fn = gjc_ff_kernel<C, INV, THREADS, LPR>;
+  cudaError_t e = set_smem(fn, bytes);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)g.WS * C);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = C > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, g.Sff, g.N, g.logdet, g.sing, g.flags, g.out, g.Np, g.s_out);
+}
+
+// CTAs per matrix: the fewest whose shared memory holds it (0: none up to 8), doubled while every
+// matrix still gets its CTAs at once and a CTA keeps 32 columns.
+int gjc_cluster(int WS, int N) {
+  if (N > 256) return 0;
+  if (N <= 64) return 1;
+  int C = 1;
+  while (C <= 8 && gc_layout(N, C).bytes > GC_SMEM_LIMIT) C *= 2;
+  if (C > 8) return 0;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return C;
+  while (C < (N <= 128 ? 4 : 8) && (long)WS * 2 * C <= sms && N >= 64 * C) C *= 2;
+  return C;
+}
+
+// Small matrices take fewer threads, so that several share an SM (the panels are latency).
+// cudaErrorNotSupported: too large for this form.
+template <bool INV>
+cudaError_t gjc_invert(const GjcArgs& g, cudaStream_t st) {
+  const int N = g.N, C = gjc_cluster(g.WS, N);
+  if (C == 0) return cudaErrorNotSupported;
+  if (N <= 32) return gjc_launch<1, INV, 128, 4>(g, st);
+  if (N <= 64) return gjc_launch<1, INV, 256, 2>(g, st);
+  if (N <= 128) return C == 1   ? gjc_launch<1, INV, 512, 2>(g, st)
+                       : C == 2 ? gjc_launch<2, INV, 512, 2>(g, st)
+                                : gjc_launch<4, INV, 512, 2>(g, st);
+  return C <= 4 ? gjc_launch<4, INV, 512, 1>(g, st) : gjc_launch<8, INV, 512, 1>(g, st);
 }
 
 }  // namespace
@@ -558,38 +997,26 @@ cudaError_t overlap(const zc* A, const zc* phi, const zc* B, float4* Sff, float2
 
 cudaError_t invert(float4* Sff, int WS, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out,
                    cudaStream_t st) {
+  const GjcArgs g = {Sff, WS, N, logdet, sing, flags, out, Np, s_out};
+  const cudaError_t ec = out ? gjc_invert<true>(g, st) : gjc_invert<false>(g, st);
+  if (ec != cudaErrorNotSupported) return ec;
   cudaError_t e;
-  if (out && N <= GJB_MAXN) {
-    const size_t bytes = ((size_t)N * N + (size_t)GJB * N) * sizeof(float4) + gj_smem_bytes(N, false);
-    if (bytes <= SMEM_LIMIT) {
-      if ((e = set_smem(gjb_ff_kernel<true>, bytes)) != cudaSuccess) return e;
-      gjb_ff_kernel<true><<<WS, GJB_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
-      return cudaGetLastError();
-    }
-  }
   if (out && N <= GJB_GLOBAL_MAXN) {
-    const size_t bytes = (size_t)GJB * N * sizeof(float4) + gj_smem_bytes(N, false);
+    const size_t bytes = (size_t)GJB * N * sizeof(float4) + gj_smem_bytes(N);
     if (bytes <= SMEM_LIMIT) {
-      if ((e = set_smem(gjb_ff_kernel<false>, bytes)) != cudaSuccess) return e;
-      gjb_ff_kernel<false><<<WS, GJB_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
+      if ((e = set_smem(gjb_ff_kernel, bytes)) != cudaSuccess) return e;
+      gjb_ff_kernel<<<WS, GJB_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
       return cudaGetLastError();
     }
   }
-  const bool in_smem = N <= GJ_SMEM_MAXN && gj_smem_bytes(N, true) <= SMEM_LIMIT;
-  const size_t bytes = gj_smem_bytes(N, in_smem);
-#define GJ_LAUNCH(S, I)                                                                              \
-  do {                                                                                               \
-    if ((e = set_smem(gj_ff_kernel<S, I>, bytes)) != cudaSuccess) return e;                         \
-    gj_ff_kernel<S, I><<<WS, GJ_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out); \
-  } while (0)
+  const size_t bytes = gj_smem_bytes(N);
   if (out) {
-    if (in_smem) GJ_LAUNCH(true, true);
-    else GJ_LAUNCH(false, true);
+    if ((e = set_smem(gj_ff_kernel<true>, bytes)) != cudaSuccess) return e;
+    gj_ff_kernel<true><<<WS, GJ_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
   } else {
-    if (in_smem) GJ_LAUNCH(true, false);
-    else GJ_LAUNCH(false, false);
+    if ((e = set_smem(gj_ff_kernel<false>, bytes)) != cudaSuccess) return e;
+    gj_ff_kernel<false><<<WS, GJ_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
   }
-#undef GJ_LAUNCH
   return cudaGetLastError();
 }
 
