@@ -535,7 +535,8 @@ struct GcPanel {          // what the owner tells every CTA about one panel
 
 template <int C, bool INV, int GC_THREADS, int LPR>
 __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
-    gjc_ff_kernel(const float4* Sff, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out) {
+    gjc_ff_kernel(float4* Sff, int N, int keep, zc* logdet, int* sing, int* flags, __half* out, int Np,
+                  float* s_out) {
   namespace cg = cooperative_groups;
   constexpr int GC_WARPS = GC_THREADS / 32, SLOTS = GJB / LPR;   // a lane's entries: columns sub + LPR k
   extern __shared__ __align__(16) unsigned char gj_smem[];
@@ -901,6 +902,7 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     const float4 v = singular ? ffa::czero() : a[r * lda + c];
     const int i = singular ? c0 + c : perm[c0 + c];
     mixed::put4f(o + mixed::sp_at(i, Np, r), v.x * sc, v.z * sc);
+    if (keep) Sff[(size_t)b * N * N + (size_t)r * N + i] = v;   // every CTA read its columns before the first panel
   }
 }
 
@@ -912,8 +914,8 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 size_t gj_smem_bytes(int N) { return (size_t)N * (sizeof(float4) + sizeof(double2) + 2 * sizeof(int)); }
 
 struct GjcArgs {
-  const float4* Sff;
-  int WS, N;
+  float4* Sff;
+  int WS, N, keep;
   zc* logdet;
   int *sing, *flags;
   __half* out;
@@ -939,7 +941,7 @@ cudaError_t gjc_launch(const GjcArgs& g, cudaStream_t st) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = C > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, fn, g.Sff, g.N, g.logdet, g.sing, g.flags, g.out, g.Np, g.s_out);
+  return cudaLaunchKernelEx(&cfg, fn, g.Sff, g.N, g.keep, g.logdet, g.sing, g.flags, g.out, g.Np, g.s_out);
 }
 
 // CTAs per matrix: the fewest whose shared memory holds it (0: none up to 8), doubled while every
@@ -995,11 +997,14 @@ cudaError_t overlap(const zc* A, const zc* phi, const zc* B, float4* Sff, float2
   return cudaGetLastError();
 }
 
+bool keeps_inverse(int N) { return gjc_cluster(1, N) > 0; }
+
 cudaError_t invert(float4* Sff, int WS, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out,
-                   cudaStream_t st) {
-  const GjcArgs g = {Sff, WS, N, logdet, sing, flags, out, Np, s_out};
+                   cudaStream_t st, bool keep) {
+  const GjcArgs g = {Sff, WS, N, keep ? 1 : 0, logdet, sing, flags, out, Np, s_out};
   const cudaError_t ec = out ? gjc_invert<true>(g, st) : gjc_invert<false>(g, st);
   if (ec != cudaErrorNotSupported) return ec;
+  if (keep) return cudaErrorNotSupported;
   cudaError_t e;
   if (out && N <= GJB_GLOBAL_MAXN) {
     const size_t bytes = (size_t)GJB * N * sizeof(float4) + gj_smem_bytes(N);

@@ -14,7 +14,6 @@
 
 #include <utility>
 
-#include "ff.cuh"
 #include "handle.hpp"
 
 namespace fp64 {
@@ -110,94 +109,6 @@ __global__ void __launch_bounds__(256) zgemm_kernel(ZGemm g) {
   }
 }
 
-// The same GEMM in double-float arithmetic on the FP32 pipe (ff.cuh): FP64 operands are
-// split into hi + lo fp32 pairs as the tiles are staged, products and sums run through the
-// error-free transformations (about 48 significant bits), and the result is rounded back to
-// FP64.  Tile 64 x 64, 4 x 4 outputs per thread.
-constexpr int FBM = 64, FBN = 64, FBK = 8;
-
-__device__ __forceinline__ float4 ff_load(const zc* M, long ld, int r, int c, int op, int rows, int cols) {
-  // element (r, c) of op(M) as a double-float complex, zero outside rows x cols
-  if (r >= rows || c >= cols) return ffa::czero();
-  zc v = op == 0 ? M[(long)r * ld + c] : M[(long)c * ld + r];
-  if (op == 2) v = zconj(v);
-  return ffa::cfrom(v);
-}
-
-__global__ void __launch_bounds__(256) zgemm_ff_kernel(ZGemm g) {
-  __shared__ float4 As[FBK][FBM];
-  __shared__ float4 Bs[FBK][FBN];
-  const int t = threadIdx.x;
-  const int ty = t >> 4, tx = t & 15;
-  const int row0 = blockIdx.y * FBM, col0 = blockIdx.x * FBN;
-  const long nbatch = (long)g.nb[0] * g.nb[1] * g.nb[2];
-  for (long z = blockIdx.z; z < nbatch; z += gridDim.z) {
-    const int b2 = (int)(z % g.nb[2]);
-    const int b1 = (int)((z / g.nb[2]) % g.nb[1]);
-    const int b0 = (int)(z / ((long)g.nb[2] * g.nb[1]));
-    const zc* A = g.A + b0 * g.sA[0] + b1 * g.sA[1] + b2 * g.sA[2];
-    const zc* B = g.B + b0 * g.sB[0] + b1 * g.sB[1] + b2 * g.sB[2];
-    zc* C = g.C + b0 * g.sC[0] + b1 * g.sC[1] + b2 * g.sC[2];
-    ffa::cacc acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = ffa::cacc_from(ffa::czero());
-    for (int p0 = 0; p0 < g.k; p0 += FBK) {
-      __syncthreads();
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int e = t + u * 256;
-        // coalesced along the operand's contiguous index
-        int i, p;
-        if (g.opA == 0) { i = e >> 3; p = e & 7; } else { p = e >> 6; i = e & 63; }
-        As[p][i] = ff_load(A, g.lda, row0 + i, p0 + p, g.opA, g.m, g.k);
-        int j, q;
-        if (g.opB == 0) { q = e >> 6; j = e & 63; } else { j = e >> 3; q = e & 7; }
-        // op(B)[q][j]: stored element (q, j) for N, (j, q) for T / C
-        float4 bv = ffa::czero();
-        if (col0 + j < g.n && p0 + q < g.k) {
-          zc v = g.opB == 0 ? B[(long)(p0 + q) * g.ldb + col0 + j] : B[(long)(col0 + j) * g.ldb + p0 + q];
-          if (g.opB == 2) v = zconj(v);
-          bv = ffa::cfrom(v);
-        }
-        Bs[q][j] = bv;
-      }
-      __syncthreads();
-#pragma unroll 2
-      for (int p = 0; p < FBK; ++p) {
-        float4 a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[p][ty * 4 + i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[p][tx * 4 + j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) ffa::cacc_fma(acc[i][j], a[i], b[j]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int gi = row0 + ty * 4 + i, gj = col0 + tx * 4 + j;
-        if (gi < g.m && gj < g.n) {
-          const float4 v = ffa::cacc_get(acc[i][j]);
-          const zc s = zmake(ffa::to_double(ffa::re(v)), ffa::to_double(ffa::im(v)));
-          zc r = zmul(g.alpha, s);
-          zc* c = C + (long)gi * g.ldc + gj;
-          if (g.beta.x != 0.0 || g.beta.y != 0.0) r = zfma(g.beta, *c, r);
-          *c = r;
-          if (g.Acc) {
-            zc* a = g.Acc + b0 * g.sAcc[0] + b1 * g.sAcc[1] + b2 * g.sAcc[2] + (long)gi * g.ldacc + gj;
-            *a = zadd(*a, zmul(g.alpha, s));
-          }
-        }
-      }
-  }
-}
-
 static ZGemm gemm_init(int m, int n, int k, int opA, int opB) {
   ZGemm g;
   memset(&g, 0, sizeof(g));
@@ -212,14 +123,6 @@ static cudaError_t gemm_launch(afqmc_kp* h, const ZGemm& g, cudaStream_t st) {
   long nb = (long)g.nb[0] * g.nb[1] * g.nb[2];
   dim3 grid((g.n + GBN - 1) / GBN, (g.m + GBM - 1) / GBM, (unsigned)(nb < 65535 ? nb : 65535));
   zgemm_kernel<<<grid, 256, 0, st>>>(g);
-  AFQMC_LAUNCHED(h);
-  return cudaGetLastError();
-}
-
-static cudaError_t gemm_launch_ff(afqmc_kp* h, const ZGemm& g, cudaStream_t st) {
-  long nb = (long)g.nb[0] * g.nb[1] * g.nb[2];
-  dim3 grid((g.n + FBN - 1) / FBN, (g.m + FBM - 1) / FBM, (unsigned)(nb < 65535 ? nb : 65535));
-  zgemm_ff_kernel<<<grid, 256, 0, st>>>(g);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
 }
@@ -257,66 +160,78 @@ __global__ void v0_reduce_kernel(const zc* part, zc* v0, int nk, int M) {
 }
 
 // Ehalf[k] = exp(-dt/2 (h[k] + v0[k])) by scaling, 24-term Taylor series and squaring.
-// tmp: [k][3][M][M].  One block per k.
-__global__ void expm_kernel(const zc* h1, const zc* v0, zc* out, zc* tmp, int M, double dt) {
+// Three launches: X = -dt/2 (h + v0) scaled by 2^-sq to a norm of at most 1/4, the Taylor series by
+// groups of rows (row i of X^j / j! needs only itself and X, so the rows spread over the GPU: one
+// block per k ran 24 dependent M^3 products at one SM's FP64 rate, 517 us at M = 26, 27 k-points),
+// and sq squarings (none at the time steps in use).  tmp: [k][3][M][M] = X, (sq in its first element), scratch.
+__global__ void expm_scale_kernel(const zc* h1, const zc* v0, zc* tmp, int M, double dt) {
   const int k = blockIdx.x;
   const long MM = (long)M * M;
   zc* Xm = tmp + (long)k * 3 * MM;
-  zc* Tm = Xm + MM;
-  zc* Rm = Tm + MM;
-  zc* E = out + k * MM;
   __shared__ double red[32];
   __shared__ int s_sq;
-  // X = -dt/2 (h + v0); 1-norm bound for scaling
   double rowmax = 0.0;
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
     double s = 0.0;
     for (int j = 0; j < M; ++j) {
       zc v = zscale(zadd(h1[k * MM + i * M + j], v0[k * MM + i * M + j]), -0.5 * dt);
-      Xm[i * M + j] = v;
       s += sqrt(zabs2(v));
     }
     rowmax = fmax(rowmax, s);
   }
-  // block max via sum of squares is not a max; do a simple max reduction
-  {
-    double v = rowmax;
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double m = 0.0;
-      for (int i = 0; i < (int)((blockDim.x + 31) >> 5); ++i) m = fmax(m, red[i]);
-      int sq = 0;
-      while (m > 0.25 && sq < 60) { m *= 0.5; ++sq; }
-      s_sq = sq;
-    }
-    __syncthreads();
+  double v = rowmax;
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double m = 0.0;
+    for (int i = 0; i < (int)((blockDim.x + 31) >> 5); ++i) m = fmax(m, red[i]);
+    int sq = 0;
+    while (m > 0.25 && sq < 60) { m *= 0.5; ++sq; }
+    s_sq = sq;
+    tmp[((long)k * 3 + 1) * MM] = zmake((double)sq, 0.0);
   }
-  const int sq = s_sq;
-  const double scl = ldexp(1.0, -sq);
-  for (long e = threadIdx.x; e < MM; e += blockDim.x) {
-    Xm[e] = zscale(Xm[e], scl);
-    const int i = (int)(e / M), j = (int)(e % M);
-    E[e] = zmake(i == j ? 1.0 : 0.0, 0.0);
-    Tm[e] = E[e];
+  __syncthreads();
+  const double scl = ldexp(1.0, -s_sq);
+  for (long e = threadIdx.x; e < MM; e += blockDim.x)
+    Xm[e] = zscale(zscale(zadd(h1[k * MM + e], v0[k * MM + e]), -0.5 * dt), scl);
+}
+constexpr int EXPM_ROWS = 4;
+// out rows of sum_{j<=24} X^j / j! ; grid (k, groups of EXPM_ROWS rows), dynamic shared memory
+// 2 EXPM_ROWS M elements
+__global__ void expm_rows_kernel(const zc* tmp, zc* out, int M) {
+  const int k = blockIdx.x, i0 = blockIdx.y * EXPM_ROWS, rows = min(EXPM_ROWS, M - i0);
+  const long MM = (long)M * M;
+  const zc* Xm = tmp + (long)k * 3 * MM;
+  zc* E = out + k * MM + (long)i0 * M;
+  extern __shared__ zc er[];   // [EXPM_ROWS][M] the term's rows, [EXPM_ROWS][M] the next term's
+  zc* Tm = er;
+  zc* Rm = er + EXPM_ROWS * M;
+  for (int e = threadIdx.x; e < rows * M; e += blockDim.x) {
+    Tm[e] = zmake(i0 + e / M == e % M ? 1.0 : 0.0, 0.0);
+    E[e] = Tm[e];
   }
   __syncthreads();
   for (int term = 1; term <= 24; ++term) {
-    // Rm = Tm * Xm / term
-    for (long e = threadIdx.x; e < MM; e += blockDim.x) {
-      const int i = (int)(e / M), j = (int)(e % M);
+    for (int e = threadIdx.x; e < rows * M; e += blockDim.x) {
+      const int i = e / M, j = e % M;
       zc s = zzero();
-      for (int l = 0; l < M; ++l) s = zfma(Tm[i * M + l], Xm[l * M + j], s);
+      for (int l = 0; l < M; ++l) s = zfma(Tm[i * M + l], Xm[(long)l * M + j], s);
       Rm[e] = zscale(s, 1.0 / term);
-    }
-    __syncthreads();
-    for (long e = threadIdx.x; e < MM; e += blockDim.x) {
-      Tm[e] = Rm[e];
       E[e] = zadd(E[e], Rm[e]);
     }
     __syncthreads();
+    zc* t = Tm;
+    Tm = Rm;
+    Rm = t;
   }
+}
+__global__ void expm_square_kernel(zc* out, zc* tmp, int M) {
+  const int k = blockIdx.x;
+  const long MM = (long)M * M;
+  zc* E = out + k * MM;
+  zc* Rm = tmp + ((long)k * 3 + 2) * MM;
+  const int sq = (int)tmp[((long)k * 3 + 1) * MM].x;
   for (int s = 0; s < sq; ++s) {
     for (long e = threadIdx.x; e < MM; e += blockDim.x) {
       const int i = (int)(e / M), j = (int)(e % M);
@@ -375,7 +290,12 @@ cudaError_t set_one_body(afqmc_kp* h, cudaStream_t st) {
   g.nb[0] = nk;
   cudaError_t e = gemm_launch(h, g, st);
   if (e != cudaSuccess) return e;
-  expm_kernel<<<nk, 256, 0, st>>>(h->h1, h->v0, h->Ehalf, h->expm_tmp, M, h->dt);
+  expm_scale_kernel<<<nk, 256, 0, st>>>(h->h1, h->v0, h->expm_tmp, M, h->dt);
+  AFQMC_LAUNCHED(h);
+  expm_rows_kernel<<<dim3(nk, (M + EXPM_ROWS - 1) / EXPM_ROWS), 128, sizeof(zc) * 2 * EXPM_ROWS * M, st>>>(
+      h->expm_tmp, h->Ehalf, M);
+  AFQMC_LAUNCHED(h);
+  expm_square_kernel<<<nk, 256, 0, st>>>(h->Ehalf, h->expm_tmp, M);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
 }
@@ -523,7 +443,7 @@ __global__ void __launch_bounds__(256) lu_kernel(zc* S, zc* Sinv, zc* logdet, in
 }
 
 // Gh[w][s] = (phi S^-1)^T = S^-T phi^T  (N x NM)
-static cudaError_t green_impl(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st, bool ff = false) {
+static cudaError_t green_impl(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st) {
   cudaError_t e = overlap(h, phi, st);
   if (e != cudaSuccess) return e;
   // pivot scratch lives in the P buffer (used otherwise only by the backward pass)
@@ -536,19 +456,12 @@ static cudaError_t green_impl(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cud
   g.B = phi; g.ldb = N; g.sB[0] = (long)NM * N;
   g.C = h->Gh; g.ldc = NM; g.sC[0] = (long)N * NM;
   g.nb[0] = 2 * h->W;
-  return ff ? gemm_launch_ff(h, g, st) : gemm_launch(h, g, st);
+  return gemm_launch(h, g, st);
 }
 
 cudaError_t green(afqmc_kp* h, const zc* phi, cudaStream_t st) {
   prof_begin(h, AFQMC_STAGE_GREEN, st);
   cudaError_t e = green_impl(h, phi, h->ld_old, h->sing_old, st);
-  prof_end(h, st);
-  return e;
-}
-
-cudaError_t green_ff(afqmc_kp* h, const zc* phi, cudaStream_t st) {
-  prof_begin(h, AFQMC_STAGE_GREEN, st);
-  cudaError_t e = green_impl(h, phi, h->ld_old, h->sing_old, st, true);
   prof_end(h, st);
   return e;
 }
@@ -1195,9 +1108,9 @@ cudaError_t grad_h1(afqmc_kp* h, const zc* grad_e, zc* gh1, cudaStream_t st) {
 // dE/dphi from Gam = conj(grad_e)-weighted dE/dGh: with Gh = S^-T phi^T and S = A^dag phi,
 // dGh = S^-T dphi^T (I - A* Gh), so grad_phi = [S^-1 (Gam - (Gam Gh^T) A^dag)]^H in the
 // conjugate convention of the binding.
-cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st, bool ff) {
+cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st) {
   cudaError_t e;
-  auto launch = [&](const ZGemm& g) { return ff ? gemm_launch_ff(h, g, st) : gemm_launch(h, g, st); };
+  auto launch = [&](const ZGemm& g) { return gemm_launch(h, g, st); };
   const int nk = h->nk, M = h->M, n = h->n, N = h->N, NM = h->NM, W = h->W;
   {  // P = Gam Gh^T  (N x N)
     ZGemm g = gemm_init(N, N, NM, 0, 1);
@@ -1242,7 +1155,7 @@ static cudaError_t backward_impl(afqmc_kp* h, const zc* grad_e, zc* grad_phi, zc
       h->LH, h->Gh, grad_e, h->Gam, h->kminus, h->minus, nk, h->G, M, n);
   AFQMC_LAUNCHED(h);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return project_gamma(h, grad_phi, st, false);
+  return project_gamma(h, grad_phi, st);
 }
 
 cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, zc* grad_phi, zc* grad_h1,

@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "mixed.hpp"
+#include "adjoint.hpp"
 #include "attr.hpp"
 #include "ffla.hpp"
 #include "split.cuh"
@@ -1352,59 +1353,6 @@ __global__ void z_partner_kernel(__half* z_sp, float* s_z, const int* pmap, int 
   }
 }
 
-// Gam[ws][(k1,a)][(k2,r)] of the adjoint, k2 = k1 - Q, in FP64 from
-//   c2 sum_g X[w][-Q][g] LH[Q][k1][g][a][r]   (Coulomb; fp32 sum over g)
-// + c1 AhH[k1][a][r] on the diagonal blocks  (one-body)
-// - c3 gam32[k1][k2][ws][(a,r)]              (exchange, from the adjoint GEMM)
-// with c = conj(grad_e) per walker.  Block (k1, Q, group of GA_W walkers).
-constexpr int GA_W = 16;
-__global__ void __launch_bounds__(128) gamma_assemble_kernel(const zc* LH, const zc* X, const zc* AhH,
-                                                             const zc* grad_e, const float2* gam32, zc* Gam,
-                                                             const int* kminus, const int* minus, int nk, int G,
-                                                             int M, int n, int Mp, int W) {
-  const int k1 = blockIdx.x, Q = blockIdx.y, w0 = blockIdx.z * GA_W;
-  const int k2 = kminus[k1 * nk + Q], mQ = minus[Q];
-  const int nw = min(GA_W, W - w0);
-  const int nM = n * M, N = nk * n, NM = nk * M, WS = 2 * W, nMp = n * Mp;
-  extern __shared__ float2 xs[];   // [GA_W][G]
-  for (int e = threadIdx.x; e < GA_W * G; e += blockDim.x) {
-    const int wi = e / G, g = e % G;
-    const zc v = wi < nw ? X[((size_t)(w0 + wi) * nk + mQ) * G + g] : zzero();
-    xs[e] = make_float2((float)v.x, (float)v.y);
-  }
-  __syncthreads();
-  const zc* lh = LH + ((size_t)Q * nk + k1) * G * nM;
-  for (int e = threadIdx.x; e < nM; e += blockDim.x) {
-    float2 acc[GA_W];
-#pragma unroll
-    for (int i = 0; i < GA_W; ++i) acc[i] = make_float2(0.f, 0.f);
-    for (int g = 0; g < G; ++g) {
-      const zc l = lh[(size_t)g * nM + e];
-      const float lr = (float)l.x, li = (float)l.y;
-#pragma unroll
-      for (int i = 0; i < GA_W; ++i) {
-        const float2 x = xs[i * G + g];
-        acc[i].x = fmaf(x.x, lr, fmaf(-x.y, li, acc[i].x));
-        acc[i].y = fmaf(x.x, li, fmaf(x.y, lr, acc[i].y));
-      }
-    }
-    const int a = e / M, r = e % M;
-#pragma unroll
-    for (int i = 0; i < GA_W; ++i) {
-      if (i >= nw) break;
-      const int w = w0 + i;
-      const zc c1 = zconj(grad_e[3 * w + 0]), c2 = zconj(grad_e[3 * w + 1]), c3 = zconj(grad_e[3 * w + 2]);
-      zc base = zmul(c2, zmake((double)acc[i].x, (double)acc[i].y));
-      if (Q == 0) base = zfma(c1, AhH[(size_t)k1 * nM + e], base);
-      for (int sp = 0; sp < 2; ++sp) {
-        const int ws = 2 * w + sp;
-        const float2 gx = gam32[(((size_t)k1 * nk + k2) * WS + ws) * nMp + a * Mp + r];
-        Gam[((size_t)ws * N + k1 * n + a) * NM + k2 * M + r] = zsub(base, zmul(c3, zmake(gx.x, gx.y)));
-      }
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // host orchestration
 // ---------------------------------------------------------------------------
@@ -1782,7 +1730,7 @@ static cudaError_t create_impl(afqmc_kp* h, cudaStream_t st) {
   MTRY(map_split(&m->m_phi_a, m->phi_sp, Np, NM, WS, 128));
   MTRY(map_split(&m->m_sinvt_b, m->sinvt_sp, Np, N, WS, BN));
   MTRY(map_split(&m->m_t0_b, m->t_sp[0], NMp, (size_t)2 * N, W, BN));
-  MTRY(set_smem_attr((const void*)gamma_assemble_kernel, sizeof(float2) * GA_W * G));
+  MTRY(adjoint::gamma_smem(G));
   MTRY(set_smem_attr((const void*)onebody_in_kernel, onebody_smem(h)));
   if (onebody_out_staged(h))
     MTRY(set_smem_attr((const void*)onebody_out_kernel<true>, onebody_out_smem(h)));
@@ -1853,7 +1801,8 @@ static cudaError_t overlap_logdet(afqmc_kp* h, const zc* phi, zc* ld, int* sing,
 
 // The Green's function in three parts: the double-float overlap, inverse and log det and
 // the split of phi_perp (green_pre); the tensor-core GEMM; its max and split (green_post).
-static cudaError_t green_pre(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st) {
+// keep: S^-1 stays in s_ff in double-float (ffla::keeps_inverse).
+static cudaError_t green_pre(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st, bool keep = false) {
   MixedState* m = h->mixed;
   const int WS = m->WS;
   unsigned long long* mx_phi = m->mx;
@@ -1866,7 +1815,7 @@ static cudaError_t green_pre(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cuda
   MTRY(cudaMemsetAsync(m->mx, 0, sizeof(unsigned long long) * (2 * WS + 3 * h->W), st));
   MTRY(ffla::overlap(h->A, phi, m->bproj, m->s_ff, phi_perp, mx_phi, WS, h->nk, h->M, h->n, h->N, st));
   AFQMC_LAUNCHED(h);
-  MTRY(ffla::invert(m->s_ff, WS, h->N, ld, sing, h->flags, m->sinvt_sp, m->Np, m->s_sinv, st));
+  MTRY(ffla::invert(m->s_ff, WS, h->N, ld, sing, h->flags, m->sinvt_sp, m->Np, m->s_sinv, st, keep));
   AFQMC_LAUNCHED(h);
   split_rows32_kernel<<<dim3(WS, SPLIT_CHUNKS), 256, 0, st>>>(phi_perp, h->NM, h->N, m->Np, mx_phi, m->s_phi,
                                                                m->phi_sp);
@@ -1883,9 +1832,9 @@ static cudaError_t green_post(afqmc_kp* h, cudaStream_t st) {
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
 }
-static cudaError_t green(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st) {
+static cudaError_t green(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st, bool keep = false) {
   MixedState* m = h->mixed;
-  MTRY(green_pre(h, phi, ld, sing, st));
+  MTRY(green_pre(h, phi, ld, sing, st, keep));
   MTRY(run_gemm(h, m->m_sinvt, m->m_phi, green_params(h), h->flags + 1, st));
   AFQMC_LAUNCHED(h);
   return green_post(h, st);
@@ -2285,27 +2234,41 @@ static cudaError_t adjoint_exchange(afqmc_kp* h, cudaStream_t st) {
 
 // The adjoint: Gam = conj(grad_e)-weighted dE/dGh with the exchange part from the
 // tensor-core GEMM over the full precontracted tensor and the Coulomb and one-body parts in
-// fp32, then the projection onto dE/dphi through S^-1 and the Green's function (FP64 LU,
-// double-float products) and dE/dh.
+// fp32, then the projection onto dE/dphi through S^-1 and the walker, and dE/dh, in double-float
+// (adjoint.cu).  S^-1 is the Green's function's own, kept in double-float; matrices too large for
+// that form go through the FP64 LU.
 cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, zc* grad_phi, zc* grad_h1,
                                   cudaStream_t st) {
   MixedState* m = h->mixed;
+  const bool keep = ffla::keeps_inverse(h->N);
+  float4* Gam = reinterpret_cast<float4*>(h->Gam);
   if (grad_phi) {
-    MSTAGE(AFQMC_STAGE_GREEN, green(h, phi, h->ld_old, h->sing_old, st));
+    MSTAGE(AFQMC_STAGE_GREEN, green(h, phi, h->ld_old, h->sing_old, st, keep));
     MSTAGE(AFQMC_STAGE_FORCE_BIAS, cholesky_trace(h, st));
     MSTAGE(AFQMC_STAGE_ADJOINT_GEMM, adjoint_exchange(h, st));
-    prof_begin(h, AFQMC_STAGE_BACKWARD, st);
-    gamma_assemble_kernel<<<dim3(h->nk, h->nk, cdiv(h->W, GA_W)), 128, sizeof(float2) * GA_W * h->G, st>>>(
-        h->LH, h->X, h->AhH, grad_e, m->gam32, h->Gam, h->kminus, h->minus, h->nk, h->G, h->M, h->n, m->Mp, h->W);
     AFQMC_LAUNCHED(h);
-    prof_end(h, st);
-    MTRY(cudaGetLastError());
+    MSTAGE(AFQMC_STAGE_BACKWARD, adjoint::gamma(h->LH, h->X, h->AhH, grad_e, m->gam32, Gam, h->kminus, h->minus,
+                                                h->nk, h->G, h->M, h->n, m->Mp, h->W, st));
+    AFQMC_LAUNCHED(h);
+  } else if (keep) {
+    MSTAGE(AFQMC_STAGE_GREEN, green_pre(h, phi, h->ld_old, h->sing_old, st, true));
   }
-  // Green's function and inverse of the same walkers for the projection: FP64 overlap and
-  // LU, the large products in double-float
-  MTRY(fp64::green_ff(h, phi, st));
-  if (grad_h1) MSTAGE(AFQMC_STAGE_BACKWARD, fp64::grad_h1(h, grad_e, grad_h1, st));
-  if (grad_phi) MSTAGE(AFQMC_STAGE_BACKWARD, fp64::project_gamma(h, grad_phi, st, true));
+  if (!keep) {
+    MSTAGE(AFQMC_STAGE_GREEN, fp64::overlap_lu(h, phi, h->ld_old, h->sing_old, 1, st));
+    MTRY(adjoint::to_ff(h->Sinv, m->s_ff, (size_t)m->WS * h->N * h->N, st));
+    AFQMC_LAUNCHED(h);
+  }
+  if (grad_h1) {
+    MSTAGE(AFQMC_STAGE_BACKWARD, adjoint::grad_h1(phi, m->s_ff, h->A, grad_e, h->Gh, h->P,
+                                                  (size_t)m->WS * h->N * h->N, grad_h1, h->W, h->nk, h->M, h->n, st));
+    h->launches += 3;
+  }
+  if (grad_phi) {
+    MSTAGE(AFQMC_STAGE_BACKWARD,
+           adjoint::project(phi, Gam, m->s_ff, h->A, reinterpret_cast<float4*>(h->P), reinterpret_cast<float4*>(h->S),
+                            keep ? h->sing_old : nullptr, h->flags, grad_phi, m->WS, h->nk, h->M, h->n, st));
+    h->launches += 4;
+  }
   return cudaSuccess;
 }
 
