@@ -38,6 +38,25 @@ __device__ __forceinline__ zc zinv(zc b) {
   return zmake(b.x / d, -b.y / d);
 }
 
+// Conversions between FP64 and FP32 on the integer pipe.  The FP64 pipe (conversions included)
+// issues two operations per clock and SM here, so an elementwise kernel that converts every value of a
+// walker spends longer on that than on its memory traffic (31 us per conversion of each real of the
+// 3x3x3 walkers, against about 10 us this way).  Values outside the common exponents take the instruction.
+__device__ __forceinline__ float d2f(double x) {   // round to nearest even, as __double2float_rn
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) return (hi & 0x7fffffffu) | lo ? __double2float_rn(x) : __uint_as_float(hi);   // zero stays here
+  unsigned r = __funnelshift_l(lo, (hi & 0x7fffffffu) - (896u << 20), 3);
+  const unsigned rem = lo << 3;
+  r += (rem > 0x80000000u || (rem == 0x80000000u && (r & 1u))) ? 1u : 0u;
+  return __uint_as_float(r | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double f2d(float x) {   // exact
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u) return m ? (double)x : __hiloint2double((int)b, 0);   // subnormal, infinite, NaN; zero
+  return __hiloint2double((int)(((m >> 3) + (896u << 20)) | (b & 0x80000000u)), (int)(b << 29));
+}
+
 // Warp / block reductions -------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -57,9 +76,13 @@ __device__ __forceinline__ zc block_zsum(zc v, zc* red) {
   __syncthreads();
   if (lane == 0) red[wid] = v;
   __syncthreads();
-  zc t = zzero();
-  for (int i = 0; i < nw; ++i) t = zadd(t, red[i]);
-  return t;
+  if (threadIdx.x == 0) {   // one thread: the FP64 pipe would spend longer on the same sum in all of them
+    zc t = zzero();
+    for (int i = 0; i < nw; ++i) t = zadd(t, red[i]);
+    red[0] = t;
+  }
+  __syncthreads();
+  return red[0];
 }
 __device__ __forceinline__ double block_dsum(double v, double* red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -67,9 +90,13 @@ __device__ __forceinline__ double block_dsum(double v, double* red) {
   __syncthreads();
   if (lane == 0) red[wid] = v;
   __syncthreads();
-  double t = 0.0;
-  for (int i = 0; i < nw; ++i) t += red[i];
-  return t;
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int i = 0; i < nw; ++i) t += red[i];
+    red[0] = t;
+  }
+  __syncthreads();
+  return red[0];
 }
 
 // Index helpers of the momentum grid --------------------------------------

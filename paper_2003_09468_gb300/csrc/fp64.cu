@@ -602,23 +602,23 @@ __global__ void weight_kernel(const double* x, const zc* xbar, const zc* ld_old,
                               const int* sing_old, const int* sing_new, double* weight, zc* logdet_out,
                               int nf) {
   const int w = blockIdx.x;
-  __shared__ zc red[32];
-  zc s = zzero();
+  __shared__ double red[32];
+  double s = 0.0;
+  // Re(x xbar - xbar^2 / 2) = xr (x - xr / 2) + xi^2 / 2: the weight needs no imaginary part, and the
+  // FP64 pipe's two operations per clock are what this kernel waits for
   for (int f = threadIdx.x; f < nf; f += blockDim.x) {
-    const double xf = x[(long)w * nf + f];
     const zc xb = xbar[(long)w * nf + f];
-    // x xbar - xbar^2 / 2
-    const zc xb2 = zmul(xb, xb);
-    s = zadd(s, zmake(xf * xb.x - 0.5 * xb2.x, xf * xb.y - 0.5 * xb2.y));
+    s = fma(xb.x, fma(-0.5, xb.x, x[(long)w * nf + f]), s);
+    s = fma(0.5 * xb.y, xb.y, s);
   }
-  s = block_zsum(s, red);
+  s = block_dsum(s, red);
   if (threadIdx.x == 0) {
     const bool dead = sing_old[2 * w] || sing_old[2 * w + 1] || sing_new[2 * w] || sing_new[2 * w + 1];
     double wn = 0.0;
     if (!dead) {
       const zc dlog = zadd(zsub(ld_new[2 * w], ld_old[2 * w]), zsub(ld_new[2 * w + 1], ld_old[2 * w + 1]));
       const double c = cos(dlog.y);
-      wn = weight[w] * exp(dlog.x + s.x) * (c > 0.0 ? c : 0.0);
+      wn = weight[w] * exp(dlog.x + s) * (c > 0.0 ? c : 0.0);
     }
     weight[w] = wn;
     if (logdet_out) {
@@ -803,7 +803,7 @@ static cudaError_t taylor(afqmc_kp* h, zc* phi, cudaStream_t st) {
 cudaError_t weights(afqmc_kp* h, const zc* phi, const double* x, double* w, zc* logdet, cudaStream_t st) {
   cudaError_t e;
   if ((e = logdet_only(h, phi, h->ld_new, h->sing_new, st)) != cudaSuccess) return e;
-  weight_kernel<<<h->W, 256, 0, st>>>(x, h->xbar, h->ld_old, h->ld_new, h->sing_old, h->sing_new, w, logdet,
+  weight_kernel<<<h->W, 512, 0, st>>>(x, h->xbar, h->ld_old, h->ld_new, h->sing_old, h->sing_new, w, logdet,
                                       2 * h->nk * h->G);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
@@ -811,7 +811,7 @@ cudaError_t weights(afqmc_kp* h, const zc* phi, const double* x, double* w, zc* 
 
 // Hybrid weight from the log dets already in ld_old / ld_new.
 cudaError_t weight_only(afqmc_kp* h, const double* x, double* w, zc* logdet, cudaStream_t st) {
-  weight_kernel<<<h->W, 256, 0, st>>>(x, h->xbar, h->ld_old, h->ld_new, h->sing_old, h->sing_new, w, logdet,
+  weight_kernel<<<h->W, 512, 0, st>>>(x, h->xbar, h->ld_old, h->ld_new, h->sing_old, h->sing_new, w, logdet,
                                       2 * h->nk * h->G);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();

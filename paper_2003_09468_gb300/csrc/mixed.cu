@@ -106,7 +106,7 @@ constexpr int ZCTAS = 304;
 // FP64 input of moderate range: rounded once to fp32 (24 bits, of which the split keeps
 // 22), then scaled (per-step operands: walkers, inverses, Green's functions)
 __device__ __forceinline__ void put4(__half* o, double re, double im, float s) {
-  put4f(o, (float)re * s, (float)im * s);
+  put4f(o, d2f(re) * s, d2f(im) * s);
 }
 // FP64 input of any range: scaled in FP64 first (set-up data only)
 __device__ __forceinline__ void put4d(__half* o, double re, double im, float s) {
@@ -561,7 +561,7 @@ struct ExchangeP {
       }
       if (cl == 0 && ws < WS) {
         const float f = inv_z * rcp2(inv[it]);   // powers of two: exact after the sum
-        xpart[((size_t)t * nt_n + nt) * WS + ws] = make_double2((double)(pr * f), (double)(pi * f));
+        xpart[((size_t)t * nt_n + nt) * WS + ws] = make_double2(f2d(pr * f), f2d(pi * f));
       }
     }
   }
@@ -839,22 +839,35 @@ __global__ void split_green_kernel(const float2* g32, const unsigned long long* 
   }
 }
 
-// y [W][Nk][G] (zc, carries sqrt(dt)) -> y_sp [Nk][W][Gp] of y / s_l[Q][g], scale s_y[Q][W]
+// y [W][Nk][G] (zc, carries sqrt(dt)) -> y_sp [Nk][W][Gp] of y / s_l[Q][g], scale s_y[Q][W].  The
+// divisors are powers of two, so the quotients' maximum comes from exponent arithmetic on the bits.
 __global__ void split_y_kernel(const zc* y, const float* s_l, __half* out, float* s_y, int nk, int W, int G, int Gp) {
   const int Q = blockIdx.x, w = blockIdx.y;
-  __shared__ double red[32];
+  __shared__ unsigned long long red[32];
   const zc* yp = y + ((size_t)w * nk + Q) * G;
-  double m = 0.0;
+  unsigned long long m = 0;
   for (int g = threadIdx.x; g < G; g += blockDim.x) {
-    const double f = 1.0 / (double)s_l[Q * G + g];
-    m = fmax(m, cabs_d(yp[g]) * f);
+    const unsigned long long re = (unsigned long long)__double_as_longlong(yp[g].x) & 0x7fffffffffffffffull;
+    const unsigned long long im = (unsigned long long)__double_as_longlong(yp[g].y) & 0x7fffffffffffffffull;
+    const unsigned long long v = max(re, im);
+    const long long sh = (long long)((__float_as_uint(s_l[Q * G + g]) >> 23) - 127u) << 52;   // log2 s_l
+    // normal quotients by exponent; anything else by the division
+    const int eb = (int)(v >> 52), eq = eb - (int)(sh >> 52);
+    const unsigned long long q =
+        (eb > 0 && eb < 0x7ff && eq > 0 && eq < 0x7ff)
+            ? v - (unsigned long long)sh
+            : (unsigned long long)__double_as_longlong(__longlong_as_double((long long)v) / (double)s_l[Q * G + g]);
+    m = max(m, v ? q : 0ull);
   }
-  m = block_max(m, red);
-  const float s = pow2_scale(m);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = max(m, red[i]);
+  const float s = pow2_scale(__longlong_as_double((long long)m));
   if (threadIdx.x == 0) s_y[Q * W + w] = s;
   for (int g = threadIdx.x; g < G; g += blockDim.x) {
-    const double f = 1.0 / (double)s_l[Q * G + g];
-    put4(out + sp_at((size_t)Q * W + w, Gp, g), yp[g].x * f, yp[g].y * f, s);
+    const float f = rcp2(s_l[Q * G + g]);
+    put4f(out + sp_at((size_t)Q * W + w, Gp, g), d2f(yp[g].x) * (f * s), d2f(yp[g].y) * (f * s));
   }
 }
 
@@ -886,7 +899,7 @@ __device__ __forceinline__ void onebody_apply4(const float2* Dt, const float2* b
 // grid (k, ws, j-chunk of 64)
 __global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float4* corr, float2* p32,
                                   unsigned long long* mx, int nk, int M, int N, int NM) {
-  __shared__ double red[32];
+  __shared__ float red[32];
   const int k = blockIdx.x, ws = blockIdx.y, j0 = blockIdx.z * 64;
   const int w = ws >> 1, sp = ws & 1;
   const int jn = min(64, N - j0);
@@ -903,12 +916,12 @@ __global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float4* co
     float2 v = make_float2(0.f, 0.f);
     if (j < jn) {
       const zc x = src[(size_t)(k * M + q) * N + j0 + j];
-      v = make_float2((float)x.x, (float)x.y);
+      v = make_float2(d2f(x.x), d2f(x.y));
     }
     blk[q * OB_LD + j] = v;
   }
   __syncthreads();
-  double m = 0.0;
+  float m = 0.f;
   for (int e = threadIdx.x; e < M * 16; e += blockDim.x) {
     const int p = e % M, jq = e / M;
     float2 c[4];
@@ -922,11 +935,11 @@ __global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float4* co
       const float2 b = blk[p * OB_LD + j];
       const float2 v = make_float2(b.x + c[u].x, b.y + c[u].y);
       p32[o] = v;
-      m = fmax(m, (double)fmaxf(fabsf(v.x), fabsf(v.y)));
+      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
     }
   }
-  m = block_max(m, red);
-  if (threadIdx.x == 0) atomic_max_pos(mx + w, m);
+  m = block_max_f(m, red);
+  if (threadIdx.x == 0) atomic_max_pos(mx + w, (double)m);
 }
 
 // Second half step: with corr.xy = d = phi'' - phi and corr.zw = phi'' (fp32) after the
@@ -961,6 +974,11 @@ __global__ void onebody_out_kernel(const float4* corr, const float2* dhalf, zc* 
   zc* dst = phi + (size_t)ws * NM * N;
   for (int e = threadIdx.x; e < M * 16; e += blockDim.x) {
     const int jq = STAGE_D ? e % 16 : e / M, p = STAGE_D ? e / 16 : e % M;
+    zc* row = dst + (size_t)(k * M + p) * N + j0;
+    zc v[4];   // the walker's entries are on their way while the products are formed
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (jq + 16 * u < jn) v[u] = row[jq + 16 * u];
     float2 c[4];
     onebody_apply4(Dt, blk, M, p, jq, c);
 #pragma unroll
@@ -968,10 +986,9 @@ __global__ void onebody_out_kernel(const float4* corr, const float2* dhalf, zc* 
       const int j = jq + 16 * u;
       if (j >= jn) continue;
       const float2 d = STAGE_D ? dd[p * OB_LD + j] : reinterpret_cast<const float2*>(src)[2 * ((size_t)j * NM + p)];
-      zc v = dst[(size_t)(k * M + p) * N + j0 + j];
-      v.x += (double)(d.x + c[u].x);
-      v.y += (double)(d.y + c[u].y);
-      dst[(size_t)(k * M + p) * N + j0 + j] = v;
+      v[u].x += f2d(d.x + c[u].x);
+      v[u].y += f2d(d.y + c[u].y);
+      row[j] = v[u];
     }
   }
 }
@@ -1196,7 +1213,8 @@ __global__ void dhalf_kernel(const zc* Ehalf, float2* d, int nk, int M) {
   }
 }
 
-// E1 and EC per walker from the fp32 Green's function and the FP64 X.
+// E1 and EC per walker from the fp32 Green's function and the FP64 X.  One block per walker, 1024
+// threads: FP64 work of two operations per clock, so the loads of many elements have to overlap.
 __global__ void e1_ec_mixed_kernel(const zc* AhH, const float2* g32, const zc* X, const int* minus, zc* eloc, int nk,
                                    int M, int n, int Mp, int G, int WS) {
   const int w = blockIdx.x;
@@ -1205,7 +1223,7 @@ __global__ void e1_ec_mixed_kernel(const zc* AhH, const float2* g32, const zc* X
   for (int e = threadIdx.x; e < 2 * nk * n * M; e += blockDim.x) {
     const int q = e % M, a = (e / M) % n, k = (e / (M * n)) % nk, sp = e / (M * n * nk);
     const float2 g = g32[((((size_t)k * nk + k) * WS + 2 * w + sp) * n + a) * Mp + q];
-    s = zfma(AhH[((size_t)k * n + a) * M + q], zmake(g.x, g.y), s);
+    s = zfma(AhH[((size_t)k * n + a) * M + q], zmake(f2d(g.x), f2d(g.y)), s);
   }
   const zc e1 = block_zsum(s, red);
   zc c = zzero();
@@ -2033,7 +2051,7 @@ cudaError_t orthonormalise(afqmc_kp* h, zc* phi, zc* logdet, cudaStream_t st) {
 
 static cudaError_t e1_ec(afqmc_kp* h, zc* eloc, cudaStream_t st) {
   MixedState* m = h->mixed;
-  e1_ec_mixed_kernel<<<h->W, 256, 0, st>>>(h->AhH, m->g32, h->X, h->minus, eloc, h->nk, h->M, h->n, m->Mp, h->G,
+  e1_ec_mixed_kernel<<<h->W, 1024, 0, st>>>(h->AhH, m->g32, h->X, h->minus, eloc, h->nk, h->M, h->n, m->Mp, h->G,
                                             m->WS);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();

@@ -7,19 +7,22 @@
 
 #include <cuda_fp16.h>
 
-#include <cmath>
 
 namespace mixed {
 
 constexpr float SCALE_TARGET = 4096.f;
 
+// The largest power of two s with maxabs * s <= SCALE_TARGET, its exponent kept within +-100; 1 for
+// zero, infinities and NaN.  From the bits: a division per thread would run on the FP64 pipe.
 __device__ __forceinline__ float pow2_scale(double maxabs) {
-  if (!(maxabs > 0.0) || !isfinite(maxabs)) return 1.f;
-  int e;
-  frexp((double)SCALE_TARGET / maxabs, &e);  // 2^(e-1) <= target/max < 2^e
-  e -= 1;
+  constexpr int TARGET_EXP = 12;
+  static_assert(SCALE_TARGET == (float)(1 << TARGET_EXP), "a power of two");
+  const unsigned hi = (unsigned)__double2hiint(maxabs), lo = (unsigned)__double2loint(maxabs);
+  const int eb = (int)(hi >> 20);   // sign and exponent
+  if (eb >= 0x7ff || !(hi | lo)) return 1.f;   // negative values do not occur
+  int e = TARGET_EXP - (eb - 1023) - (((hi & 0xfffffu) | lo) ? 1 : 0);
   e = max(-100, min(100, e));
-  return (float)ldexp(1.0, e);
+  return __uint_as_float((unsigned)(e + 127) << 23);
 }
 
 // x*s split into hi = fp16(x*s) and lo = fp16(x*s - hi), in fp32 (s is a power of two, so
