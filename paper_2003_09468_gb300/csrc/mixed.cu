@@ -243,7 +243,7 @@ struct GreenP {
       if (i >= N) break;
       // i / n: (i + 1/2) / n is at least 1 / 2n from the next integer, far more than its rounding
       const int k1 = __float2int_rz(((float)i + 0.5f) * inv_n), a = i - k1 * n;
-      const float2 v = tile[r * tcg::STAGE_LD + c];
+      const float2 v = tile[tcg::tile_at(r, c)];
       float gr = v.x * st, gi = v.y * st;
       if (k1 == k2) {
         const float2 bp = bproj32[((size_t)k1 * M + p) * n + a];
@@ -294,8 +294,8 @@ struct ForceBiasP {
       const int w = nt * BN + c;
       if (w >= W) break;
       const float f = fg * rcp2(s_gsum[w]);
-      const float2 v = tile[r * tcg::STAGE_LD + c];
-      o[(size_t)c * nk * G] = make_double2((double)(v.x * f), (double)(v.y * f));
+      const float2 v = tile[tcg::tile_at(r, c)];
+      o[(size_t)c * nk * G] = make_double2(f2d(v.x * f), f2d(v.y * f));
     }
   }
 };
@@ -350,7 +350,7 @@ struct VhsP {
 #pragma unroll 4
       for (int c = tid / 64; c < wn; c += ST / 64) {
         const float st = V_SCALE * rcp2(sy[c]);
-        const float2 v0 = tile[(2 * rp) * tcg::STAGE_LD + c], v1 = tile[(2 * rp + 1) * tcg::STAGE_LD + c];
+        const float2 v0 = tile[tcg::tile_at(2 * rp, c)], v1 = tile[tcg::tile_at(2 * rp + 1, c)];
         const float r0 = v0.x * st, i0 = v0.y * st, r1 = v1.x * st, i1 = v1.y * st;
         bad |= !(fmaxf(fmaxf(fabsf(r0), fabsf(i0)), fmaxf(fabsf(r1), fabsf(i1))) < 60000.f);
         put4f_pair(o + (size_t)c * pw, r0, i0, r1, i1);
@@ -363,7 +363,7 @@ struct VhsP {
 #pragma unroll 4
       for (int c = tid / 128; c < wn; c += ST / 128) {
         const float st = V_SCALE * rcp2(sy[c]);
-        const float2 v = tile[r * tcg::STAGE_LD + c];
+        const float2 v = tile[tcg::tile_at(r, c)];
         const float vr = v.x * st, vi = v.y * st;
         bad |= !(fabsf(vr) < 60000.f && fabsf(vi) < 60000.f);
         put4f(o + (size_t)c * pw, vr, vi);
@@ -444,7 +444,7 @@ struct TaylorP {
           [&](int e, const float4& x) {
             const int r = e / BN, c = e % BN, j = mt * 128 + r, i = nt * BN + c;
             if (j >= R || i >= NM) return;
-            const float2 v = tile[r * tcg::STAGE_LD + c];
+            const float2 v = tile[tcg::tile_at(r, c)];
             const float vr = v.x * st * inv_s, vi = v.y * st * inv_s;   // V u
             cb[(size_t)j * NM + i] = make_float4(x.x + vr, x.y + vi, x.z + vr, x.w + vi);
           },
@@ -463,9 +463,9 @@ struct TaylorP {
           [&](int e, const float4& x) {
             const int r = e / (BN / 2), c = 2 * (e % (BN / 2)), j = mt * 128 + r, i = nt * BN + c;
             if (j >= R || i >= NM) return;
-            const float2 v0 = tile[r * tcg::STAGE_LD + c], v1 = tile[r * tcg::STAGE_LD + c + 1];
-            put4f_pair(tb + sp_at(j, NMp, i), fmaf(x.x, sc, v0.x * st), fmaf(x.y, sc, v0.y * st),
-                       fmaf(x.z, sc, v1.x * st), fmaf(x.w, sc, v1.y * st));
+            const float4 v = *reinterpret_cast<const float4*>(tile + tcg::tile_at(r, c));   // two columns
+            put4f_pair(tb + sp_at(j, NMp, i), fmaf(x.x, sc, v.x * st), fmaf(x.y, sc, v.y * st),
+                       fmaf(x.z, sc, v.z * st), fmaf(x.w, sc, v.w * st));
           },
           ready);
     } else {
@@ -480,7 +480,7 @@ struct TaylorP {
           [&](int e, const float2& x) {
             const int r = e / BN, c = e % BN, j = mt * 128 + r, i = nt * BN + c;
             if (j >= R || i >= NM) return;
-            const float2 v = tile[r * tcg::STAGE_LD + c];
+            const float2 v = tile[tcg::tile_at(r, c)];
             put4f(tb + sp_at(j, NMp, i), fmaf(x.x, sc, v.x * st), fmaf(x.y, sc, v.y * st));
           },
           ready);
@@ -546,12 +546,12 @@ struct ExchangeP {
 #pragma unroll
       for (int u = 0; u < UJ; ++u) {
         const int j = cl + 8 * u;
-        const float2 y0 = tile[r * tcg::STAGE_LD + 2 * j], y1 = tile[r * tcg::STAGE_LD + 2 * j + 1];
+        const float4 y = *reinterpret_cast<const float4*>(tile + tcg::tile_at(r, 2 * j));
         const float4 g = gv[it][u];
-        pr0 = fmaf(y0.x, g.x, fmaf(-y0.y, g.y, pr0));
-        pi0 = fmaf(y0.x, g.y, fmaf(y0.y, g.x, pi0));
-        pr1 = fmaf(y1.x, g.z, fmaf(-y1.y, g.w, pr1));
-        pi1 = fmaf(y1.x, g.w, fmaf(y1.y, g.z, pi1));
+        pr0 = fmaf(y.x, g.x, fmaf(-y.y, g.y, pr0));
+        pi0 = fmaf(y.x, g.y, fmaf(y.y, g.x, pi0));
+        pr1 = fmaf(y.z, g.z, fmaf(-y.w, g.w, pr1));
+        pi1 = fmaf(y.z, g.w, fmaf(y.w, g.z, pi1));
       }
       float pr = pr0 + pr1, pi = pi0 + pi1;
 #pragma unroll
@@ -623,7 +623,7 @@ struct AdjointP {
       const int ws = mt * 128 + r;
       if (ws >= WS) break;
       const float inv = rcp2(s_g[ws]);
-      const float2 v = tile[r * tcg::STAGE_LD + c];
+      const float2 v = tile[tcg::tile_at(r, c)];
       o[(size_t)r * nMp] = make_float2(v.x * inv, v.y * inv);
     }
   }
@@ -657,7 +657,7 @@ struct GramP {
     for (int r = tid / BN; r < 128; r += ST / BN) {
       const int i = mt * 128 + r;
       if (i >= N) break;
-      const float2 v = tile[r * tcg::STAGE_LD + c];
+      const float2 v = tile[tcg::tile_at(r, c)];
       gram[((size_t)ws * N + i) * N + j] = make_float2(v.x * st, v.y * st);
     }
   }
@@ -690,7 +690,7 @@ struct ApplyRP {
     for (int r = tid / BN; r < 128; r += ST / BN) {
       const int row = mt * 128 + r;
       if (row >= NM) break;
-      const float2 v = tile[r * tcg::STAGE_LD + c];
+      const float2 v = tile[tcg::tile_at(r, c)];
       phi[((size_t)ws * NM + row) * N + j] = make_double2((double)(v.x * st), (double)(v.y * st));
     }
   }

@@ -65,7 +65,7 @@ struct Coords {
 //                                                 R ready) const;
 //       called by the STORE_THREADS store threads (tid 0..STORE_THREADS-1) while the drain warps
 //       already accumulate the next tile.  Every thread calls ready() exactly once: it waits
-//       until the finished 128 x 64 tile is in shared memory, tile[r * STAGE_LD + c] = (re, im),
+//       until the finished 128 x 64 tile is in shared memory, tile[tile_at(r, c)] = (re, im),
 //       and returns false when the kernel is giving up (nothing may be stored then).  Loads
 //       that do not depend on the tile go before it, so that they are in flight while the
 //       tile is still being accumulated.
@@ -151,9 +151,16 @@ constexpr int BNP = 64;
 // few wide loads (with 8 columns a chunk's drain took 1250 clocks, longer than its MMAs).
 constexpr int DRAIN_COLS = 16;
 
-// Epilogue staging: the finished 128 x 64 tile as (re, im) fp32 pairs, rows padded to 65
-// entries so that row-per-thread and column-per-thread accesses both avoid bank conflicts.
-constexpr int STAGE_LD = BNP + 1;
+// Epilogue staging: the finished 128 x 64 tile as (re, im) fp32 pairs, column pairs (16 bytes)
+// permuted within each row's 128-byte groups by a function of the row that differs over eight
+// consecutive rows and over eight consecutive even rows: the drain's stores (a row per lane), row
+// runs read 16 bytes per lane and columns read down the rows or down every second row are then as
+// free of bank conflicts as their width allows.  Shared memory is what the MMAs' operands come
+// through, so every wavefront saved here is one for them.
+__device__ __forceinline__ int tile_swz(int r) { return (r & 6) | ((r ^ (r >> 3)) & 1); }
+__device__ __forceinline__ int tile_at(int r, int c) {   // index of (r, c) in the staged tile
+  return r * BNP + ((((c >> 1) ^ tile_swz(r)) << 1) | (c & 1));
+}
 
 // PAIR: a stage holds one half (re or im planes) of the paired B tile.
 template <int STAGES, bool PAIR = false>
@@ -161,7 +168,7 @@ struct LayoutP {
   static constexpr int A_BYTES = NPLANE * BM * 64;
   static constexpr int B_BYTES = NPLANE * BNP * 64 / (PAIR ? 2 : 1);
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int TILE_BYTES = BM * STAGE_LD * 8;
+  static constexpr int TILE_BYTES = BM * BNP * 8;
   static constexpr int BAR_BYTES = 256;
   static constexpr int SMEM = STAGES * STAGE_BYTES + TILE_BYTES + BAR_BYTES + 1024;
   static constexpr uint32_t TMEM_COLS = 512;
@@ -461,7 +468,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       __syncwarp();
       if (ntile > 0) tc::named_sync<3, TILE_BAR_THREADS>();   // previous tile stored
 #pragma unroll
-      for (int c = 0; c < BNP; ++c) tile_buf[r * STAGE_LD + c] = make_float2(sre[c], sim[c]);
+      for (int c = 0; c < BNP; c += 2)
+        *reinterpret_cast<float4*>(tile_buf + tile_at(r, c)) = make_float4(sre[c], sim[c], sre[c + 1], sim[c + 1]);
       __threadfence_block();
       __syncwarp();
       tc::named_arrive<2, TILE_BAR_THREADS>();
