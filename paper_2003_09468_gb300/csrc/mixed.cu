@@ -672,6 +672,7 @@ struct ApplyRP {
   const float* s_phi;
   const float* s_r;
   zc* phi;
+  unsigned long long* mx;   // [WS] max |phi| of the new walkers (atomic maximum of the bits), or NULL
   __device__ void tile(int t, int& b, int& mt, int& nt) const {
     nt = t % nt_n;
     mt = (t / nt_n) % mt_n;
@@ -682,16 +683,26 @@ struct ApplyRP {
     return c;
   }
   template <class R>
-  __device__ void store_tile(int ws, int mt, int nt, const float2* tile, int tid, int, R ready) const {
+  __device__ void store_tile(int ws, int mt, int nt, const float2* tile, int tid, int lane, R ready) const {
     const float st = rcp2(s_phi[ws] * s_r[ws]);
     const int c = tid % BN, j = nt * BN + c;
-    if (!ready() || j >= N) return;
+    if (!ready()) return;
+    unsigned m = 0;   // bits of |x|: ordered as the values, NaN above all
+    if (j < N) {
 #pragma unroll 4
-    for (int r = tid / BN; r < 128; r += ST / BN) {
-      const int row = mt * 128 + r;
-      if (row >= NM) break;
-      const float2 v = tile[tcg::tile_at(r, c)];
-      phi[((size_t)ws * NM + row) * N + j] = make_double2((double)(v.x * st), (double)(v.y * st));
+      for (int r = tid / BN; r < 128; r += ST / BN) {
+        const int row = mt * 128 + r;
+        if (row >= NM) break;
+        const float2 v = tile[tcg::tile_at(r, c)];
+        const float re = v.x * st, im = v.y * st;
+        phi[((size_t)ws * NM + row) * N + j] = make_double2(f2d(re), f2d(im));
+        m = max(m, max(__float_as_uint(re) & 0x7fffffffu, __float_as_uint(im) & 0x7fffffffu));
+      }
+    }
+    if (mx) {
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0)
+        atomicMax(mx + ws, (unsigned long long)__double_as_longlong((double)__uint_as_float(m)));
     }
   }
 };
@@ -730,22 +741,6 @@ __global__ void maxabs_kernel(const zc* src, size_t per, unsigned long long* out
   if (threadIdx.x == 0) {
     for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = max(m, red[i]);
     atomicMax(out + blockIdx.x, m);
-  }
-}
-
-// src[m][rows][cols] (FP64) -> dst[m][rows][ldd] with the per-matrix scale; grid (nmat, chunks)
-__global__ void split_rows_kernel(const zc* src, int rows, int cols, int ldd, const unsigned long long* mx,
-                                  float* scale, __half* dst) {
-  const int mI = blockIdx.x;
-  const float s = scale_from_bits(mx + mI);
-  if (blockIdx.y == 0 && threadIdx.x == 0) scale[mI] = s;
-  const size_t per = (size_t)rows * cols, chunk = (per + gridDim.y - 1) / gridDim.y;
-  const size_t b = blockIdx.y * chunk, e_end = min(per, b + chunk);
-  const zc* p = src + (size_t)mI * per;
-  __half* o = dst + (size_t)mI * 4 * rows * ldd;
-  for (size_t e = b + threadIdx.x; e < e_end; e += blockDim.x) {
-    const size_t i = e / cols, j = e % cols;
-    put4(o + sp_at(i, ldd, (int)j), p[e].x, p[e].y, s);
   }
 }
 
@@ -1033,45 +1028,256 @@ __global__ void trial_projector_kernel(const zc* A, zc* B, zc* scratch, int M, i
   }
 }
 
-// phi [W][2][NM][N] (FP64) -> transposed split planes [W][2N][NMp] (rows = (spin, column)),
-// per-walker scale; grid (W, chunks)
-__global__ void split_T_kernel(const zc* phi, const unsigned long long* mx, float* scale, __half* out, int NM, int N,
-                               int NMp) {
-  // one 32 x 32 block (orbital rows r, columns j) of one walker-spin, transposed through
-  // shared memory so that both the FP64 reads (along j) and the fp16 writes (along r)
-  // are coalesced; grid (ceil(NM/32), ceil(N/32), 2W)
+// phi [WS][NM][N] (FP64) -> split planes [WS][NM][Np] with a scale per walker-spin, and the
+// transposed ones [W][2N][NMp] (rows = (spin, column)) with a scale per walker, in one pass: a block
+// takes 32 x 32 (orbital rows r, columns j) of one walker-spin, transposed through shared memory
+// so that the FP64 reads and the fp16 writes of both are coalesced.  mx[ws] = max |phi| bits.
+// grid (ceil(NM/32), ceil(N/32), WS).  (Two kernels took 124 + 58 us per pass at 3x3x3, 64 walkers.)
+__global__ void __launch_bounds__(256) split_qr_kernel(const zc* phi, const unsigned long long* mx, float* s_phi,
+                                                       __half* phi_sp, float* s_t, __half* t_sp, int NM, int N,
+                                                       int Np, int NMp) {
   __shared__ float2 t[32][33];
-  const int r0 = blockIdx.x * 32, j0 = blockIdx.y * 32, w = blockIdx.z >> 1, sp = blockIdx.z & 1;
-  const float s = scale_from_bits(mx + w);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && sp == 0 && threadIdx.x == 0) scale[w] = s;
-  const zc* p = phi + ((size_t)w * 2 + sp) * NM * N;
-  for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
-    const int rr = e / 32, jj = e % 32, r = r0 + rr, j = j0 + jj;
+  const int r0 = blockIdx.x * 32, j0 = blockIdx.y * 32, ws = blockIdx.z, w = ws >> 1, sp = ws & 1;
+  const float sw = scale_from_bits(mx + ws);
+  const unsigned long long mw = max(mx[ws], mx[ws ^ 1]);   // of both spins
+  const float st = scale_from_bits(&mw);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    s_phi[ws] = sw;
+    if (sp == 0) s_t[w] = st;
+  }
+  const zc* p = phi + (size_t)ws * NM * N;
+  __half* o = phi_sp + (size_t)ws * 4 * NM * Np;
+  const int jj = threadIdx.x & 31, j = j0 + jj;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int rr = (threadIdx.x >> 5) + 8 * u, r = r0 + rr;
     float2 v = make_float2(0.f, 0.f);
     if (r < NM && j < N) {
       const zc x = p[(size_t)r * N + j];
-      v = make_float2((float)x.x * s, (float)x.y * s);
+      v = make_float2(d2f(x.x), d2f(x.y));
+      put4f(o + sp_at(r, Np, j), v.x * sw, v.y * sw);
     }
     t[rr][jj] = v;
   }
   __syncthreads();
-  __half* o = out + (size_t)w * 4 * 2 * N * NMp;
-  for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
-    const int jj = e / 32, rr = e % 32, r = r0 + rr, j = j0 + jj;
-    if (r < NM && j < N) put4f(o + sp_at(sp * N + j, NMp, r), t[rr][jj].x, t[rr][jj].y);
+  __half* ot = t_sp + (size_t)w * 4 * 2 * N * NMp;
+  const int rr = threadIdx.x & 31, r = r0 + rr;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int jc = (threadIdx.x >> 5) + 8 * u;
+    if (r < NM && j0 + jc < N) put4f(ot + sp_at(sp * N + j0 + jc, NMp, r), t[rr][jc].x * st, t[rr][jc].y * st);
   }
 }
 
-// Gram = R^dag R (Cholesky, upper R in place) and X = R^-1, both in fp32 (the Gram
-// comes from the split GEMM, about 22 bits, so FP64 would add nothing), then the split
-// planes of X^T [WS][N][Np] with a per-ws scale.  One block per walker-spin, the
-// matrix in shared memory when it fits (SMEM), else in place in global memory.
-// R^-1 is formed by Gauss-Jordan elimination on the upper triangle: step j scales row j
-// by 1/r_jj and clears column j from the rows above it, N^3/6 complex multiply-adds with
-// every step fully parallel.  A Gram matrix that is not positive definite leaves X = I
-// (the walker is kept) and is counted with the singular walkers.
+// Gram = R^dag R (Cholesky) and X = R^-1, both in fp32 (the Gram comes from the split GEMM,
+// about 22 bits, so FP64 would add nothing), then the split planes of X^T [WS][N][Np] with a
+// per-ws scale.  One block per walker-spin, the matrix in shared memory when it fits (SMEM), else in
+// place in global memory.  A Gram matrix that is not positive definite leaves X = I (the
+// walker is kept) and is counted with the singular walkers.
+//
+// Both halves are short of parallel steps rather than of arithmetic, so barriers are what counts:
+//   Cholesky in panels of CH_P rows: every thread factors the panel's diagonal block for itself in
+//     registers and carries its own column along (no barrier inside the panel), then a warp
+//     updates two rows of the trailing triangle at a time, each element once per panel;
+//   X row by row: with the rows of R scaled by 1 / r_jj, row i of X needs only row i and the scaled
+//     rows below it, so a warp runs RB rows from registers, no barriers at all, and leaves them in the
+//     lower triangle (X^T, the layout that goes out).
+// Per element the operations and their order are those of the column-by-column elimination of
+// chol_inv_kernel (three barriers per column, twice): the same bits.  N = 108, 128 matrices: 213 us
+// there; N = 256, 64 matrices: 1950 us.
+constexpr int CH_P = 4;
+constexpr int CH_MAXN = 512;   // one column per thread
+// t - conj(u) v and t - f v, the fused product of each sum spelled out (the form in which the compiler
+// contracts chol_inv_kernel's), so that the bits do not depend on where the expression stands
+__device__ __forceinline__ float2 csub_conj(float2 t, float2 u, float2 v) {
+  t.x = __fsub_rn(t.x, fmaf(u.x, v.x, __fmul_rn(u.y, v.y)));
+  t.y = __fsub_rn(t.y, fmaf(u.x, v.y, -__fmul_rn(u.y, v.x)));
+  return t;
+}
+__device__ __forceinline__ float2 csub_mul(float2 t, float2 f, float2 v) {
+  t.x = __fsub_rn(t.x, fmaf(f.x, v.x, -__fmul_rn(f.y, v.y)));
+  t.y = __fsub_rn(t.y, fmaf(f.y, v.x, __fmul_rn(f.x, v.y)));
+  return t;
+}
+template <int CH_THREADS, int CPL, int RB, bool SMEM>
+__global__ void __launch_bounds__(CH_THREADS, 512 / CH_THREADS) chol_rows_kernel(float2* gram, __half* out, float* scale, int* flags,
+                                                                  int N, int Np, double* logr) {
+  extern __shared__ __align__(16) unsigned char ci_smem[];
+  constexpr int NW = CH_THREADS / 32;
+  __shared__ float s_red[NW];
+  __shared__ double s_lr[NW];
+  const int ws = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lda = SMEM ? (N | 1) : N;   // odd: columns of 8-byte elements are free of bank conflicts
+  float2* g = gram + (size_t)ws * N * N;
+  float2* a = SMEM ? reinterpret_cast<float2*>(ci_smem) : g;
+  float* rinv = reinterpret_cast<float*>(ci_smem + (SMEM ? (size_t)N * lda * sizeof(float2) : 0));
+  if (SMEM)
+    for (int e = tid; e < N * N; e += CH_THREADS) a[(e / N) * lda + e % N] = g[e];
+  __syncthreads();
+  bool fail = false;   // every thread factors the same diagonal blocks, so it is the same in all
+  for (int j0 = 0; j0 < N && !fail; j0 += CH_P) {
+    const int jb = min(CH_P, N - j0), c = tid;   // N <= CH_THREADS: one column per thread
+    float2 D[CH_P][CH_P], v[CH_P];
+#pragma unroll
+    for (int l = 0; l < CH_P; ++l) {
+#pragma unroll
+      for (int m = l; m < CH_P; ++m)
+        D[l][m] = m < jb ? a[(size_t)(j0 + l) * lda + j0 + m] : make_float2(l == m ? 1.f : 0.f, 0.f);
+      v[l] = (l < jb && c >= j0 + l && c < N) ? a[(size_t)(j0 + l) * lda + c] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();   // everyone has read the diagonal block
+#pragma unroll
+    for (int l = 0; l < CH_P; ++l) {
+      const float d = D[l][l].x;
+      if (!(d > 0.f) || !isfinite(d)) fail = true;
+      const float r = sqrtf(d), ir = 1.f / r;
+      D[l][l] = make_float2(r, 0.f);
+#pragma unroll
+      for (int m = l + 1; m < CH_P; ++m) D[l][m] = make_float2(D[l][m].x * ir, D[l][m].y * ir);
+      v[l] = c == j0 + l ? make_float2(r, 0.f) : make_float2(v[l].x * ir, v[l].y * ir);
+#pragma unroll
+      for (int i = l + 1; i < CH_P; ++i) {
+#pragma unroll
+        for (int m = i; m < CH_P; ++m) D[i][m] = csub_conj(D[i][m], D[l][i], D[l][m]);
+        v[i] = csub_conj(v[i], D[l][i], v[l]);
+      }
+    }
+#pragma unroll
+    for (int l = 0; l < CH_P; ++l)
+      if (l < jb && c >= j0 + l && c < N) a[(size_t)(j0 + l) * lda + c] = v[l];
+    __syncthreads();
+    if (fail) break;
+    for (int i = j0 + CH_P + 2 * warp; i < N; i += 2 * NW) {
+      const bool two = i + 1 < N;
+      float2 u0[CH_P], u1[CH_P];
+#pragma unroll
+      for (int l = 0; l < CH_P; ++l) {
+        u0[l] = a[(size_t)(j0 + l) * lda + i];
+        u1[l] = a[(size_t)(j0 + l) * lda + (two ? i + 1 : i)];
+      }
+      for (int k = i + lane; k < N; k += 32) {
+        float2 t0 = a[(size_t)i * lda + k], t1 = two ? a[(size_t)(i + 1) * lda + k] : t0;
+#pragma unroll
+        for (int l = 0; l < CH_P; ++l) {
+          const float2 x = a[(size_t)(j0 + l) * lda + k];
+          t0 = csub_conj(t0, u0[l], x);
+          t1 = csub_conj(t1, u1[l], x);
+        }
+        a[(size_t)i * lda + k] = t0;
+        if (two && k > i) a[(size_t)(i + 1) * lda + k] = t1;
+      }
+    }
+    __syncthreads();
+  }
+  if (fail && tid == 0) atomicAdd(&flags[0], 1);
+  if (logr) {
+    // log det R = sum_j log r_jj (real, r_jj > 0): the change of log det (A^dag phi)
+    // under phi <- phi R^-1; nothing on failure (the walker is kept as it is)
+    double lr = 0.0;
+    if (!fail)
+      for (int j = tid; j < N; j += CH_THREADS) lr += log((double)a[(size_t)j * lda + j].x);
+    for (int o = 16; o > 0; o >>= 1) lr += __shfl_xor_sync(0xffffffffu, lr, o);
+    if (lane == 0) s_lr[warp] = lr;
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      for (int w = 0; w < NW; ++w) t += s_lr[w];
+      logr[ws] += t;
+    }
+  }
+  if (!fail) {
+    for (int j = tid; j < N; j += CH_THREADS) rinv[j] = 1.f / a[(size_t)j * lda + j].x;
+    __syncthreads();
+    for (int j = warp; j < N; j += NW) {
+      const float inv = rinv[j];
+      for (int c = j + 1 + lane; c < N; c += 32) {
+        const float2 x = a[(size_t)j * lda + c];
+        a[(size_t)j * lda + c] = make_float2(x.x * inv, x.y * inv);
+      }
+    }
+    __syncthreads();
+    const int groups = (N + RB - 1) / RB;
+    for (int k = 0; k * NW < groups; ++k) {
+      // the first rows are the longest: every other round deals them out backwards
+      const int gi = k * NW + ((k & 1) ? NW - 1 - warp : warp), i0 = gi * RB;
+      if (gi >= groups) continue;
+      float2 x[RB][CPL];
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+#pragma unroll
+        for (int q = 0; q < CPL; ++q) {
+          const int c = lane + 32 * q, i = i0 + r;
+          x[r][q] = (i < N && c > i && c < N) ? a[(size_t)i * lda + c] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+      for (int qj = 0; qj < CPL; ++qj) {
+        const int jlo = max(i0 + 1, 32 * qj), jhi = min(N, 32 * qj + 32);
+        for (int j = jlo; j < jhi; ++j) {
+          const float inv = rinv[j];
+          float2 v[CPL];
+#pragma unroll
+          for (int q = qj; q < CPL; ++q) {
+            const int c = lane + 32 * q;
+            v[q] = (c > j && c < N) ? a[(size_t)j * lda + c] : make_float2(0.f, 0.f);
+          }
+#pragma unroll
+          for (int r = 0; r < RB; ++r) {
+            if (j <= i0 + r) continue;   // row i starts at column i + 1
+            const float2 f = make_float2(__shfl_sync(0xffffffffu, x[r][qj].x, j & 31),
+                                         __shfl_sync(0xffffffffu, x[r][qj].y, j & 31));
+#pragma unroll
+            for (int q = qj; q < CPL; ++q) {
+              const float2 t = csub_mul(x[r][q], f, v[q]);
+              if (q > qj || lane + 32 * q > j) x[r][q] = t;
+            }
+            if (lane == (j & 31)) x[r][qj] = make_float2(-f.x * inv, -f.y * inv);
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+#pragma unroll
+        for (int q = 0; q < CPL; ++q) {
+          const int c = lane + 32 * q, i = i0 + r;
+          if (i < N && c > i && c < N) a[(size_t)c * lda + i] = x[r][q];
+        }
+    }
+    __syncthreads();
+  }
+  // out row jr, column i = X[i][jr] (i <= jr; identity on failure)
+  float m = 0.f;
+  for (int e = tid; e < N * N; e += CH_THREADS) {
+    const int jr = e / N, i = e - jr * N;
+    if (fail) {
+      if (i == jr) m = 1.f;
+    } else if (i < jr) {
+      const float2 v = a[(size_t)jr * lda + i];
+      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+    } else if (i == jr) {
+      m = fmaxf(m, fabsf(rinv[jr]));
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) s_red[warp] = m;
+  __syncthreads();
+  m = 0.f;
+  for (int w = 0; w < NW; ++w) m = fmaxf(m, s_red[w]);
+  const float sc = pow2_scale((double)m);
+  if (tid == 0) scale[ws] = sc;
+  __half* o = out + (size_t)ws * 4 * N * Np;
+  for (int e = tid; e < N * N; e += CH_THREADS) {
+    const int jr = e / N, i = e - jr * N;
+    float2 v = make_float2(0.f, 0.f);
+    if (i == jr)
+      v.x = fail ? 1.f : rinv[jr];
+    else if (i < jr && !fail)
+      v = a[(size_t)jr * lda + i];
+    put4f(o + sp_at(jr, Np, i), v.x * sc, v.y * sc);
+  }
+}
+
+// The same for N > 512, column by column in global memory.
 constexpr int CI_THREADS = 512;
-template <bool SMEM>
 __global__ void __launch_bounds__(CI_THREADS) chol_inv_kernel(float2* gram, __half* out, float* scale, int* flags,
                                                               int N, int Np, double* logr) {
   extern __shared__ __align__(16) unsigned char ci_smem[];
@@ -1079,11 +1285,8 @@ __global__ void __launch_bounds__(CI_THREADS) chol_inv_kernel(float2* gram, __ha
   __shared__ int s_fail;
   __shared__ float s_red[NW];
   const int ws = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float2* g = gram + (size_t)ws * N * N;
-  float2* a = SMEM ? reinterpret_cast<float2*>(ci_smem) : g;
-  float2* fcol = reinterpret_cast<float2*>(ci_smem + (SMEM ? (size_t)N * N * sizeof(float2) : 0));
-  if (SMEM)
-    for (int e = tid; e < N * N; e += CI_THREADS) a[e] = g[e];
+  float2* a = gram + (size_t)ws * N * N;
+  float2* fcol = reinterpret_cast<float2*>(ci_smem);
   if (tid == 0) s_fail = 0;
   __syncthreads();
   // Cholesky, right-looking, upper triangle only
@@ -1982,17 +2185,21 @@ cudaError_t propagate(afqmc_kp* h, zc* phi, const double* x, double* w, zc* logd
 static cudaError_t chol_inv(afqmc_kp* h, double* logr, cudaStream_t st) {
   MixedState* m = h->mixed;
   const int N = h->N;
-  const size_t full = (size_t)N * N * sizeof(float2) + (size_t)N * sizeof(float2);
-  const bool in_smem = full <= 220 * 1024;
-  const size_t bytes = in_smem ? full : (size_t)N * sizeof(float2);
   float2* gram = reinterpret_cast<float2*>(h->P);
-  if (in_smem) {
-    MTRY(set_smem_attr((const void*)chol_inv_kernel<true>, bytes));
-    chol_inv_kernel<true><<<m->WS, CI_THREADS, bytes, st>>>(gram, m->sinvt_sp, m->s_sinv, h->flags, N, m->Np, logr);
-  } else {
-    MTRY(set_smem_attr((const void*)chol_inv_kernel<false>, bytes));
-    chol_inv_kernel<false><<<m->WS, CI_THREADS, bytes, st>>>(gram, m->sinvt_sp, m->s_sinv, h->flags, N, m->Np, logr);
-  }
+  const size_t row = (size_t)N * sizeof(float), full = (size_t)N * (N | 1) * sizeof(float2) + row;
+  const bool in_smem = full <= 220 * 1024;
+  const size_t bytes = N > CH_MAXN ? (size_t)N * sizeof(float2) : (in_smem ? full : row);
+  // CPL columns per lane; small matrices take fewer threads, so that several share an SM
+  auto fn = N > CH_MAXN           ? chol_inv_kernel
+            : N <= 32             ? chol_rows_kernel<128, 1, 4, true>
+            : N <= 64             ? chol_rows_kernel<256, 2, 4, true>
+            : N <= 128            ? chol_rows_kernel<512, 4, 4, true>
+            : N <= 256 && in_smem ? chol_rows_kernel<512, 8, 4, true>
+            : N <= 256            ? chol_rows_kernel<512, 8, 4, false>
+                                  : chol_rows_kernel<512, 16, 2, false>;
+  const int threads = N > CH_MAXN ? CI_THREADS : N <= 32 ? 128 : N <= 64 ? 256 : 512;
+  MTRY(set_smem_attr((const void*)fn, bytes));
+  fn<<<m->WS, threads, bytes, st>>>(gram, m->sinvt_sp, m->s_sinv, h->flags, N, m->Np, logr);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
 }
@@ -2004,15 +2211,15 @@ static cudaError_t chol_inv(afqmc_kp* h, double* logr, cudaStream_t st) {
 static cudaError_t cholqr2(afqmc_kp* h, zc* phi, double* logr, cudaStream_t st) {
   MixedState* m = h->mixed;
   if (logr) MTRY(cudaMemsetAsync(logr, 0, sizeof(double) * m->WS, st));
-  const int WS = m->WS, N = h->N, NM = h->NM, W = h->W;
-  unsigned long long* mx_phi = m->mx;
-  unsigned long long* mx_w = m->mx + 2 * WS + 3 * W;
+  const int WS = m->WS, N = h->N, NM = h->NM;
+  // maxima of the input walkers and of the first pass's result (which ApplyRP collects as it stores)
+  unsigned long long* mx[2] = {m->mx, m->mx + WS};
+  MTRY(cudaMemsetAsync(m->mx, 0, sizeof(unsigned long long) * 2 * WS, st));
+  maxabs_kernel<<<dim3(WS, SPLIT_CHUNKS), 256, 0, st>>>(phi, (size_t)NM * N, mx[0]);
+  AFQMC_LAUNCHED(h);
   for (int pass = 0; pass < 2; ++pass) {
-    MTRY(cudaMemsetAsync(m->mx, 0, sizeof(unsigned long long) * (2 * WS + 3 * W + W), st));
-    maxabs_kernel<<<dim3(W, SPLIT_CHUNKS), 256, 0, st>>>(phi, (size_t)2 * NM * N, mx_w);
-    AFQMC_LAUNCHED(h);
-    split_T_kernel<<<dim3(cdiv(NM, 32), cdiv(N, 32), 2 * W), 256, 0, st>>>(phi, mx_w, m->s_t, m->t_sp[0], NM, N,
-                                                                          m->NMp);
+    split_qr_kernel<<<dim3(cdiv(NM, 32), cdiv(N, 32), WS), 256, 0, st>>>(phi, mx[pass], m->s_phi, m->phi_sp, m->s_t,
+                                                                        m->t_sp[0], NM, N, m->Np, m->NMp);
     AFQMC_LAUNCHED(h);
     MTRY(cudaGetLastError());
     GramP g;
@@ -2024,17 +2231,13 @@ static cudaError_t cholqr2(afqmc_kp* h, zc* phi, double* logr, cudaStream_t st) 
     MTRY(run_gemm(h, m->m_t[0], m->m_t0_b, g, h->flags + 1, st));
     AFQMC_LAUNCHED(h);
     MTRY(chol_inv(h, logr, st));
-    maxabs_kernel<<<dim3(WS, SPLIT_CHUNKS), 256, 0, st>>>(phi, (size_t)NM * N, mx_phi);
-    AFQMC_LAUNCHED(h);
-    split_rows_kernel<<<dim3(WS, SPLIT_CHUNKS), 256, 0, st>>>(phi, NM, N, m->Np, mx_phi, m->s_phi, m->phi_sp);
-    AFQMC_LAUNCHED(h);
-    MTRY(cudaGetLastError());
     ApplyRP a;
     a.mt_n = cdiv(NM, 128);
     a.nt_n = cdiv(N, BN);
     a.tiles = WS * a.mt_n * a.nt_n;
     a.kchunks = m->Np / 32;
     a.NM = NM; a.N = N; a.s_phi = m->s_phi; a.s_r = m->s_sinv; a.phi = phi;
+    a.mx = pass == 0 ? mx[1] : nullptr;
     MTRY(run_gemm(h, m->m_phi_a, m->m_sinvt_b, a, h->flags + 1, st));
     AFQMC_LAUNCHED(h);
   }
