@@ -12,8 +12,10 @@
 //                                 Sec. 3.2 energy steps 1-3
 #include <math.h>
 
+#include <algorithm>
 #include <utility>
 
+#include "attr.hpp"
 #include "handle.hpp"
 
 namespace fp64 {
@@ -339,45 +341,53 @@ static cudaError_t overlap(afqmc_kp* h, const zc* phi, cudaStream_t st) {
 
 // In-place LU of S (row pivoting), log det, optional inverse.  sing[b] = 1 if a
 // pivot is zero or not finite; then Sinv = 0 and logdet = (-inf, 0).
+// A chain of short steps: SA keeps the matrix in shared memory while it is factored, SX the
+// inverse too (from global memory every step waited for L2); the pivot search is a warp maximum and
+// one pass over the warps; the logarithms of the pivots and the reciprocals of U's diagonal, which
+// one thread formed column by column while the others waited, are formed for all columns at once.
+// N = 16, 32 matrices: 146 us before.
+template <bool SA, bool SX>
 __global__ void __launch_bounds__(256) lu_kernel(zc* S, zc* Sinv, zc* logdet, int* sing, int* flags,
                                                  int N, int want_inv, int* perm_ws) {
-  const int b = blockIdx.x;
-  zc* a = S + (long)b * N * N;
+  const int b = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  extern __shared__ __align__(16) unsigned char lu_smem[];
+  zc* g = S + (long)b * N * N;
+  zc* a = SA ? reinterpret_cast<zc*>(lu_smem) : g;
   int* perm = perm_ws + (long)b * N;
-  __shared__ double s_val[256];
-  __shared__ int s_idx[256];
-  __shared__ int s_sing;
-  __shared__ double s_logabs, s_arg;
-  __shared__ int s_swaps;
-  if (threadIdx.x == 0) { s_sing = 0; s_logabs = 0.0; s_arg = 0.0; s_swaps = 0; }
+  __shared__ unsigned long long s_val[8];
+  __shared__ int s_idx[8];
+  __shared__ zc s_red[8];
+  int swaps = 0;   // the same in every thread
+  bool singular = false;
+  if (SA)
+    for (long e = threadIdx.x; e < (long)N * N; e += blockDim.x) a[e] = g[e];
   for (int i = threadIdx.x; i < N; i += blockDim.x) perm[i] = i;
   __syncthreads();
   for (int j = 0; j < N; ++j) {
-    double best = -1.0;
-    int bi = j;
+    // largest |a_ij|^2, the smallest row among equals, compared by bits (ordered as the values,
+    // NaN left out): 64-bit compares would go through the FP64 pipe
+    unsigned long long best = 0;
+    int bi = N;
     for (int i = j + threadIdx.x; i < N; i += blockDim.x) {
-      double v = zabs2(a[(long)i * N + j]);
-      if (v > best) { best = v; bi = i; }
+      const unsigned long long v = (unsigned long long)__double_as_longlong(zabs2(a[(long)i * N + j]));
+      if (v <= 0x7ff0000000000000ull && (v > best || bi == N)) { best = v; bi = i; }
     }
-    s_val[threadIdx.x] = best;
-    s_idx[threadIdx.x] = bi;
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long v2 = __shfl_xor_sync(0xffffffffu, best, o);
+      const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (v2 > best || (v2 == best && i2 < bi)) { best = v2; bi = i2; }
+    }
+    if (lane == 0) { s_val[wid] = best; s_idx[wid] = bi; }
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) {
-        double v2 = s_val[threadIdx.x + o];
-        int i2 = s_idx[threadIdx.x + o];
-        if (v2 > s_val[threadIdx.x] || (v2 == s_val[threadIdx.x] && i2 < s_idx[threadIdx.x])) {
-          s_val[threadIdx.x] = v2;
-          s_idx[threadIdx.x] = i2;
-        }
-      }
-      __syncthreads();
+    unsigned long long pv = s_val[0];
+    int p = s_idx[0];
+    for (int w = 1; w < nw; ++w) {
+      const unsigned long long v2 = s_val[w];
+      const int i2 = s_idx[w];
+      if (v2 > pv || (v2 == pv && i2 < p)) { pv = v2; p = i2; }
     }
-    const int p = s_idx[0];
-    const double pv = s_val[0];
-    if (!(pv > 0.0) || !isfinite(pv)) {
-      if (threadIdx.x == 0) s_sing = 1;
-      __syncthreads();
+    if (pv == 0 || pv >= 0x7ff0000000000000ull) {   // zero, infinite or all NaN; the same in every thread
+      singular = true;
       break;
     }
     if (p != j) {
@@ -386,19 +396,14 @@ __global__ void __launch_bounds__(256) lu_kernel(zc* S, zc* Sinv, zc* logdet, in
         a[(long)j * N + c] = a[(long)p * N + c];
         a[(long)p * N + c] = t;
       }
-      if (threadIdx.x == 0) {
-        int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
-        s_swaps++;
-      }
+      if (threadIdx.x == 0) { int t = perm[j]; perm[j] = perm[p]; perm[p] = t; }
+      ++swaps;
     }
     __syncthreads();
-    const zc piv = a[(long)j * N + j];
-    if (threadIdx.x == 0) {
-      s_logabs += 0.5 * log(zabs2(piv));
-      s_arg += atan2(piv.y, piv.x);
+    if (j + 1 + (int)threadIdx.x < N) {   // only the warps that use it: an FP64 division of 8 warps is a column's longest step
+      const zc inv = zinv(a[(long)j * N + j]);
+      for (int i = j + 1 + threadIdx.x; i < N; i += blockDim.x) a[(long)i * N + j] = zmul(a[(long)i * N + j], inv);
     }
-    const zc inv = zinv(piv);
-    for (int i = j + 1 + threadIdx.x; i < N; i += blockDim.x) a[(long)i * N + j] = zmul(a[(long)i * N + j], inv);
     __syncthreads();
     const int rem = N - j - 1;
     for (long e = threadIdx.x; e < (long)rem * rem; e += blockDim.x) {
@@ -408,23 +413,63 @@ __global__ void __launch_bounds__(256) lu_kernel(zc* S, zc* Sinv, zc* logdet, in
     }
     __syncthreads();
   }
-  const int singular = s_sing;
+  zc la = zzero();   // (log |pivot|, arg pivot) sums
+  if (!singular)
+    for (int j = threadIdx.x; j < N; j += blockDim.x) {
+      const zc piv = a[(long)j * N + j];
+      la = zadd(la, zmake(0.5 * log(zabs2(piv)), atan2(piv.y, piv.x)));
+    }
+  la = block_zsum(la, s_red);
   if (threadIdx.x == 0) {
     if (singular) {
       logdet[b] = zmake(-INFINITY, 0.0);
       sing[b] = 1;
       atomicAdd(&flags[0], 1);
     } else {
-      double ang = s_arg + (s_swaps & 1 ? M_PI : 0.0);
+      double ang = la.y + (swaps & 1 ? M_PI : 0.0);
       ang = remainder(ang, 2.0 * M_PI);
-      logdet[b] = zmake(s_logabs, ang);
+      logdet[b] = zmake(la.x, ang);
       sing[b] = 0;
     }
   }
+  if (SA)   // the factors, as callers of the in-place form find them
+    for (long e = threadIdx.x; e < (long)N * N; e += blockDim.x) g[e] = a[e];
   if (!want_inv) return;
-  zc* x = Sinv + (long)b * N * N;
+  zc* out = Sinv + (long)b * N * N;
   if (singular) {
-    for (long e = threadIdx.x; e < (long)N * N; e += blockDim.x) x[e] = zzero();
+    for (long e = threadIdx.x; e < (long)N * N; e += blockDim.x) out[e] = zzero();
+    return;
+  }
+  // U's diagonal by its reciprocals: the solves below read nothing else of it, and nothing reads the
+  // factors after them
+  __syncthreads();
+  for (int j = threadIdx.x; j < N; j += blockDim.x) a[(long)j * N + j] = zinv(a[(long)j * N + j]);
+  __syncthreads();
+  zc* x = SX ? a + (long)N * N : out;
+  if (SX) {
+    // L U X = P by rows: once row l of X is known, every thread takes its share of the rows still to
+    // come (a column per thread, as below, is one dependent chain of N^2 multiply-adds)
+    for (int e = threadIdx.x; e < N * N; e += blockDim.x) x[e] = zmake(perm[e / N] == e % N ? 1.0 : 0.0, 0.0);
+    __syncthreads();
+    for (int l = 0; l < N; ++l) {
+      for (int e = threadIdx.x; e < (N - 1 - l) * N; e += blockDim.x) {
+        const int i = l + 1 + e / N, c = e % N;
+        const zc f = a[i * N + l];
+        x[i * N + c] = zfma(zmake(-f.x, -f.y), x[l * N + c], x[i * N + c]);
+      }
+      __syncthreads();
+    }
+    for (int l = N - 1; l >= 0; --l) {
+      for (int c = threadIdx.x; c < N; c += blockDim.x) x[l * N + c] = zmul(x[l * N + c], a[l * N + l]);
+      __syncthreads();
+      for (int e = threadIdx.x; e < l * N; e += blockDim.x) {
+        const int i = e / N, c = e % N;
+        const zc f = a[i * N + l];
+        x[i * N + c] = zfma(zmake(-f.x, -f.y), x[l * N + c], x[i * N + c]);
+      }
+      __syncthreads();
+    }
+    for (int e = threadIdx.x; e < N * N; e += blockDim.x) out[e] = x[e];
     return;
   }
   // Column c of S^-1 solves L U x = P e_c: forward (unit lower), then backward.
@@ -437,19 +482,30 @@ __global__ void __launch_bounds__(256) lu_kernel(zc* S, zc* Sinv, zc* logdet, in
     for (int i = N - 1; i >= 0; --i) {
       zc s = x[(long)i * N + c];
       for (int l = i + 1; l < N; ++l) s = zfma(zmake(-a[(long)i * N + l].x, -a[(long)i * N + l].y), x[(long)l * N + c], s);
-      x[(long)i * N + c] = zmul(s, zinv(a[(long)i * N + i]));
+      x[(long)i * N + c] = zmul(s, a[(long)i * N + i]);
     }
   }
+}
+
+static cudaError_t lu_launch(afqmc_kp* h, zc* ld, int* sing, int want_inv, cudaStream_t st) {
+  // pivot scratch lives in the P buffer (used otherwise only by the backward pass)
+  int* perm = reinterpret_cast<int*>(h->P);
+  const size_t one = sizeof(zc) * (size_t)h->N * h->N, cap = 200 * 1024;
+  const bool sx = want_inv && 2 * one <= cap, sa = one <= cap;
+  auto fn = sx ? lu_kernel<true, true> : sa ? lu_kernel<true, false> : lu_kernel<false, false>;
+  const size_t bytes = sx ? 2 * one : sa ? one : 0;
+  cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(fn), bytes);
+  if (e != cudaSuccess) return e;
+  fn<<<2 * h->W, 256, bytes, st>>>(h->S, h->Sinv, ld, sing, h->flags, h->N, want_inv, perm);
+  AFQMC_LAUNCHED(h);
+  return cudaGetLastError();
 }
 
 // Gh[w][s] = (phi S^-1)^T = S^-T phi^T  (N x NM)
 static cudaError_t green_impl(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st) {
   cudaError_t e = overlap(h, phi, st);
   if (e != cudaSuccess) return e;
-  // pivot scratch lives in the P buffer (used otherwise only by the backward pass)
-  lu_kernel<<<2 * h->W, 256, 0, st>>>(h->S, h->Sinv, ld, sing, h->flags, h->N, 1, reinterpret_cast<int*>(h->P));
-  AFQMC_LAUNCHED(h);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = lu_launch(h, ld, sing, 1, st)) != cudaSuccess) return e;
   const int N = h->N, NM = h->NM;
   ZGemm g = gemm_init(N, NM, N, 1, 1);
   g.A = h->Sinv; g.lda = N; g.sA[0] = (long)N * N;
@@ -468,7 +524,9 @@ cudaError_t green(afqmc_kp* h, const zc* phi, cudaStream_t st) {
 
 // ---------------------------------------------------------------------------
 // Cholesky trace X[w][Q][g] = sum_k sum_{a,r} LH[Q][k][g][a][r] (Gh_up + Gh_dn)[(k,a)][(k-Q,r)]
-// Block (Q, walker chunk); one warp per g at a time, lanes over (a, r).
+// Block (Q, walker chunk, vectors); one warp per g at a time, lanes over (a, r).  The vectors are
+// spread over as many blocks as fill the GPU (with all of them in one block the 2x2x2 system of 16
+// walkers ran on 16 SMs, 168 us).
 // ---------------------------------------------------------------------------
 constexpr int XWC = 8;  // walkers per block
 
@@ -478,7 +536,7 @@ __global__ void __launch_bounds__(256) xtrace_kernel(const zc* LH, const zc* Gh,
   const int Q = blockIdx.x, w0 = blockIdx.y * XWC;
   const int N = nk * n, NM = nk * M, nM = n * M;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  for (int g0 = 0; g0 < G; g0 += nwarp) {
+  for (int g0 = blockIdx.z * nwarp; g0 < G; g0 += nwarp * gridDim.z) {
     const int g = g0 + wid;
     zc acc[XWC];
 #pragma unroll
@@ -516,7 +574,9 @@ __global__ void __launch_bounds__(256) xtrace_kernel(const zc* LH, const zc* Gh,
 }
 
 cudaError_t cholesky_trace(afqmc_kp* h, cudaStream_t st) {
-  dim3 grid(h->nk, (h->W + XWC - 1) / XWC);
+  const int wc = (h->W + XWC - 1) / XWC, groups = (h->G + 7) / 8;   // 8 warps, one vector each
+  const long filled = (long)h->nk * wc;
+  dim3 grid(h->nk, wc, (unsigned)std::max(1L, std::min((long)groups, (912 + filled - 1) / filled)));   // 6 blocks per SM
   size_t smem = sizeof(zc) * XWC * h->n * h->M;
   xtrace_kernel<<<grid, 256, smem, st>>>(h->LH, h->Gh, h->X, h->kminus, h->nk, h->G, h->M, h->n, h->W);
   AFQMC_LAUNCHED(h);
@@ -742,19 +802,13 @@ static cudaError_t one_body(afqmc_kp* h, const zc* in, zc* out, cudaStream_t st)
 // The two halves of overlap_lu, for callers that use S before it is factorised.
 cudaError_t overlap_only(afqmc_kp* h, const zc* phi, cudaStream_t st) { return overlap(h, phi, st); }
 cudaError_t lu_only(afqmc_kp* h, zc* ld, int* sing, int want_inv, cudaStream_t st) {
-  lu_kernel<<<2 * h->W, 256, 0, st>>>(h->S, h->Sinv, ld, sing, h->flags, h->N, want_inv,
-                                      reinterpret_cast<int*>(h->P));
-  AFQMC_LAUNCHED(h);
-  return cudaGetLastError();
+  return lu_launch(h, ld, sing, want_inv, st);
 }
 
 cudaError_t overlap_lu(afqmc_kp* h, const zc* phi, zc* ld, int* sing, int want_inv, cudaStream_t st) {
   cudaError_t e = overlap(h, phi, st);
   if (e != cudaSuccess) return e;
-  lu_kernel<<<2 * h->W, 256, 0, st>>>(h->S, h->Sinv, ld, sing, h->flags, h->N, want_inv,
-                                      reinterpret_cast<int*>(h->P));
-  AFQMC_LAUNCHED(h);
-  return cudaGetLastError();
+  return lu_launch(h, ld, sing, want_inv, st);
 }
 
 static cudaError_t logdet_only(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st) {
