@@ -846,14 +846,19 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     }
   }
   __syncthreads();
-  // ---- log det from the pivots (each CTA its own columns')
+  // ---- log det from the pivots (each CTA its own columns'): the logarithms on one half of the threads,
+  // the arguments on the other, so that the two long FP64 sequences run side by side
   double lg = 0.0, an = 0.0;
-  if (!singular)
-    for (int c = tid; c < nc; c += GC_THREADS) {
+  if (!singular) {
+    constexpr int HALF = GC_THREADS / 2;
+    for (int c = tid % HALF; c < nc; c += HALF) {
       const double2 v = make_double2(ffa::to_double(ffa::re(piv[c])), ffa::to_double(ffa::im(piv[c])));
-      lg += 0.5 * log(v.x * v.x + v.y * v.y);
-      an += atan2(v.y, v.x);
+      if (tid < HALF)
+        lg += 0.5 * log(v.x * v.x + v.y * v.y);
+      else
+        an += atan2(v.y, v.x);
     }
+  }
   lg = block_sum_d(lg, s_red);
   an = block_sum_d(an, s_red);
   float m = 0.f;

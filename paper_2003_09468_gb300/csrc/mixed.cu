@@ -49,8 +49,8 @@ struct MixedState {
   __half* y_sp = nullptr;     float* s_y = nullptr;     // [Nk][W][Gp], s_y[Q][W]
   __half* v_sp = nullptr;                                // [W][NM][NMp]
   __half* t_sp[2] = {nullptr, nullptr}; float* s_t = nullptr;  // [W][2N][NMp]
-  double2* acc = nullptr;                                // [W][2N][NM] (scratch: float4 Taylor corrections, phi_perp)
-  float2* p32 = nullptr;                                 // [W][2N][NM] phi' in fp32 (Taylor series)
+  float2* corr = nullptr;                                // [W][2N][NM] corrections of the walker (before the series: phi_perp)
+  float2* p32 = nullptr;                                 // [W][2N][NM] phi', then phi'', in fp32 (Taylor series)
   double2* xpart = nullptr;                              // [T][ntile][WS]
   double2* xk = nullptr;                                 // [fb_groups][W][Nk][G] Cholesky traces per group of k blocks
   int fb_groups = 1;                                     // groups of k blocks in the force-bias GEMM
@@ -389,8 +389,8 @@ struct TaylorP {
   float inv_j;
   int last;
   const float* s_t;
-  const float2* p32;  // [W][R][NM] phi' in fp32
-  float4* corr;       // [W][R][NM] (d, .) with d = phi' - phi on entry; (phi'' - phi, phi'') after the last step
+  float2* p32;        // [W][R][NM] phi' in fp32; phi'' after the last step
+  float2* corr;       // [W][R][NM] phi' - phi; phi'' - phi after the last step
   __half* t_next;     // [W][R][NMp]
   __device__ void tile(int t, int& b, int& mt, int& nt) const {
     nt = t % nt_n;
@@ -430,15 +430,15 @@ struct TaylorP {
     const float st = inv_j / V_SCALE, sc = s_t[b];
     if (last) {
       const float inv_s = rcp2(sc);
-      float4* cb = corr + (size_t)b * R * NM;
-      const float2* pb = p32 + (size_t)b * R * NM;
+      float2* cb = corr + (size_t)b * R * NM;
+      float2* pb = p32 + (size_t)b * R * NM;
       batches<128 * BN, float4>(
           tid,
           [&](int e) {
             const int j = mt * 128 + e / BN, i = nt * BN + e % BN;
             if (j >= R || i >= NM) return make_float4(0.f, 0.f, 0.f, 0.f);
             const size_t o = (size_t)j * NM + i;
-            const float2 d = reinterpret_cast<const float2*>(cb)[2 * o], q = pb[o];
+            const float2 d = cb[o], q = pb[o];
             return make_float4(d.x, d.y, q.x, q.y);
           },
           [&](int e, const float4& x) {
@@ -446,7 +446,9 @@ struct TaylorP {
             if (j >= R || i >= NM) return;
             const float2 v = tile[tcg::tile_at(r, c)];
             const float vr = v.x * st * inv_s, vi = v.y * st * inv_s;   // V u
-            cb[(size_t)j * NM + i] = make_float4(x.x + vr, x.y + vi, x.z + vr, x.w + vi);
+            const size_t o = (size_t)j * NM + i;
+            cb[o] = make_float2(x.x + vr, x.y + vi);
+            pb[o] = make_float2(x.z + vr, x.w + vi);
           },
           ready);
     } else if ((NM & 1) == 0) {
@@ -889,10 +891,10 @@ __device__ __forceinline__ void onebody_apply4(const float2* Dt, const float2* b
 
 // First one-body half step, phi' = phi + D phi (Sec. 3.2 step 3), in the transposed
 // (row = (spin, column), column = orbital) layout of the Taylor series, as fp32 parts only:
-// p32 = phi' (rounded) and corr.xy = D phi.  The FP64 walker itself is added back once,
+// p32 = phi' (rounded) and corr = D phi.  The FP64 walker itself is added back once,
 // after the series (onebody_out_kernel).  mx[w] = max |p32|.
 // grid (k, ws, j-chunk of 64)
-__global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float4* corr, float2* p32,
+__global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float2* corr, float2* p32,
                                   unsigned long long* mx, int nk, int M, int N, int NM) {
   __shared__ float red[32];
   const int k = blockIdx.x, ws = blockIdx.y, j0 = blockIdx.z * 64;
@@ -926,7 +928,7 @@ __global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float4* co
       const int j = jq + 16 * u;
       if (j >= jn) continue;
       const size_t o = ((size_t)w * 2 * N + sp * N + j0 + j) * NM + k * M + p;
-      reinterpret_cast<float2*>(corr)[2 * o] = c[u];
+      corr[o] = c[u];
       const float2 b = blk[p * OB_LD + j];
       const float2 v = make_float2(b.x + c[u].x, b.y + c[u].y);
       p32[o] = v;
@@ -937,15 +939,15 @@ __global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float4* co
   if (threadIdx.x == 0) atomic_max_pos(mx + w, (double)m);
 }
 
-// Second half step: with corr.xy = d = phi'' - phi and corr.zw = phi'' (fp32) after the
-// Taylor series, phi <- phi + d + D phi'' (the sum of fp32 corrections is added to the
-// FP64 walker once).  grid (k, ws, j-chunk of 64).  STAGE_D: both parts of corr are staged in
+// Second half step: with corr = d = phi'' - phi and p32 = phi'' (fp32) after the Taylor series, phi <- phi + d + D phi'' (the sum of fp32 corrections is added to the
+// FP64 walker once).  grid (k, ws, j-chunk of 64).  STAGE_D: both are staged in
 // shared memory by one coalesced pass (rows j, orbitals contiguous), and the FP64 walker
 // (orbital rows, columns j contiguous) is updated with sixteen consecutive threads on sixteen
 // consecutive columns; without it (M too large for the second staging buffer) the threads
 // run down the orbitals and read d from global memory.
 template <bool STAGE_D>
-__global__ void onebody_out_kernel(const float4* corr, const float2* dhalf, zc* phi, int nk, int M, int N, int NM) {
+__global__ void onebody_out_kernel(const float2* corr, const float2* p32, const float2* dhalf, zc* phi, int nk, int M,
+                                   int N, int NM) {
   const int k = blockIdx.x, ws = blockIdx.y, j0 = blockIdx.z * 64;
   const int w = ws >> 1, sp = ws & 1;
   const int jn = min(64, N - j0);
@@ -957,13 +959,13 @@ __global__ void onebody_out_kernel(const float4* corr, const float2* dhalf, zc* 
     const int p = e / M, q = e % M;
     Dt[q * M + p] = dhalf[(size_t)k * M * M + e];
   }
-  const float4* src = corr + ((size_t)w * 2 * N + sp * N + j0) * NM + k * M;
+  const size_t at = ((size_t)w * 2 * N + sp * N + j0) * NM + k * M;
+  const float2* ds = corr + at;
+  const float2* ps = p32 + at;
   for (int e = threadIdx.x; e < M * 64; e += blockDim.x) {
     const int j = e / M, q = e % M;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (j < jn) x = src[(size_t)j * NM + q];
-    blk[q * OB_LD + j] = make_float2(x.z, x.w);
-    if (STAGE_D) dd[q * OB_LD + j] = make_float2(x.x, x.y);
+    blk[q * OB_LD + j] = j < jn ? ps[(size_t)j * NM + q] : make_float2(0.f, 0.f);
+    if (STAGE_D) dd[q * OB_LD + j] = j < jn ? ds[(size_t)j * NM + q] : make_float2(0.f, 0.f);
   }
   __syncthreads();
   zc* dst = phi + (size_t)ws * NM * N;
@@ -980,7 +982,7 @@ __global__ void onebody_out_kernel(const float4* corr, const float2* dhalf, zc* 
     for (int u = 0; u < 4; ++u) {
       const int j = jq + 16 * u;
       if (j >= jn) continue;
-      const float2 d = STAGE_D ? dd[p * OB_LD + j] : reinterpret_cast<const float2*>(src)[2 * ((size_t)j * NM + p)];
+      const float2 d = STAGE_D ? dd[p * OB_LD + j] : ds[(size_t)j * NM + p];
       v[u].x += f2d(d.x + c[u].x);
       v[u].y += f2d(d.y + c[u].y);
       row[j] = v[u];
@@ -1416,7 +1418,7 @@ __global__ void dhalf_kernel(const zc* Ehalf, float2* d, int nk, int M) {
   }
 }
 
-// E1 and EC per walker from the fp32 Green's function and the FP64 X.  One block per walker, 1024
+// E1 and EC per walker from the fp32 Green's function and the FP64 X.  One block per walker, up to 1024
 // threads: FP64 work of two operations per clock, so the loads of many elements have to overlap.
 __global__ void e1_ec_mixed_kernel(const zc* AhH, const float2* g32, const zc* X, const int* minus, zc* eloc, int nk,
                                    int M, int n, int Mp, int G, int WS) {
@@ -1653,7 +1655,7 @@ static TaylorP taylor_params(const afqmc_kp* h, int j, int nxt) {
   p.R = R; p.NM = h->NM; p.NMp = m->NMp;
   p.inv_j = 1.f / (float)j;
   p.last = (j == 1);
-  p.s_t = m->s_t; p.p32 = m->p32; p.corr = reinterpret_cast<float4*>(m->acc); p.t_next = m->t_sp[nxt];
+  p.s_t = m->s_t; p.p32 = m->p32; p.corr = m->corr; p.t_next = m->t_sp[nxt];
   return p;
 }
 // The same term in the CTA-pair form: mt_n counts pairs of 128-row tiles.
@@ -1899,7 +1901,7 @@ static cudaError_t create_impl(afqmc_kp* h, cudaStream_t st) {
   MTRY(dalloc(h, &m->t_sp[0], (size_t)W * 4 * 2 * N * NMp, true, st));
   MTRY(dalloc(h, &m->t_sp[1], (size_t)W * 4 * 2 * N * NMp, true, st));
   MTRY(dalloc(h, &m->s_t, W, true, st));
-  MTRY(dalloc(h, &m->acc, (size_t)W * 2 * N * NM, true, st));
+  MTRY(dalloc(h, &m->corr, (size_t)W * 2 * N * NM, true, st));
   MTRY(dalloc(h, &m->p32, (size_t)W * 2 * N * NM, true, st));
   MTRY(dalloc(h, &m->xpart, (size_t)T * ntx * WS, true, st));
   // force-bias GEMM: the fewest groups of k blocks (a divisor of Nk) that give every SM a tile
@@ -2030,7 +2032,7 @@ static cudaError_t green_pre(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cuda
   // phi (A^dag phi)^-1 = B + phi_perp S^-1 with B = A (A^dag A)^-1 and phi_perp = phi - B S:
   // the trial-subspace part is exact, so the split GEMM never forms the large
   // cancelling partial sums of S^-1 (A^dag phi) = I.
-  float2* phi_perp = reinterpret_cast<float2*>(m->acc);  // free until the Taylor series
+  float2* phi_perp = m->corr;  // free until the Taylor series
   // S = A^dag phi, phi_perp and S^-1 / log det in double-float (ffla.cu); the inverse
   // leaves the kernel as the split planes of S^-T
   MTRY(cudaMemsetAsync(m->mx, 0, sizeof(unsigned long long) * (2 * WS + 3 * h->W), st));
@@ -2113,9 +2115,8 @@ static cudaError_t taylor_pre(afqmc_kp* h, const zc* phi, cudaStream_t st) {
   dim3 g1(h->nk, m->WS, cdiv(h->N, 64));
   unsigned long long* mx_acc = m->mx + 2 * m->WS + 3 * h->W;
   MTRY(cudaMemsetAsync(mx_acc, 0, sizeof(unsigned long long) * h->W, st));
-  float4* corr = reinterpret_cast<float4*>(m->acc);
   prof_begin(h, AFQMC_STAGE_ONEBODY, st);
-  onebody_in_kernel<<<g1, 256, onebody_smem(h), st>>>(phi, m->dhalf, corr, m->p32, mx_acc, h->nk, h->M, h->N,
+  onebody_in_kernel<<<g1, 256, onebody_smem(h), st>>>(phi, m->dhalf, m->corr, m->p32, mx_acc, h->nk, h->M, h->N,
                                                        h->NM);
   AFQMC_LAUNCHED(h);
   split_rows32_kernel<<<dim3(h->W, SPLIT_CHUNKS), 256, 0, st>>>(m->p32, R, h->NM, m->NMp, mx_acc, m->s_t, m->t_sp[0]);
@@ -2126,12 +2127,11 @@ static cudaError_t taylor_pre(afqmc_kp* h, const zc* phi, cudaStream_t st) {
 static cudaError_t taylor_post(afqmc_kp* h, zc* phi, cudaStream_t st) {
   MixedState* m = h->mixed;
   dim3 g1(h->nk, m->WS, cdiv(h->N, 64));
-  float4* corr = reinterpret_cast<float4*>(m->acc);
   prof_begin(h, AFQMC_STAGE_ONEBODY, st);
   if (onebody_out_staged(h))
-    onebody_out_kernel<true><<<g1, 256, onebody_out_smem(h), st>>>(corr, m->dhalf, phi, h->nk, h->M, h->N, h->NM);
+    onebody_out_kernel<true><<<g1, 256, onebody_out_smem(h), st>>>(m->corr, m->p32, m->dhalf, phi, h->nk, h->M, h->N, h->NM);
   else
-    onebody_out_kernel<false><<<g1, 256, onebody_smem(h), st>>>(corr, m->dhalf, phi, h->nk, h->M, h->N, h->NM);
+    onebody_out_kernel<false><<<g1, 256, onebody_smem(h), st>>>(m->corr, m->p32, m->dhalf, phi, h->nk, h->M, h->N, h->NM);
   AFQMC_LAUNCHED(h);
   prof_end(h, st);
   return cudaGetLastError();
@@ -2254,7 +2254,8 @@ cudaError_t orthonormalise(afqmc_kp* h, zc* phi, zc* logdet, cudaStream_t st) {
 
 static cudaError_t e1_ec(afqmc_kp* h, zc* eloc, cudaStream_t st) {
   MixedState* m = h->mixed;
-  e1_ec_mixed_kernel<<<h->W, 1024, 0, st>>>(h->AhH, m->g32, h->X, h->minus, eloc, h->nk, h->M, h->n, m->Mp, h->G,
+  const int threads = std::max(2 * h->N * h->M, h->nk * h->G) >= 4096 ? 1024 : 256;   // a few terms per thread at least
+  e1_ec_mixed_kernel<<<h->W, threads, 0, st>>>(h->AhH, m->g32, h->X, h->minus, eloc, h->nk, h->M, h->n, m->Mp, h->G,
                                             m->WS);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
