@@ -13,6 +13,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <cmath>
 
 #include "attr.hpp"
@@ -497,12 +498,17 @@ __global__ void __launch_bounds__(GJB_THREADS)
 //      down), two barriers a pivot.  A pivot is a chain of about 250 dependent instructions
 //      (reciprocal, scaled row, update); several lanes per row keep the loop body short
 //      enough for the instruction cache (one lane with all eight entries took 3200 clocks a pivot);
-//   2. T - I (T the panel's accumulated transform) and the row moves go to every CTA of the cluster;
+//   2. T - I (T the panel's accumulated transform) goes to every CTA of the cluster through L2: each
+//      fetches it with all its threads, where the owner's 256 row threads storing it eight times into the
+//      others' shared memory lengthened the chain that everybody waits for (N = 256, 64 matrices:
+//      6.3 ms; 4.75 ms this way);
 //   3. each CTA moves the affected rows of its other columns and updates them,
-//      c += (T - I)[:, panel] c[panel rows]: a thread takes two rows of one column, consecutive
-//      threads consecutive columns, so that T is a broadcast.  INV: element by element the
-//      arithmetic of gjb_ff_kernel, so that both give the same bits; the log det alone, which is
-//      never rounded to a GEMM operand, uses biased accumulators (ff.cuh) of half the instructions.
+//      c += (T - I)[:, panel] c[panel rows]: a thread takes four rows of one column (Rows), consecutive
+//      threads consecutive columns, so that T is a broadcast and tmp is read once per four rows
+//      (2 / 4 rows: N = 256 4.75 / 4.65 ms, N = 108 459 / 451 us; N = 54 114 us with 2, 117 with 4; the
+//      log det alone runs out of registers at 4).  INV: element by element the arithmetic of gjb_ff_kernel, so
+//      that both give the same bits; the log det alone, which is never rounded to a GEMM operand,
+//      uses biased accumulators (ff.cuh) of half the instructions.
 // The INV update is N^3 complex multiply-adds of 48 FP32 instructions, the panels 8 N^2 of 60: 230 us
 // at 128 instructions per clock and SM for one matrix of N = 108 per SM.
 constexpr size_t GC_SMEM_LIMIT = 228000;   // dynamic, beside 3.4 KB of static
@@ -515,12 +521,11 @@ __host__ __device__ inline GcLayout gc_layout(int N, int C) {
   GcLayout L;
   L.nloc = C == 1 ? N : ((N + C - 1) / C + GJB - 1) / GJB * GJB;
   L.lda = L.nloc | 1;
-  const int tb = C == 1 ? 1 : 2;   // the next panel's owner writes T while this panel's is still read
   L.T = (size_t)N * L.lda * sizeof(float4);
-  L.tmp = L.T + (size_t)tb * N * GJB * sizeof(float4);
+  L.tmp = L.T + (size_t)N * GJB * sizeof(float4);
   L.piv = L.tmp + (size_t)GJB * L.nloc * sizeof(float4);
   L.rmax = L.piv + (size_t)L.nloc * sizeof(float4);
-  L.cs = L.rmax + (size_t)tb * N * sizeof(float);
+  L.cs = L.rmax + (size_t)N * sizeof(float);
   L.perm = L.cs + (size_t)L.nloc * sizeof(float);
   L.bytes = L.perm + (size_t)N * sizeof(int);
   return L;
@@ -538,6 +543,10 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     gjc_ff_kernel(float4* Sff, int N, int keep, zc* logdet, int* sing, int* flags, __half* out, int Np,
                   float* s_out) {
   namespace cg = cooperative_groups;
+  // rows of a column that a thread updates together; in the next panel's eight columns, which everybody
+  // waits for, two up to N = 128 (LPR 2), where four would leave half of the threads without any
+  using Rows = std::integral_constant<int, INV && GC_THREADS == 512 ? 4 : 2>;
+  using RowsNext = std::integral_constant<int, LPR == 1 ? Rows::value : 2>;
   constexpr int GC_WARPS = GC_THREADS / 32, SLOTS = GJB / LPR;   // a lane's entries: columns sub + LPR k
   extern __shared__ __align__(16) unsigned char gj_smem[];
   __shared__ GcPanel s_panel[2];
@@ -553,10 +562,10 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
   const GcLayout L = gc_layout(N, C);
   const int lda = L.lda, nloc = L.nloc, c0 = rank * nloc, nc = max(0, min(nloc, N - c0));
   float4* a = reinterpret_cast<float4*>(gj_smem);
-  float4* Tbuf = reinterpret_cast<float4*>(gj_smem + L.T);
+  float4* T = reinterpret_cast<float4*>(gj_smem + L.T);
   float4* tmp = reinterpret_cast<float4*>(gj_smem + L.tmp);
   float4* piv = reinterpret_cast<float4*>(gj_smem + L.piv);
-  float* rmaxbuf = reinterpret_cast<float*>(gj_smem + L.rmax);
+  float* rmax = reinterpret_cast<float*>(gj_smem + L.rmax);
   float* cs = reinterpret_cast<float*>(gj_smem + L.cs);
   int* perm = reinterpret_cast<int*>(gj_smem + L.perm);
   const float4* g = Sff + (size_t)b * N * N + c0;
@@ -566,7 +575,7 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       a[i * lda + c] = g[(size_t)i * N + c];
     }
   for (int i = tid; i < N; i += GC_THREADS) perm[i] = i;
-  int swaps = 0;   // thread 0's count
+  int swaps = 0;   // the last thread's count
   bool singular = false;
   // the panel's row threads: LPR lanes per row
   const int rows_threads = (N * LPR + 31) & ~31, row_warps = rows_threads >> 5;
@@ -670,80 +679,77 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       }
     }
   };
-  // ---- T - I (v) to every CTA of the cluster; for C > 1 the row moves and the verdict too
-  auto publish = [&](int par) {
-    const int i = ri;
-    if (!s_panel[par].singular && i < N) {
-      float m = 0.f;
-      if constexpr (!INV) {   // the row's largest multiplier, for the biased accumulators
+  // ---- T - I (v): into shared memory, or (C > 1) through the matrix's global copy, which nobody
+  // reads after the start: eight CTAs fetch it from L2 sooner than one can store it to all of them.  Two
+  // slots in turn; the row moves and the verdict go into the other CTAs' shared memory.
+  auto put_T = [&](float4* dst) {
+    if (ri < N) {
 #pragma unroll
-        for (int k = 0; k < SLOTS; ++k) m = fmaxf(m, fabsf(v[k].x) + fabsf(v[k].z));
-        const unsigned lanes = (LPR == 32 ? 0u : (1u << LPR)) - 1u;   // rows are whole groups of lanes
-#pragma unroll
-        for (int o = 1; o < LPR; o <<= 1) m = fmaxf(m, __shfl_xor_sync(lanes << group, m, o));
-      }
-#pragma unroll
-      for (int r = 0; r < C; ++r) {
-        float4* T = Tbuf + (size_t)par * N * GJB;
-        float* rm = rmaxbuf + (size_t)par * N;
-        if (C > 1) {
-          T = cg::this_cluster().map_shared_rank(T, r);
-          rm = cg::this_cluster().map_shared_rank(rm, r);
-        }
-#pragma unroll
-        for (int k = 0; k < SLOTS; ++k) T[i * GJB + sub + LPR * k] = v[k];
-        if (!INV && sub == 0) rm[i] = m;
-      }
+      for (int k = 0; k < SLOTS; ++k) dst[ri * GJB + sub + LPR * k] = v[k];
     }
-    if (C > 1 && tid < (int)(sizeof(GcPanel) / sizeof(int))) {
+  };
+  float4* Tg = Sff + (size_t)b * N * N;   // [2][N][GJB], C > 1 (N > 64, so it fits)
+  auto publish = [&](int par) {
+    if (!s_panel[par].singular) put_T(Tg + (size_t)par * N * GJB);
+    if (tid < (int)(sizeof(GcPanel) / sizeof(int))) {
       const int val = reinterpret_cast<const int*>(&s_panel[par])[tid];
       for (int r = 0; r < C; ++r)
         if (r != rank) reinterpret_cast<int*>(cg::this_cluster().map_shared_rank(&s_panel[par], r))[tid] = val;
     }
   };
-  // ---- 3. rows i0, i0 + 1 of local column c: += (T - I) tmp
-  auto update = [&](int j0, int par, int ip, int c) {
-    const int jb = min(GJB, N - j0), i0 = (INV ? 0 : j0 + jb) + 2 * ip;
-    const int i1 = min(i0 + 1, N - 1);   // an odd last row is done twice, stored once
-    const float4 a0 = a[i0 * lda + c], a1 = a[i1 * lda + c];
-    const float4* d0 = Tbuf + ((size_t)par * N + i0) * GJB;
-    const float4* d1 = Tbuf + ((size_t)par * N + i1) * GJB;
-    float4 v0, v1;
+  // ---- 3. rows i0 .. of local column c: += (T - I) tmp
+  auto update = [&](auto rows, int j0, int ip, int c) {
+    constexpr int GC_ROWS = decltype(rows)::value;
+    const int jb = min(GJB, N - j0), i0 = (INV ? 0 : j0 + jb) + GC_ROWS * ip;
+    float4 v[GC_ROWS];
+    const float4* d[GC_ROWS];   // rows past the last repeat it and are not stored
+#pragma unroll
+    for (int r = 0; r < GC_ROWS; ++r) {
+      const int i = min(i0 + r, N - 1);
+      v[r] = a[i * lda + c];
+      d[r] = T + i * GJB;
+    }
     if constexpr (INV) {
-      ffa::cacc x0 = ffa::cacc_from(a0), x1 = ffa::cacc_from(a1);
+      ffa::cacc x[GC_ROWS];
+#pragma unroll
+      for (int r = 0; r < GC_ROWS; ++r) x[r] = ffa::cacc_from(v[r]);
 #pragma unroll 4
       for (int l = 0; l < jb; ++l) {
         const float4 t = tmp[l * nloc + c];
-        ffa::cacc_fma(x0, d0[l], t);
-        ffa::cacc_fma(x1, d1[l], t);
+#pragma unroll
+        for (int r = 0; r < GC_ROWS; ++r) ffa::cacc_fma(x[r], d[r][l], t);
       }
-      v0 = ffa::cacc_get(x0);
-      v1 = ffa::cacc_get(x1);
+#pragma unroll
+      for (int r = 0; r < GC_ROWS; ++r) v[r] = ffa::cacc_get(x[r]);
     } else {
-      const float* rmax = rmaxbuf + (size_t)par * N;
       const float cc = cs[c];
-      // a hair more than the exact sums: rmax and cs are sums of rounded leading parts
-      const float B0 = ffa::bias_of(fmaf(rmax[i0] * cc, 1.001f, 1.001f * fmaxf(fabsf(a0.x), fabsf(a0.z))));
-      const float B1 = ffa::bias_of(fmaf(rmax[i1] * cc, 1.001f, 1.001f * fmaxf(fabsf(a1.x), fabsf(a1.z))));
-      ffa::bacc r0 = ffa::bacc_from(ffa::re(a0), B0), m0 = ffa::bacc_from(ffa::im(a0), B0);
-      ffa::bacc r1 = ffa::bacc_from(ffa::re(a1), B1), m1 = ffa::bacc_from(ffa::im(a1), B1);
+      float B[GC_ROWS];
+      ffa::bacc re[GC_ROWS], im[GC_ROWS];
+#pragma unroll
+      for (int r = 0; r < GC_ROWS; ++r) {
+        // a hair more than the exact sums: rmax and cs are sums of rounded leading parts
+        B[r] = ffa::bias_of(fmaf(rmax[min(i0 + r, N - 1)] * cc, 1.001f, 1.001f * fmaxf(fabsf(v[r].x), fabsf(v[r].z))));
+        re[r] = ffa::bacc_from(ffa::re(v[r]), B[r]);
+        im[r] = ffa::bacc_from(ffa::im(v[r]), B[r]);
+      }
 #pragma unroll 4
       for (int l = 0; l < GJB; ++l) {
-        const float4 t = tmp[l * nloc + c], x = d0[l], y = d1[l];
-        ffa::bacc_fma(r0, x.x, x.y, t.x, t.y);
-        ffa::bacc_fma(m0, x.x, x.y, t.z, t.w);
-        ffa::bacc_fma(r1, y.x, y.y, t.x, t.y);
-        ffa::bacc_fma(m1, y.x, y.y, t.z, t.w);
-        ffa::bacc_fma(r0, -x.z, -x.w, t.z, t.w);
-        ffa::bacc_fma(m0, x.z, x.w, t.x, t.y);
-        ffa::bacc_fma(r1, -y.z, -y.w, t.z, t.w);
-        ffa::bacc_fma(m1, y.z, y.w, t.x, t.y);
+        const float4 t = tmp[l * nloc + c];
+#pragma unroll
+        for (int r = 0; r < GC_ROWS; ++r) {
+          const float4 x = d[r][l];
+          ffa::bacc_fma(re[r], x.x, x.y, t.x, t.y);
+          ffa::bacc_fma(im[r], x.x, x.y, t.z, t.w);
+          ffa::bacc_fma(re[r], -x.z, -x.w, t.z, t.w);
+          ffa::bacc_fma(im[r], x.z, x.w, t.x, t.y);
+        }
       }
-      v0 = ffa::pack(ffa::bacc_get(r0, B0), ffa::bacc_get(m0, B0));
-      v1 = ffa::pack(ffa::bacc_get(r1, B1), ffa::bacc_get(m1, B1));
+#pragma unroll
+      for (int r = 0; r < GC_ROWS; ++r) v[r] = ffa::pack(ffa::bacc_get(re[r], B[r]), ffa::bacc_get(im[r], B[r]));
     }
-    a[i0 * lda + c] = v0;
-    if (i0 + 1 < N) a[(i0 + 1) * lda + c] = v1;
+#pragma unroll
+    for (int r = 0; r < GC_ROWS; ++r)
+      if (i0 + r < N) a[(i0 + r) * lda + c] = v[r];
   };
 
   if (rank == 0 && row_thread) {
@@ -752,31 +758,43 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     if (C > 1) publish(0);
   }
   for (int j0 = 0, pan = 0; j0 < N; j0 += GJB, ++pan) {
-    const int jb = min(GJB, N - j0), par = C == 1 ? 0 : (pan & 1);
+    const int jb = min(GJB, N - j0), par = pan & 1;
     const int owner = C == 1 ? 0 : j0 / nloc, jl = j0 - owner * nloc;   // the panel's first local column
-    if (C > 1) {
+    if (C > 1)
       cg::this_cluster().sync();
-    } else {
+    else
       __syncthreads();   // the previous panel's T has been read for the last time
-      if (row_thread) publish(0);
-      __syncthreads();
-    }
     if (s_panel[par].singular) {
       singular = true;
       break;
     }
-    if (tid == 0) {
-      s_next = 0;
-      for (int l = 0; l < jb; ++l) {
-        const int p = s_panel[par].prow[l];
-        if (p != j0 + l) {
-          const int t = perm[j0 + l];
-          perm[j0 + l] = perm[p];
-          perm[p] = t;
-          ++swaps;
+    // with every row's largest multiplier for the biased accumulators, a maximum over the row's lanes
+    if (C == 1) {
+      if (row_thread) {
+        put_T(T);
+        if (!INV) {
+          float m = 0.f;
+#pragma unroll
+          for (int k = 0; k < SLOTS; ++k) m = fmaxf(m, fabsf(v[k].x) + fabsf(v[k].z));
+#pragma unroll
+          for (int o = 1; o < LPR; o <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+          if (ri < N && sub == 0) rmax[ri] = m;
+        }
+      }
+    } else {
+      const float4* src = Tg + (size_t)par * N * GJB;
+      for (int e = tid; e - lane < N * GJB; e += GC_THREADS) {
+        const float4 t = e < N * GJB ? __ldcg(src + e) : ffa::czero();
+        if (e < N * GJB) T[e] = t;
+        if (!INV) {
+          float m = fabsf(t.x) + fabsf(t.z);
+#pragma unroll
+          for (int o = 1; o < GJB; o <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+          if (e < N * GJB && (e & (GJB - 1)) == 0) rmax[e / GJB] = m;
         }
       }
     }
+    if (tid == 0) s_next = 0;
     // ---- 2. the affected rows of the other columns (LU: those right of the panel): thread
     // (column, half), half 0 the panel's rows (also kept in tmp), half 1 the rows they displaced
     {
@@ -791,7 +809,7 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
         const bool need = has && l < jb && (!half || s_panel[par].prow[l] >= j0 + jb);
         x[l] = need ? a[src * lda + c] : ffa::czero();
       }
-      __syncthreads();
+      __syncthreads();   // T and rmax are complete too
       if (has && !half) {
         float m = 0.f;
 #pragma unroll
@@ -812,14 +830,14 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     // while the other warps update the rest, and join them.
     const int jn = j0 + GJB, jbn = min(GJB, N - jn);
     const int nowner = jn >= N ? -1 : (C == 1 ? 0 : jn / nloc), nl = jn - nowner * nloc;
-    const int np = (N - (INV ? 0 : j0 + jb) + 1) / 2;
+    const int below = N - (INV ? 0 : j0 + jb), np = (below + Rows::value - 1) / Rows::value;
     const bool mine = rank == nowner;
     if (mine) {
-      for (int u = tid; u < np * GJB; u += GC_THREADS)
-        if ((u & (GJB - 1)) < jbn) update(j0, par, u / GJB, nl + (u & (GJB - 1)));
+      for (int u = tid; u < (below + RowsNext::value - 1) / RowsNext::value * GJB; u += GC_THREADS)
+        if ((u & (GJB - 1)) < jbn) update(RowsNext(), j0, u / GJB, nl + (u & (GJB - 1)));
       __syncthreads();
       if (row_thread) {
-        const int parn = C == 1 ? 0 : ((pan + 1) & 1);
+        const int parn = par ^ 1;
         factor(jn, nl, parn);
         if (C > 1) {
           asm volatile("bar.sync 1, %0;" ::"r"(rows_threads) : "memory");
@@ -828,6 +846,17 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       }
       __syncwarp();
     }
+    if (tid == GC_THREADS - 1)   // beside the panel's factorisation
+      for (int l = 0; l < jb; ++l) {
+        const int p = s_panel[par].prow[l];
+        if (p != j0 + l) {
+          const int t = perm[j0 + l];
+          perm[j0 + l] = perm[p];
+          perm[p] = t;
+          ++swaps;
+        }
+      }
+    __syncwarp();
     // the rest: columns [first, nc) without [x0, x1)
     const int first = INV ? 0 : (rank < owner ? nc : (rank == owner ? jl + jb + (mine ? jbn : 0) : (mine ? jbn : 0)));
     const int x0 = !INV ? nc : (rank == owner ? jl : (mine ? nl : nc));
@@ -840,7 +869,7 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       if (u - lane >= total) break;
       if (u < total) {
         const int ip = u / R, c1 = first + u - ip * R;
-        update(j0, par, ip, c1 + (c1 >= x0 ? xn : 0));
+        update(Rows(), j0, ip, c1 + (c1 >= x0 ? xn : 0));
       }
       __syncwarp();
     }
@@ -886,7 +915,7 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       m = fmaxf(m, s_max[r]);
     }
   }
-  if (rank == 0 && tid == 0) {
+  if (rank == 0 && tid == GC_THREADS - 1) {
     if (singular) {
       logdet[b] = make_double2(-INFINITY, 0.0);
       sing[b] = 1;
