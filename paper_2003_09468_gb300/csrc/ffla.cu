@@ -100,34 +100,22 @@ __global__ void __launch_bounds__(OV_THREADS)
   if (tid == 0) atomicMax(mx + ws, static_cast<unsigned long long>(__double_as_longlong((double)m)));
 }
 
-// Gauss-Jordan elimination with partial (row) pivoting of one N x N matrix per CTA, in
-// place, in double-float.  Step j: pick the row p >= j with the largest |re| + |im| in
-// column j, swap rows j and p, then
-//   INV:  scale row j by 1/a_jj (a_jj itself becomes 1/a_jj) and eliminate column j
-//         from every other row (a_ij becomes -a_ij / a_jj): after N steps the array
-//         holds (P S)^-1, P the row permutation, so S^-1[:, perm[i]] = column i;
-//   !INV: eliminate below the diagonal only (LU), for the log-determinant alone.
-// Either way the pivots are the diagonal of U in P S = L U, so
+// log det of one N x N matrix per CTA, by an in-place LU factorisation with partial (row)
+// pivoting in double-float.  Step j: pick the row p >= j with the largest |re| + |im| in column j,
+// swap rows j and p, eliminate below the diagonal.  The pivots are the diagonal of U in P S = L U, so
 //   log det S = sum_j log a_jj + i pi (number of swaps mod 2).
 // A zero or non-finite pivot marks the matrix singular: logdet = (-inf, 0), sing = 1,
-// flags[0] counts it, and the inverse written is zero.
-// INV output: the split planes of S^-T, out[b][N][Np] (split.cuh) with scale s_out[b].
+// flags[0] counts it.
 // For matrices too large for the cluster form below; the matrix stays in global memory (L2).
-template <bool INV>
-__global__ void __launch_bounds__(GJ_THREADS)
-    gj_ff_kernel(float4* Sff, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out) {
+__global__ void __launch_bounds__(GJ_THREADS) gj_ff_kernel(float4* Sff, int N, zc* logdet, int* sing, int* flags) {
   extern __shared__ __align__(16) unsigned char gj_smem[];
   __shared__ int s_p, s_sing, s_swaps;
   __shared__ float4 s_pv, s_ajj;
   __shared__ double s_red[GJ_WARPS];
-  __shared__ float s_redf[GJ_WARPS];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float4* a = Sff + (size_t)b * N * N;
   float4* f = reinterpret_cast<float4*>(gj_smem);
   double2* piv = reinterpret_cast<double2*>(f + N);
-  int* perm = reinterpret_cast<int*>(piv + N);
-  int* iperm = perm + N;
-  for (int i = tid; i < N; i += GJ_THREADS) perm[i] = i;
   if (tid == 0) {
     s_sing = 0;
     s_swaps = 0;
@@ -160,9 +148,6 @@ __global__ void __launch_bounds__(GJ_THREADS)
         if (!(best > 0.f) || !isfinite(best)) {
           s_sing = 1;
         } else if (bi != j) {
-          const int t = perm[j];
-          perm[j] = perm[bi];
-          perm[bi] = t;
           ++s_swaps;
         }
       }
@@ -173,18 +158,11 @@ __global__ void __launch_bounds__(GJ_THREADS)
     const float4 pv = s_pv, ajj = s_ajj;
     const float4 inv = ffa::crecip(pv);
     if (tid == 0) piv[j] = make_double2(ffa::to_double(ffa::re(pv)), ffa::to_double(ffa::im(pv)));
-    // swap rows j and p (each thread owns whole columns), and, INV, scale row j
+    // swap rows j and p (each thread owns whole columns)
     for (int c = tid; c < N; c += GJ_THREADS) {
       const float4 tj = a[(size_t)j * N + c];
       const float4 tp = (p == j) ? tj : a[(size_t)p * N + c];
-      if (INV) {
-        if (c == j)
-          a[(size_t)j * N + c] = inv;
-        else
-          a[(size_t)j * N + c] = ffa::cmul(tp, inv);
-      } else {
-        a[(size_t)j * N + c] = tp;
-      }
+      a[(size_t)j * N + c] = tp;
       if (p != j) a[(size_t)p * N + c] = tj;
     }
     // multipliers: column j after the swap (rows j and p are the only ones moved)
@@ -194,29 +172,14 @@ __global__ void __launch_bounds__(GJ_THREADS)
         fi = ffa::czero();
       else
         fi = (i == p) ? ajj : a[(size_t)i * N + j];
-      if (!INV) fi = ffa::cmul(fi, inv);
-      f[i] = fi;
+      f[i] = ffa::cmul(fi, inv);
     }
     __syncthreads();
     const float4* aj = a + (size_t)j * N;
-    if (INV) {
-      for (int i = warp; i < N; i += GJ_WARPS) {
-        if (i == j) continue;
-        const float4 fi = f[i];
-        float4* ai = a + (size_t)i * N;
-        for (int c = lane; c < N; c += 32) {
-          if (c == j)
-            ai[c] = ffa::cneg(ffa::cmul(fi, inv));
-          else
-            ai[c] = ffa::cfms(ai[c], fi, aj[c]);
-        }
-      }
-    } else {
-      for (int i = j + 1 + warp; i < N; i += GJ_WARPS) {
-        const float4 fi = f[i];
-        float4* ai = a + (size_t)i * N;
-        for (int c = j + 1 + lane; c < N; c += 32) ai[c] = ffa::cfms(ai[c], fi, aj[c]);
-      }
+    for (int i = j + 1 + warp; i < N; i += GJ_WARPS) {
+      const float4 fi = f[i];
+      float4* ai = a + (size_t)i * N;
+      for (int c = j + 1 + lane; c < N; c += 32) ai[c] = ffa::cfms(ai[c], fi, aj[c]);
     }
     __syncthreads();
   }
@@ -242,31 +205,16 @@ __global__ void __launch_bounds__(GJ_THREADS)
       sing[b] = 0;
     }
   }
-  if (!INV) return;
-  __half* o = out + (size_t)b * 4 * N * Np;
-  if (singular) {
-    for (int e = tid; e < N * N; e += GJ_THREADS) mixed::put4f(o + mixed::sp_at(e / N, Np, e % N), 0.f, 0.f);
-    if (tid == 0) s_out[b] = 1.f;
-    return;
-  }
-  for (int c = tid; c < N; c += GJ_THREADS) iperm[perm[c]] = c;
-  float m = 0.f;
-  for (int e = tid; e < N * N; e += GJ_THREADS) {
-    const float4 v = a[e];
-    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.z)));
-  }
-  m = block_max_f(m, s_redf);   // its barriers also publish iperm
-  const float s = mixed::pow2_scale((double)m);
-  if (tid == 0) s_out[b] = s;
-  // out row i, column c = S^-T[i][c] = S^-1[c][i] = a[c][iperm[i]]
-  for (int e = tid; e < N * N; e += GJ_THREADS) {
-    const int i = e / N, c = e % N;
-    const float4 v = a[(size_t)c * N + iperm[i]];
-    mixed::put4f(o + mixed::sp_at(i, Np, c), v.x * s, v.z * s);
-  }
 }
 
-// Blocked form of the same Gauss-Jordan inverse.  Pivots are taken in panels of GJB columns:
+// The inverse of one matrix per CTA by Gauss-Jordan elimination with partial (row) pivoting, in place.
+// An unblocked step j picks and swaps rows as above, scales row j by 1/a_jj (a_jj itself becomes 1/a_jj)
+// and eliminates column j from every other row (a_ij becomes -a_ij / a_jj): after N steps the
+// array holds (P S)^-1, P the row permutation, so S^-1[:, perm[i]] = column i.  A singular matrix's
+// inverse is written as zero.  Output: the split planes of S^-T, out[b][N][Np] (split.cuh) with scale
+// s_out[b].
+//
+// Pivots are taken in panels of GJB columns:
 // within a panel every step updates only the panel's columns (all rows), so that afterwards
 // those columns hold the panel's accumulated transform T (T - I has non-zeros only there); every
 // other column c then receives the panel's row swaps and one rank-GJB update
@@ -277,7 +225,7 @@ constexpr int GJB = 8;
 static_assert(GJB == 8, "the panel's index arithmetic uses shifts by 3");
 constexpr int GJB_THREADS = 512;
 constexpr int GJB_WARPS = GJB_THREADS / 32;
-constexpr int GJB_GLOBAL_MAXN = 1024;   // GJB N float4 + per-row arrays within SMEM_LIMIT
+constexpr int GJB_GLOBAL_MAXN = 1024;   // a handle's largest N; GJB N float4 + per-row arrays are within SMEM_LIMIT
 
 // Pivot candidate key: larger |value| first, then the smaller row (m >= 0 and not NaN, so its
 // bits order as the values do).
@@ -1040,22 +988,16 @@ cudaError_t invert(float4* Sff, int WS, int N, zc* logdet, int* sing, int* flags
   if (ec != cudaErrorNotSupported) return ec;
   if (keep) return cudaErrorNotSupported;
   cudaError_t e;
-  if (out && N <= GJB_GLOBAL_MAXN) {
+  if (out) {
     const size_t bytes = (size_t)GJB * N * sizeof(float4) + gj_smem_bytes(N);
-    if (bytes <= SMEM_LIMIT) {
-      if ((e = set_smem(gjb_ff_kernel, bytes)) != cudaSuccess) return e;
-      gjb_ff_kernel<<<WS, GJB_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
-      return cudaGetLastError();
-    }
+    if (N > GJB_GLOBAL_MAXN || bytes > SMEM_LIMIT) return cudaErrorInvalidValue;
+    if ((e = set_smem(gjb_ff_kernel, bytes)) != cudaSuccess) return e;
+    gjb_ff_kernel<<<WS, GJB_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
+    return cudaGetLastError();
   }
   const size_t bytes = gj_smem_bytes(N);
-  if (out) {
-    if ((e = set_smem(gj_ff_kernel<true>, bytes)) != cudaSuccess) return e;
-    gj_ff_kernel<true><<<WS, GJ_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
-  } else {
-    if ((e = set_smem(gj_ff_kernel<false>, bytes)) != cudaSuccess) return e;
-    gj_ff_kernel<false><<<WS, GJ_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags, out, Np, s_out);
-  }
+  if ((e = set_smem(gj_ff_kernel, bytes)) != cudaSuccess) return e;
+  gj_ff_kernel<<<WS, GJ_THREADS, bytes, st>>>(Sff, N, logdet, sing, flags);
   return cudaGetLastError();
 }
 
