@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(OV_THREADS)
 //   log det S = sum_j log a_jj + i pi (number of swaps mod 2).
 // A zero or non-finite pivot marks the matrix singular: logdet = (-inf, 0), sing = 1,
 // flags[0] counts it.
-// For matrices too large for the cluster form below; the matrix stays in global memory (L2).
+// For matrices that the cluster form below does not take; the matrix stays in global memory (L2).
 __global__ void __launch_bounds__(GJ_THREADS) gj_ff_kernel(float4* Sff, int N, zc* logdet, int* sing, int* flags) {
   extern __shared__ __align__(16) unsigned char gj_smem[];
   __shared__ int s_p, s_sing, s_swaps;
@@ -942,18 +942,40 @@ int gjc_cluster(int WS, int N) {
   return C;
 }
 
+// Whether a cluster of C CTAs per matrix beats one CTA per matrix in the global form.  Of the clusters
+// only 76 / 36 / 15 (C = 2 / 4 / 8) run at once on 152 SMs, so many matrices take many waves; `gain` is
+// what one wave of the global form costs in waves of clusters (a little less beyond one wave, when its
+// CTAs no longer move in step).  Measured, cluster | global, ms:
+//   inverse  N = 256: 64 matrices 4.69 | 6.56, 128 8.43 | 7.06, 304 19.6 | 12.7, 512 32.7 | 24.1
+//            N = 160: 64 1.07 | 1.84, 128 2.13 | 1.85, 512 7.96 | 6.47;  N = 120: 128 0.77 | 0.89, 512 2.68 | 2.99
+//   log det  N = 256: 64 3.21 | 4.84, 128 5.78 | 6.98, 304 13.5 | 11.3, 512 22.4 | 20.1
+//            N = 160: 64 0.75 | 1.29, 128 1.49 | 1.28, 512 5.57 | 4.03;  N = 120: 128 0.47 | 0.49, 304 0.94 | 0.84
+bool cluster_pays(int WS, int C, bool inv, int sms) {
+  const int at_once = std::max(1, sms * (C == 8 ? 15 : C == 4 ? 36 : 76) / 152);
+  const int waves = (WS + at_once - 1) / at_once;
+  const double gain = C == 8 ? (inv ? 7.0 : 10.0) : C == 4 ? 3.45 : (inv ? 2.3 : 2.0);
+  return waves <= gain * (WS <= sms ? 1.0 : 0.97 * WS / sms);
+}
+
 // Small matrices take fewer threads, so that several share an SM (the panels are latency).
-// cudaErrorNotSupported: too large for this form.
+// cudaErrorNotSupported: too large for this form, or faster in the global one.
 template <bool INV>
 cudaError_t gjc_invert(const GjcArgs& g, cudaStream_t st) {
-  const int N = g.N, C = gjc_cluster(g.WS, N);
+  const int N = g.N;
+  int C = gjc_cluster(g.WS, N);
   if (C == 0) return cudaErrorNotSupported;
+  if (N > 128) C = C <= 4 ? 4 : 8;
+  int dev = 0, sms = 0;
+  if (C > 1 && !g.keep && cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+      !cluster_pays(g.WS, C, INV, sms))
+    return cudaErrorNotSupported;
   if (N <= 32) return gjc_launch<1, INV, 128, 4>(g, st);
   if (N <= 64) return gjc_launch<1, INV, 256, 2>(g, st);
   if (N <= 128) return C == 1   ? gjc_launch<1, INV, 512, 2>(g, st)
                        : C == 2 ? gjc_launch<2, INV, 512, 2>(g, st)
                                 : gjc_launch<4, INV, 512, 2>(g, st);
-  return C <= 4 ? gjc_launch<4, INV, 512, 1>(g, st) : gjc_launch<8, INV, 512, 1>(g, st);
+  return C == 4 ? gjc_launch<4, INV, 512, 1>(g, st) : gjc_launch<8, INV, 512, 1>(g, st);
 }
 
 }  // namespace

@@ -38,6 +38,8 @@ MIXED = {
     "N160": spec(8, 20, 21), "N165": spec(15, 11, 12), "N168": spec(12, 14, 15),
     "N256": spec(16, 16, 17), "N258": spec(43, 6, 7),
     "G401": spec(1, 2, 3, nchol=401),   # the adjoint takes 16 walkers per block, not 32
+    # more matrices than clusters of eight or four can take at once with profit: the global forms
+    "N256-many": spec(16, 16, 17, nw=64), "N160-many": spec(8, 20, 21, nw=64),
     # more matrices than SMs: no doubling of the CTAs per matrix
     "N66-many": spec(3, 22, 23, nw=90),
 }
