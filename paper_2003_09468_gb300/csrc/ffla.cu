@@ -442,28 +442,34 @@ __global__ void __launch_bounds__(GJB_THREADS)
 //   1. the CTA that owns the panel's columns eliminates them in registers, LPR lanes per row with
 //      8 / LPR of the row's entries each: per pivot a warp maximum and one more over the warps'
 //      candidates pick the row, the pivot row and the row it displaces go through shared memory,
-//      and every lane eliminates its own entries (INV: all rows, else the rows from the panel
-//      down), two barriers a pivot.  A pivot is a chain of about 250 dependent instructions
-//      (reciprocal, scaled row, update); several lanes per row keep the loop body short
-//      enough for the instruction cache (one lane with all eight entries took 3200 clocks a pivot);
-//   2. T - I (T the panel's accumulated transform) goes to every CTA of the cluster through L2: each
-//      fetches it with all its threads, where the owner's 256 row threads storing it eight times into the
-//      others' shared memory lengthened the chain that everybody waits for (N = 256, 64 matrices:
-//      6.3 ms; 4.75 ms this way);
-//   3. each CTA moves the affected rows of its other columns and updates them,
-//      c += (T - I)[:, panel] c[panel rows]: a thread takes four rows of one column (Rows), consecutive
-//      threads consecutive columns, so that T is a broadcast and tmp is read once per four rows
-//      (2 / 4 rows: N = 256 4.75 / 4.65 ms, N = 108 459 / 451 us; N = 54 114 us with 2, 117 with 4; the
-//      log det alone runs out of registers at 4).  INV: element by element the arithmetic of gjb_ff_kernel, so
-//      that both give the same bits; the log det alone, which is never rounded to a GEMM operand,
-//      uses biased accumulators (ff.cuh) of half the instructions.
+//      and every lane eliminates its own entries (INV: all rows by Gauss-Jordan; else the rows below the
+//      pivot, whose multipliers stay in the eliminated column), two barriers a pivot.  A pivot is a
+//      chain of about 250 dependent instructions (reciprocal, scaled row, update); several lanes per row
+//      keep the loop body short enough for the instruction cache (one lane with all eight entries took 3200
+//      clocks a pivot);
+//   2. T - I (INV: T the panel's accumulated transform; else the multipliers, L) goes to every CTA of the
+//      cluster through L2: each fetches it with all its threads, where the owner's 256 row threads storing
+//      it eight times into the others' shared memory lengthened the chain that everybody waits for (N = 256,
+//      64 matrices: 6.3 ms; 4.75 ms this way);
+//   3. each CTA moves the affected rows of its other columns (the log det also solves the panel's 8 x 8
+//      triangle for its rows of U, a column per thread) and updates the rest, c += (T - I)[:, panel]
+//      c[panel rows]: a thread takes four rows of one column (Rows), consecutive threads consecutive
+//      columns, so that T is a broadcast and tmp is read once per four rows (2 / 4 rows: inverse N = 256
+//      4.75 / 4.65 ms, N = 108 459 / 451 us; N = 54 114 us with 2, 117 with 4; the log det is faster with
+//      two: N = 256 3.19 / 3.32 ms, N = 108 267 / 269 us).
+// Both are element by element, in one order, the arithmetic of the global form: INV that of gjb_ff_kernel, the
+// log det that of gj_ff_kernel (one normalised multiply-add per pivot), so that both forms give the same
+// bits, whichever the number of matrices selects.  (Biased accumulators, with an error of 2^-47 of a row
+// maximum times a column sum instead of 2^-48 of the terms, took 217 us for the log det at N = 108 where
+// these take 267, and lost one to two decimal digits on walkers near the trial, three on rows graded over six
+// decades: 1e-13 became 1e-10.)
 // The INV update is N^3 complex multiply-adds of 48 FP32 instructions, the panels 8 N^2 of 60: 230 us
-// at 128 instructions per clock and SM for one matrix of N = 108 per SM.
+// at 128 instructions per clock and SM for one matrix of N = 108 per SM; the log det N^3 / 3 of 60, 95 us.
 constexpr size_t GC_SMEM_LIMIT = 228000;   // dynamic, beside 3.4 KB of static
 
 struct GcLayout {
   int nloc, lda;   // columns per CTA (a multiple of GJB for C > 1), row stride in float4 (odd: columns and rows both conflict-free)
-  size_t T, tmp, piv, rmax, cs, perm, bytes;   // byte offsets
+  size_t T, tmp, piv, perm, bytes;   // byte offsets
 };
 __host__ __device__ inline GcLayout gc_layout(int N, int C) {
   GcLayout L;
@@ -472,9 +478,7 @@ __host__ __device__ inline GcLayout gc_layout(int N, int C) {
   L.T = (size_t)N * L.lda * sizeof(float4);
   L.tmp = L.T + (size_t)N * GJB * sizeof(float4);
   L.piv = L.tmp + (size_t)GJB * L.nloc * sizeof(float4);
-  L.rmax = L.piv + (size_t)L.nloc * sizeof(float4);
-  L.cs = L.rmax + (size_t)N * sizeof(float);
-  L.perm = L.cs + (size_t)L.nloc * sizeof(float);
+  L.perm = L.piv + (size_t)L.nloc * sizeof(float4);
   L.bytes = L.perm + (size_t)N * sizeof(int);
   return L;
 }
@@ -513,8 +517,6 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
   float4* T = reinterpret_cast<float4*>(gj_smem + L.T);
   float4* tmp = reinterpret_cast<float4*>(gj_smem + L.tmp);
   float4* piv = reinterpret_cast<float4*>(gj_smem + L.piv);
-  float* rmax = reinterpret_cast<float*>(gj_smem + L.rmax);
-  float* cs = reinterpret_cast<float*>(gj_smem + L.cs);
   int* perm = reinterpret_cast<int*>(gj_smem + L.perm);
   const float4* g = Sff + (size_t)b * N * N + c0;
   if (nc > 0)
@@ -579,16 +581,22 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       }
       if (tid == 0) s_panel[par].prow[jj] = p;
       asm volatile("bar.sync 1, %0;" ::"r"(rows_threads) : "memory");
-      // every warp scales the pivot row for itself, one entry per lane
       const float4 inv = ffa::crecip(s_prow[q][jj]);
-      if (lane < GJB) s_scaled[warp][lane] = lane == jj ? inv : ffa::cmul(s_prow[q][lane], inv);
+      // INV: every warp scales the pivot row for itself, one entry per lane
+      if (INV && lane < GJB) s_scaled[warp][lane] = lane == jj ? inv : ffa::cmul(s_prow[q][lane], inv);
       if (p != j) {   // rows j and p trade places
         if (i == p) {
 #pragma unroll
           for (int k = 0; k < SLOTS; ++k) v[k] = s_jrow[q][sub + LPR * k];
           orig = s_jorig[q];
         }
-        if (i == j) orig = s_porig[q];
+        if (i == j) {
+          orig = s_porig[q];
+          if (!INV) {   // its multipliers move with it (INV: the scaled row, below)
+#pragma unroll
+            for (int k = 0; k < SLOTS; ++k) v[k] = s_prow[q][sub + LPR * k];
+          }
+        }
       }
       vj = v[0];
 #pragma unroll
@@ -599,26 +607,41 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       if (LPR > 1)
         f = make_float4(__shfl_sync(FULL, vj.x, from), __shfl_sync(FULL, vj.y, from), __shfl_sync(FULL, vj.z, from),
                         __shfl_sync(FULL, vj.w, from));
-      __syncwarp();
-      // row i -= f (row j / pivot); column j, whose entry of the scaled row is 1 / pivot, starts
-      // from zero (bit for bit -(f / pivot)), and the pivot row becomes the scaled row
+      if constexpr (INV) {
+        __syncwarp();
+        // row i -= f (row j / pivot); column j, whose entry of the scaled row is 1 / pivot, starts
+        // from zero (bit for bit -(f / pivot)), and the pivot row becomes the scaled row
 #pragma unroll
-      for (int k = 0; k < SLOTS; ++k) {
-        const float4 t = s_scaled[warp][sub + LPR * k];
-        const float4 from0 = (holds && slot == k) ? ffa::czero() : v[k];
-        const float4 e = ffa::cfms(from0, f, t);
-        v[k] = i == j ? t : e;
+        for (int k = 0; k < SLOTS; ++k) {
+          const float4 t = s_scaled[warp][sub + LPR * k];
+          const float4 from0 = (holds && slot == k) ? ffa::czero() : v[k];
+          const float4 e = ffa::cfms(from0, f, t);
+          v[k] = i == j ? t : e;
+        }
+        __syncwarp();
+      } else if (i > j) {
+        // row i -= (f / pivot) row j; the multiplier takes the place of the entry it eliminates
+        const float4 mult = ffa::cmul(f, inv);
+#pragma unroll
+        for (int k = 0; k < SLOTS; ++k) {
+          const int l = sub + LPR * k;
+          if (l > jj) v[k] = ffa::cfms(v[k], mult, s_prow[q][l]);
+          if (l == jj) v[k] = mult;
+        }
       }
-      __syncwarp();
     }
     if (tid == 0) s_panel[par].singular = bad;
     if (!bad && i < N) {
 #pragma unroll
       for (int k = 0; k < SLOTS; ++k) {
         const int l = sub + LPR * k;
-        if (active && l < jb) a[i * lda + jl + l] = v[k];
-        if (l >= jb || !active) v[k] = ffa::czero();
-        else if (i == j0 + l) v[k] = ffa::pack(ffa::add(ffa::re(v[k]), ffa::make(-1.f, 0.f)), ffa::im(v[k]));
+        if constexpr (INV) {
+          if (l < jb) a[i * lda + jl + l] = v[k];
+          if (l >= jb) v[k] = ffa::czero();
+          else if (i == j0 + l) v[k] = ffa::pack(ffa::add(ffa::re(v[k]), ffa::make(-1.f, 0.f)), ffa::im(v[k]));
+        } else if (l >= jb || i <= j0 + l) {   // rows above the panel (i < j0) among them
+          v[k] = ffa::czero();
+        }
       }
       if (sub == 0) {
         if (i >= j0 && i < j0 + jb) s_panel[par].srcp[i - j0] = orig;
@@ -670,30 +693,12 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
 #pragma unroll
       for (int r = 0; r < GC_ROWS; ++r) v[r] = ffa::cacc_get(x[r]);
     } else {
-      const float cc = cs[c];
-      float B[GC_ROWS];
-      ffa::bacc re[GC_ROWS], im[GC_ROWS];
-#pragma unroll
-      for (int r = 0; r < GC_ROWS; ++r) {
-        // a hair more than the exact sums: rmax and cs are sums of rounded leading parts
-        B[r] = ffa::bias_of(fmaf(rmax[min(i0 + r, N - 1)] * cc, 1.001f, 1.001f * fmaxf(fabsf(v[r].x), fabsf(v[r].z))));
-        re[r] = ffa::bacc_from(ffa::re(v[r]), B[r]);
-        im[r] = ffa::bacc_from(ffa::im(v[r]), B[r]);
-      }
 #pragma unroll 4
       for (int l = 0; l < GJB; ++l) {
         const float4 t = tmp[l * nloc + c];
 #pragma unroll
-        for (int r = 0; r < GC_ROWS; ++r) {
-          const float4 x = d[r][l];
-          ffa::bacc_fma(re[r], x.x, x.y, t.x, t.y);
-          ffa::bacc_fma(im[r], x.x, x.y, t.z, t.w);
-          ffa::bacc_fma(re[r], -x.z, -x.w, t.z, t.w);
-          ffa::bacc_fma(im[r], x.z, x.w, t.x, t.y);
-        }
+        for (int r = 0; r < GC_ROWS; ++r) v[r] = ffa::cfms(v[r], d[r][l], t);
       }
-#pragma unroll
-      for (int r = 0; r < GC_ROWS; ++r) v[r] = ffa::pack(ffa::bacc_get(re[r], B[r]), ffa::bacc_get(im[r], B[r]));
     }
 #pragma unroll
     for (int r = 0; r < GC_ROWS; ++r)
@@ -716,31 +721,11 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       singular = true;
       break;
     }
-    // with every row's largest multiplier for the biased accumulators, a maximum over the row's lanes
     if (C == 1) {
-      if (row_thread) {
-        put_T(T);
-        if (!INV) {
-          float m = 0.f;
-#pragma unroll
-          for (int k = 0; k < SLOTS; ++k) m = fmaxf(m, fabsf(v[k].x) + fabsf(v[k].z));
-#pragma unroll
-          for (int o = 1; o < LPR; o <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
-          if (ri < N && sub == 0) rmax[ri] = m;
-        }
-      }
+      if (row_thread) put_T(T);
     } else {
       const float4* src = Tg + (size_t)par * N * GJB;
-      for (int e = tid; e - lane < N * GJB; e += GC_THREADS) {
-        const float4 t = e < N * GJB ? __ldcg(src + e) : ffa::czero();
-        if (e < N * GJB) T[e] = t;
-        if (!INV) {
-          float m = fabsf(t.x) + fabsf(t.z);
-#pragma unroll
-          for (int o = 1; o < GJB; o <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
-          if (e < N * GJB && (e & (GJB - 1)) == 0) rmax[e / GJB] = m;
-        }
-      }
+      for (int e = tid; e < N * GJB; e += GC_THREADS) T[e] = __ldcg(src + e);
     }
     if (tid == 0) s_next = 0;
     // ---- 2. the affected rows of the other columns (LU: those right of the panel): thread
@@ -748,7 +733,8 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     {
       const int first = INV ? 0 : (rank < owner ? nc : (rank == owner ? jl + jb : 0));
       const int x0 = INV && rank == owner ? jl : nc, own = INV && rank == owner ? jb : 0;
-      const int c1 = first + (tid >> 1), c = c1 + (c1 >= x0 ? own : 0), half = tid & 1;
+      const int half = INV ? tid & 1 : tid / (GC_THREADS / 2), c1 = first + (INV ? tid >> 1 : tid % (GC_THREADS / 2));
+      const int c = c1 + (c1 >= x0 ? own : 0);
       const bool has = c < nc;
       float4 x[GJB];
 #pragma unroll
@@ -757,16 +743,20 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
         const bool need = has && l < jb && (!half || s_panel[par].prow[l] >= j0 + jb);
         x[l] = need ? a[src * lda + c] : ffa::czero();
       }
-      __syncthreads();   // T and rmax are complete too
+      __syncthreads();   // T is complete too
       if (has && !half) {
-        float m = 0.f;
+        if (!INV) {   // the panel's rows of U (jb = GJB: only the last panel is narrower, and no column is right of it)
+#pragma unroll
+          for (int l = 0; l < GJB; ++l)
+#pragma unroll
+            for (int i = 1; i < GJB; ++i)
+              if (i > l) x[i] = ffa::cfms(x[i], T[(j0 + i) * GJB + l], x[l]);
+        }
 #pragma unroll
         for (int l = 0; l < GJB; ++l) {
           tmp[l * nloc + c] = x[l];
-          if (l < jb) a[(j0 + l) * lda + c] = x[l];
-          m += fmaxf(fabsf(x[l].x), fabsf(x[l].z));
+          if (INV && l < jb) a[(j0 + l) * lda + c] = x[l];
         }
-        cs[c] = m;
       } else if (has) {
 #pragma unroll
         for (int l = 0; l < GJB; ++l)
@@ -948,12 +938,12 @@ int gjc_cluster(int WS, int N) {
 // CTAs no longer move in step).  Measured, cluster | global, ms:
 //   inverse  N = 256: 64 matrices 4.69 | 6.56, 128 8.43 | 7.06, 304 19.6 | 12.7, 512 32.7 | 24.1
 //            N = 160: 64 1.07 | 1.84, 128 2.13 | 1.85, 512 7.96 | 6.47;  N = 120: 128 0.77 | 0.89, 512 2.68 | 2.99
-//   log det  N = 256: 64 3.21 | 4.84, 128 5.78 | 6.98, 304 13.5 | 11.3, 512 22.4 | 20.1
-//            N = 160: 64 0.75 | 1.29, 128 1.49 | 1.28, 512 5.57 | 4.03;  N = 120: 128 0.47 | 0.49, 304 0.94 | 0.84
+//   log det  N = 256: 64 3.19 | 4.81, 128 5.75 | 7.09, 304 13.4 | 11.4, 512 22.3 | 20.4
+//            N = 160: 64 0.71 | 1.30, 128 1.40 | 1.29, 512 5.22 | 4.04;  N = 120: 64 0.26 | 0.48, 128 0.50 | 0.48
 bool cluster_pays(int WS, int C, bool inv, int sms) {
   const int at_once = std::max(1, sms * (C == 8 ? 15 : C == 4 ? 36 : 76) / 152);
   const int waves = (WS + at_once - 1) / at_once;
-  const double gain = C == 8 ? (inv ? 7.0 : 10.0) : C == 4 ? 3.45 : (inv ? 2.3 : 2.0);
+  const double gain = C == 8 ? (inv ? 7.0 : 10.0) : C == 4 ? 3.45 : (inv ? 2.3 : 1.9);
   return waves <= gain * (WS <= sms ? 1.0 : 0.97 * WS / sms);
 }
 

@@ -1,0 +1,93 @@
+"""The log det of the mixed path at the precision of its arithmetic (double-float, 48 bits).
+
+The reference is the FP64 log det of the walker that the call returned, so that nothing of the
+22-bit split GEMMs enters.  An error dS of the overlap and its factorisation moves log det S by
+tr(S^-1 dS), so the bar is
+  u sum_ij |S^-1|_ji (|A^dag| |phi| + P |L| |U|)_ij,  S = P L U.
+Each entry of dS gathers up to M products and up to N updates whose roundings are at most 2^-47 of
+the terms and about 2^-49 in the mean; they differ in sign from entry to entry, so that the sum
+of absolute values over all N^2 entries outweighs their number: u = 2^-48.  The inverse's elimination
+(the log det of a step with energies) forms the panels' transforms explicitly, one rounding more per
+update: u = 2^-47.
+
+Walkers: near the trial; random (row exchanges in every panel); random with the occupied rows
+graded over six decades, where M >= 2 nocc keeps the walker's columns independent (orthonormalise only:
+one propagation from there overflows).
+"""
+import numpy as np
+import pytest
+import scipy.linalg
+
+import gen
+
+torch = pytest.importorskip("torch")
+from gpu_util import dev, host, make, wrap_phase  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def spec(grid, nocc, M, nw=2):
+    return gen.SystemSpec(grid=grid, M=M, nocc=nocc, nchol=2, nwalkers=nw, dt=0.01, seed=1)
+
+
+# one CTA per matrix with four, two and two lanes per row; two, four and eight CTAs
+SIZES = {"N16": ((2, 2, 2), 2, 4), "N27": ((3, 3, 3), 1, 2), "N48": ((2, 2, 3), 4, 8), "N65": ((5, 1, 1), 13, 15),
+         "N108": ((3, 3, 3), 4, 8), "N128": ((4, 4, 1), 8, 16), "N120": ((4, 2, 1), 15, 16), "N160": ((4, 4, 1), 10, 11),
+         "N256": ((4, 4, 1), 16, 17)}
+
+
+def walkers(sp, kind):
+    """Two walkers."""
+    if kind == "near":
+        return gen.near_trial_walkers(sp, 2)
+    phi = gen.walkers(sp, 2)
+    if kind == "graded":   # the trial is the first nocc orbitals of every k: row (k, a) of S is row (k, a) of phi
+        grade = 10.0 ** (-6.0 * np.random.default_rng(3).permutation(sp.N) / (sp.N - 1))
+        phi.reshape(2, 2, sp.nk, sp.M, sp.N)[:, :, :, :sp.nocc] *= grade.reshape(sp.nk, sp.nocc)[..., None]
+    return phi
+
+
+def calls(sys_, phis, kind):
+    """{call: (walkers it returned, their log det)}"""
+    sp_w = phis.shape[0]
+    x = torch.zeros(sys_.field_shape, dtype=torch.float64, device="cuda")
+    out = {}
+    for call in ("orthonormalise",) if kind == "graded" else ("orthonormalise", "propagate", "step"):
+        phi, w = dev(phis), torch.ones(sp_w, dtype=torch.float64, device="cuda")
+        ld = torch.empty((sp_w, 2), dtype=torch.complex128, device="cuda")
+        if call == "orthonormalise":
+            sys_.orthonormalise(phi, ld)
+        elif call == "propagate":
+            sys_.propagate(phi, x, w, logdet=ld)
+        else:
+            sys_.step(phi, x, w, logdet=ld, reuse=False)
+        out[call] = host(phi), host(ld)
+    return out
+
+
+def reference(Ad, phi):
+    """(log det A^dag phi, the bar's sum)"""
+    S = Ad.conj().T @ phi
+    P, L, U = scipy.linalg.lu(S)
+    terms = np.abs(Ad).T @ np.abs(phi) + P @ (np.abs(L) @ np.abs(U))
+    sign, mag = np.linalg.slogdet(S)
+    return mag + 1j * np.angle(sign), np.sum(np.abs(np.linalg.inv(S)).T * terms)
+
+
+@pytest.mark.parametrize("kind", ["near", "random", "graded"])
+@pytest.mark.parametrize("name", list(SIZES))
+def test_log_det(name, kind):
+    sp = spec(*SIZES[name])
+    if kind == "graded" and sp.M < 2 * sp.nocc:
+        pytest.skip("the graded rows leave fewer rows than columns")
+    sys_, osys = make(sp, "mixed")
+    Ad = osys.A_dense()
+    for call, (phi, ld) in calls(sys_, walkers(sp, kind), kind).items():
+        u = 2.0 ** (-47 if call == "step" else -48)
+        for w in range(2):
+            for s in range(2):
+                ref, bar = reference(Ad, phi[w, s])
+                d = ld[w, s] - ref
+                assert max(abs(d.real), abs(wrap_phase(d.imag))) < u * bar, (call, w, s, d, u * bar)
+    assert sys_.last_error() == (0, 0)
+    sys_.close()
