@@ -456,12 +456,12 @@ __global__ void __launch_bounds__(GJB_THREADS)
 //      c[panel rows]: a thread takes four rows of one column (Rows), consecutive threads consecutive
 //      columns, so that T is a broadcast and tmp is read once per four rows (2 / 4 rows: inverse N = 256
 //      4.75 / 4.65 ms, N = 108 459 / 451 us; N = 54 114 us with 2, 117 with 4; the log det is faster with
-//      two: N = 256 3.19 / 3.32 ms, N = 108 267 / 269 us).
+//      two: N = 256 3.19 / 3.32 ms, N = 108 261 / 263 us).
 // Both are element by element, in one order, the arithmetic of the global form: INV that of gjb_ff_kernel, the
 // log det that of gj_ff_kernel (one normalised multiply-add per pivot), so that both forms give the same
 // bits, whichever the number of matrices selects.  (Biased accumulators, with an error of 2^-47 of a row
 // maximum times a column sum instead of 2^-48 of the terms, took 217 us for the log det at N = 108 where
-// these take 267, and lost one to two decimal digits on walkers near the trial, three on rows graded over six
+// these take 261, and lost one to two decimal digits on walkers near the trial, three on rows graded over six
 // decades: 1e-13 became 1e-10.)
 // The INV update is N^3 complex multiply-adds of 48 FP32 instructions, the panels 8 N^2 of 60: 230 us
 // at 128 instructions per clock and SM for one matrix of N = 108 per SM; the log det N^3 / 3 of 60, 95 us.
@@ -505,9 +505,8 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
   __shared__ uint2 s_cand[2][GC_WARPS];   // a warp's pivot candidate: |value| bits, row
   __shared__ float4 s_prow[2][GJB], s_jrow[2][GJB], s_scaled[GC_WARPS][GJB];
   __shared__ int s_porig[2], s_jorig[2], s_next;
-  __shared__ double s_red[GC_WARPS];
+  __shared__ double2 s_red[GC_WARPS];
   __shared__ float s_redf[GC_WARPS];
-  __shared__ double s_ld[8][2];
   __shared__ float s_max[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = C == 1 ? 0 : (int)(blockIdx.x % C), b = blockIdx.x / C;
@@ -813,21 +812,20 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     }
   }
   __syncthreads();
-  // ---- log det from the pivots (each CTA its own columns'): the logarithms on one half of the threads,
-  // the arguments on the other, so that the two long FP64 sequences run side by side
-  double lg = 0.0, an = 0.0;
-  if (!singular) {
-    constexpr int HALF = GC_THREADS / 2;
-    for (int c = tid % HALF; c < nc; c += HALF) {
+  // ---- log det from the pivots: each CTA the logarithms (one half of its threads) and the arguments (the
+  // other, so that the two long FP64 sequences run side by side) of its own columns' pivots, in their place
+  if (!singular) {   // the same in every thread of the cluster
+    constexpr int HALF = GC_THREADS / 2;   // at least a CTA's columns
+    const int c = tid % HALF;
+    double z = 0.0;
+    if (c < nc) {
       const double2 v = make_double2(ffa::to_double(ffa::re(piv[c])), ffa::to_double(ffa::im(piv[c])));
-      if (tid < HALF)
-        lg += 0.5 * log(v.x * v.x + v.y * v.y);
-      else
-        an += atan2(v.y, v.x);
+      z = tid < HALF ? 0.5 * log(v.x * v.x + v.y * v.y) : atan2(v.y, v.x);
     }
+    __syncthreads();
+    if (c < nc) reinterpret_cast<double*>(piv + c)[tid / HALF] = z;
+    __syncthreads();
   }
-  lg = block_sum_d(lg, s_red);
-  an = block_sum_d(an, s_red);
   float m = 0.f;
   if (INV && !singular) {
     for (int e = tid; e < N * nc; e += GC_THREADS) {
@@ -838,19 +836,32 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     m = block_max_f(m, s_redf);
   }
   if (C > 1) {
-    if (tid < C) {
-      double(*ld)[2] = cg::this_cluster().map_shared_rank(s_ld, tid);
-      ld[rank][0] = lg;
-      ld[rank][1] = an;
-      cg::this_cluster().map_shared_rank(s_max, tid)[rank] = m;
-    }
+    if (tid < C) cg::this_cluster().map_shared_rank(s_max, tid)[rank] = m;
     cg::this_cluster().sync();
-    lg = an = 0.0;
     m = 0.f;
-    for (int r = 0; r < C; ++r) {
-      lg += s_ld[r][0];
-      an += s_ld[r][1];
-      m = fmaxf(m, s_max[r]);
+    for (int r = 0; r < C; ++r) m = fmaxf(m, s_max[r]);
+  }
+  // Summed by the first CTA, 32 pivots per warp, then the warps in order: the order depends on N alone, so that
+  // neither the size of the cluster nor the choice of the global form (block_sum_d) shows in the result.
+  double lg = 0.0, an = 0.0;
+  if (rank == 0 && !singular) {
+    if (tid < ((N + 31) & ~31)) {
+      double2 z = make_double2(0.0, 0.0);
+      if (tid < N) {
+        const float4* pr = piv;
+        if (C > 1) pr = cg::this_cluster().map_shared_rank(piv, tid / nloc);
+        z = reinterpret_cast<const double2*>(pr)[C > 1 ? tid % nloc : tid];
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        z.x += __shfl_xor_sync(FULL, z.x, o);
+        z.y += __shfl_xor_sync(FULL, z.y, o);
+      }
+      if (lane == 0) s_red[warp] = z;
+    }
+    __syncthreads();
+    for (int w = 0; w < (N + 31) / 32; ++w) {
+      lg += s_red[w].x;
+      an += s_red[w].y;
     }
   }
   if (rank == 0 && tid == GC_THREADS - 1) {
@@ -864,6 +875,7 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
       sing[b] = 0;
     }
   }
+  if (C > 1 && !INV) cg::this_cluster().sync();   // the first CTA has read the others' pivots
   if (!INV) return;
   __half* o = out + (size_t)b * 4 * N * Np;
   const float sc = singular ? 1.f : mixed::pow2_scale((double)m);
@@ -876,6 +888,7 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     mixed::put4f(o + mixed::sp_at(i, Np, r), v.x * sc, v.z * sc);
     if (keep) Sff[(size_t)b * N * N + (size_t)r * N + i] = v;   // every CTA read its columns before the first panel
   }
+  if (C > 1) cg::this_cluster().sync();
 }
 
 template <class K>
@@ -936,8 +949,8 @@ int gjc_cluster(int WS, int N) {
 // only 76 / 36 / 15 (C = 2 / 4 / 8) run at once on 152 SMs, so many matrices take many waves; `gain` is
 // what one wave of the global form costs in waves of clusters (a little less beyond one wave, when its
 // CTAs no longer move in step).  Measured, cluster | global, ms:
-//   inverse  N = 256: 64 matrices 4.69 | 6.56, 128 8.43 | 7.06, 304 19.6 | 12.7, 512 32.7 | 24.1
-//            N = 160: 64 1.07 | 1.84, 128 2.13 | 1.85, 512 7.96 | 6.47;  N = 120: 128 0.77 | 0.89, 512 2.68 | 2.99
+//   inverse  N = 256: 64 matrices 4.63 | 6.55, 128 8.33 | 7.08, 304 19.4 | 12.7, 512 32.3 | 24.2
+//            N = 160: 64 1.05 | 1.84, 128 2.09 | 1.85, 512 7.80 | 6.46;  N = 120: 128 0.73 | 0.89, 512 2.58 | 2.99
 //   log det  N = 256: 64 3.19 | 4.81, 128 5.75 | 7.09, 304 13.4 | 11.4, 512 22.3 | 20.4
 //            N = 160: 64 0.71 | 1.30, 128 1.40 | 1.29, 512 5.22 | 4.04;  N = 120: 64 0.26 | 0.48, 128 0.50 | 0.48
 bool cluster_pays(int WS, int C, bool inv, int sms) {

@@ -91,3 +91,23 @@ def test_log_det(name, kind):
                 assert max(abs(d.real), abs(wrap_phase(d.imag))) < u * bar, (call, w, s, d, u * bar)
     assert sys_.last_error() == (0, 0)
     sys_.close()
+
+
+# both sides of the choice between clusters and the global form, and clusters of different sizes
+BATCH = {"N27": 64, "N108": 64, "N120": 152, "N160": 64, "N256": 64}
+
+
+@pytest.mark.parametrize("name", list(BATCH))
+def test_log_det_does_not_depend_on_the_batch(name):
+    """A walker's log det has the same bits alone (two walkers) and among many (of the sizes at which the force
+    bias, whose k blocks are grouped by the number of tiles, returns the same walkers)."""
+    got = []
+    for nw in (2, BATCH[name]):
+        sp = spec(*SIZES[name], nw=nw)
+        sys_, _ = make(sp, "mixed")
+        phis = np.concatenate([walkers(sp, "random")] * (nw // 2))
+        got.append({call: (phi[:2], ld[:2]) for call, (phi, ld) in calls(sys_, phis, "random").items()})
+        sys_.close()
+    for call in got[0]:
+        assert np.array_equal(got[0][call][0], got[1][call][0]), call
+        assert np.array_equal(got[0][call][1], got[1][call][1]), call
