@@ -1,7 +1,7 @@
-// The adjoint's dense parts on the tensor-core path: dE/dGh from its three pieces, the
-// projection through S^-1 and the walker, and dE/dh.  Everything here carries at least 40 bits
-// (double-float, ff.cuh): the projection multiplies by S^-1, whose condition number would eat the
-// 22 bits of the split GEMMs.
+// The adjoint's dense parts on the tensor-core path: dE/dGh from its three pieces (the Coulomb sum in
+// fp32, the exchange from the split GEMM's 22 bits), the projection through S^-1 and the walker, and
+// dE/dh.  The projection and dE/dh are in double-float (ff.cuh, 48 bits): they multiply by S^-1, whose
+// condition number would eat the 22 bits of the split GEMMs.
 #include <algorithm>
 
 #include "adjoint.hpp"
@@ -27,18 +27,18 @@ __global__ void to_ff_kernel(const zc* in, float4* out, size_t n) {
 // C = op(A) op(B) per matrix of a batch (op 0: as stored, 2: conjugate transpose), operands FP64 or
 // double-float, sums in double-float.
 //
-// Bound by the FP32 issue rate: with biased accumulators (ff.cuh) a complex multiply-add is 24
-// instructions, half of the TwoSum form, for an absolute error of 2^-47 of the accumulator's
-// bias per product.  The bias is set per element and k chunk of 32 from the chunk's largest row entry
-// of A and column sum of B, and the chunk's sum is folded into a normalised double-float total: about
-// 2^-41 of the result, far below the 22 bits of the exchange part that passes through.  Tile 64 x
-// 32, a thread holds rows ty + 16 i, columns tx + 16 j, so a tile's unused rows and columns are
-// skipped in steps of 16 (N = 108: 7 % of the work is padding).
-// Three products of 128 matrices, 108 x 702 x 108 twice and 108^3 once: 8.6 ms in the TwoSum form
-// with 4 x 4 outputs per thread, 1.74 + 1.53 + 0.31 = 3.6 ms here.
+// Bound by the FP32 issue rate: 48 instructions per complex multiply-add, its TwoSum and TwoProduct
+// errors collected beside the running sum, which is normalised after every k chunk of 32 so that the
+// collected part stays small: its own roundings are the largest error of a long sum.  Tile 64 x 32,
+// a thread holds rows ty + 16 i, columns tx + 16 j, so a tile's unused rows and columns are skipped in
+// steps of 16 (N = 108: 7 % of the work is padding).
+// Three products of 128 matrices, 108 x 702 x 108 twice and 108^3 once: 8.6 ms with 4 x 4
+// outputs per thread and tiles of 64 x 64, 2.29 + 2.23 + 0.41 = 4.9 ms here.  (Biased accumulators, 24
+// instructions per multiply-add for an error of 2^-47 of a row maximum times a column sum per product,
+// took 3.6 ms and made the gradient of E1 alone 25 to 60 times less exact on walkers near the trial.)
 constexpr int BM = 64, BN = 32, BK = 32, TI = 4, TJ = 2;
 constexpr int LDA = BM + 1, LDB = BN + 1;
-constexpr size_t GEMM_SMEM = sizeof(float4) * BK * (LDA + LDB) + sizeof(float) * (BM + BN);
+constexpr size_t GEMM_SMEM = sizeof(float4) * BK * (LDA + LDB);
 
 struct Dims {
   int m, n, k;
@@ -50,19 +50,17 @@ __global__ void __launch_bounds__(256, 2) gemm_ff_kernel(const TA* Ab, const TB*
   extern __shared__ __align__(16) unsigned char sm_raw[];
   float4* As = reinterpret_cast<float4*>(sm_raw);   // [BK][LDA]
   float4* Bs = As + BK * LDA;                         // [BK][LDB]
-  float* rmax = reinterpret_cast<float*>(Bs + BK * LDB);
-  float* csum = rmax + BM;
   const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
   const int row0 = blockIdx.y * BM, col0 = blockIdx.x * BN;
   const TA* A = Ab + (size_t)blockIdx.z * d.sa;
   const TB* B = Bb + (size_t)blockIdx.z * d.sb;
   TC* C = Cb + (size_t)blockIdx.z * d.sc;
   const int ni = (min(BM, d.m - row0) + 15) >> 4, nj = (min(BN, d.n - col0) + 15) >> 4;   // used steps of 16
-  float4 tot[TI][TJ];
+  ffa::cacc acc[TI][TJ];
 #pragma unroll
   for (int i = 0; i < TI; ++i)
 #pragma unroll
-    for (int j = 0; j < TJ; ++j) tot[i][j] = ffa::czero();
+    for (int j = 0; j < TJ; ++j) acc[i][j] = ffa::cacc_from(ffa::czero());
   for (int p0 = 0; p0 < d.k; p0 += BK) {
     __syncthreads();
     for (int e = t; e < BM * BK; e += 256) {   // along the operand's contiguous index
@@ -84,33 +82,6 @@ __global__ void __launch_bounds__(256, 2) gemm_ff_kernel(const TA* Ab, const TB*
       Bs[p * LDB + j] = v;
     }
     __syncthreads();
-    if (t < BM) {
-      float m = 0.f;
-#pragma unroll 8
-      for (int p = 0; p < BK; ++p) {
-        const float4 v = As[p * LDA + t];
-        m = fmaxf(m, fabsf(v.x) + fabsf(v.z));
-      }
-      rmax[t] = m;
-    } else if (t < BM + BN) {
-      float s = 0.f;
-#pragma unroll 8
-      for (int p = 0; p < BK; ++p) {
-        const float4 v = Bs[p * LDB + t - BM];
-        s += fmaxf(fabsf(v.x), fabsf(v.z));
-      }
-      csum[t - BM] = s;
-    }
-    __syncthreads();
-    ffa::bacc r[TI][TJ], m[TI][TJ];
-    float bias[TI][TJ];
-#pragma unroll
-    for (int i = 0; i < TI; ++i)
-#pragma unroll
-      for (int j = 0; j < TJ; ++j) {
-        bias[i][j] = ffa::bias_of(1.001f * rmax[ty + 16 * i] * csum[tx + 16 * j]);   // a hair for the sums' rounding
-        r[i][j] = m[i][j] = ffa::bacc{bias[i][j], 0.f};
-      }
 #pragma unroll 1
     for (int p = 0; p < BK; ++p) {
       float4 b[TJ];
@@ -123,10 +94,7 @@ __global__ void __launch_bounds__(256, 2) gemm_ff_kernel(const TA* Ab, const TB*
 #pragma unroll
         for (int j = 0; j < TJ; ++j) {
           if (j >= nj) break;
-          ffa::bacc_fma(r[i][j], a.x, a.y, b[j].x, b[j].y);
-          ffa::bacc_fma(m[i][j], a.x, a.y, b[j].z, b[j].w);
-          ffa::bacc_fma(r[i][j], -a.z, -a.w, b[j].z, b[j].w);
-          ffa::bacc_fma(m[i][j], a.z, a.w, b[j].x, b[j].y);
+          ffa::cacc_fma(acc[i][j], a, b[j]);
         }
       }
     }
@@ -134,15 +102,14 @@ __global__ void __launch_bounds__(256, 2) gemm_ff_kernel(const TA* Ab, const TB*
     for (int i = 0; i < TI; ++i)
 #pragma unroll
       for (int j = 0; j < TJ; ++j)
-        tot[i][j] = ffa::pack(ffa::add(ffa::re(tot[i][j]), ffa::bacc_get(r[i][j], bias[i][j])),
-                              ffa::add(ffa::im(tot[i][j]), ffa::bacc_get(m[i][j], bias[i][j])));
+        acc[i][j] = ffa::cacc_from(ffa::cacc_get(acc[i][j]));
   }
 #pragma unroll
   for (int i = 0; i < TI; ++i)
 #pragma unroll
     for (int j = 0; j < TJ; ++j) {
       const int gi = row0 + ty + 16 * i, gj = col0 + tx + 16 * j;
-      if (gi < d.m && gj < d.n) put(C + (size_t)gi * d.ldc + gj, tot[i][j]);
+      if (gi < d.m && gj < d.n) put(C + (size_t)gi * d.ldc + gj, ffa::cacc_get(acc[i][j]));
     }
 }
 
@@ -245,7 +212,7 @@ __global__ void __launch_bounds__(256) gamma_project_kernel(float4* Gam, const f
 }
 
 // The diagonal k blocks of the Green's function, ghd[ws][k][a][q] = sum_j S^-1[j][(k,a)] phi[(k,q)][j]:
-// all that dE/dh reads (1 / Nk of Gh).  grid (ws, k), sums in normalised double-float.
+// all that dE/dh reads (1 / Nk of Gh).  grid (ws, k), sums in double-float, normalised per chunk of j.
 constexpr int GD_J = 32;
 __global__ void __launch_bounds__(256) green_diag_kernel(const zc* phi, const float4* Sinv, zc* ghd, int nk, int M,
                                                          int n) {
@@ -268,6 +235,7 @@ __global__ void __launch_bounds__(256) green_diag_kernel(const zc* phi, const fl
       __syncthreads();
       if (e < n * M)
         for (int j = 0; j < jn; ++j) ffa::cacc_fma(acc, sv[j * n + a], gd[q * (GD_J + 1) + j]);
+      acc = ffa::cacc_from(ffa::cacc_get(acc));
     }
     if (e < n * M) put(ghd + ((size_t)ws * nk + k) * n * M + e, ffa::cacc_get(acc));
   }

@@ -129,36 +129,6 @@ __device__ __forceinline__ f2 acc_get(acc a) {
   return f2{s, e};
 }
 
-// Biased accumulator for a run of products whose size is known beforehand: s carries the sum
-// plus a power of two B with |sum of any part| <= B / 2 throughout, so that s stays within
-// [B/2, 3B/2], every s - s' is exact, and the rounding error of s + x.hi y.hi is one fused
-// multiply-add: six instructions a product where acc_fma's TwoSum takes twelve.  The price is an
-// absolute error: 2^-47 B per product (t collects errors of at most 2^-24 B), so B should be
-// no more than a few times the largest partial sum.
-struct bacc {
-  float s, t;
-};
-// the smallest B for a run bounded by `bound` (>= 0): 2 bound < B <= 4 bound
-__device__ __forceinline__ float bias_of(float bound) {
-  return __uint_as_float(min((__float_as_uint(bound) & 0x7f800000u) + (2u << 23), 0x7f000000u));
-}
-__device__ __forceinline__ bacc bacc_from(f2 x, float B) {
-  const float s = __fadd_rn(B, x.hi);
-  return bacc{s, __fadd_rn(__fsub_rn(x.hi, __fsub_rn(s, B)), x.lo)};
-}
-// a += x y
-__device__ __forceinline__ void bacc_fma(bacc& a, float xh, float xl, float yh, float yl) {
-  const float s = fmaf(xh, yh, a.s);
-  const float e = fmaf(xh, yh, __fsub_rn(a.s, s));
-  a.t = fmaf(xl, yh, fmaf(xh, yl, __fadd_rn(a.t, e)));
-  a.s = s;
-}
-__device__ __forceinline__ f2 bacc_get(bacc a, float B) {
-  float s, e;
-  two_sum(__fsub_rn(a.s, B), a.t, s, e);
-  return f2{s, e};
-}
-
 // ---------------------------------------------------------------- complex
 __device__ __forceinline__ f2 re(float4 v) { return f2{v.x, v.y}; }
 __device__ __forceinline__ f2 im(float4 v) { return f2{v.z, v.w}; }

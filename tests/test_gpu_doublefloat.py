@@ -1,6 +1,6 @@
-"""The log det of the mixed path at the precision of its arithmetic (double-float, 48 bits).
+"""The log det and the gradient of E1 of the mixed path at the precision of their arithmetic (double-float, 48 bits).
 
-The reference is the FP64 log det of the walker that the call returned, so that nothing of the
+Log det: the reference is the FP64 log det of the walker that the call returned, so that nothing of the
 22-bit split GEMMs enters.  An error dS of the overlap and its factorisation moves log det S by
 tr(S^-1 dS), so the bar is
   u sum_ij |S^-1|_ji (|A^dag| |phi| + P |L| |U|)_ij,  S = P L U.
@@ -19,6 +19,7 @@ import pytest
 import scipy.linalg
 
 import gen
+from oracle import afqmc_kp as ok
 
 torch = pytest.importorskip("torch")
 from gpu_util import dev, host, make, wrap_phase  # noqa: E402
@@ -111,3 +112,49 @@ def test_log_det_does_not_depend_on_the_batch(name):
     for call in got[0]:
         assert np.array_equal(got[0][call][0], got[1][call][0]), call
         assert np.array_equal(got[0][call][1], got[1][call][1]), call
+
+
+def gradient_bounds(osys, phi, g1):
+    """Sums of absolute values behind dE/dphi = [S^-1 (Gam - (Gam phi S^-1) A^dag)]^H of E1 and behind dE/dh, one
+    walker: the scale of one relative rounding of every operand."""
+    Ad, nk = osys.A_dense(), osys.nk
+    bphi, bh = np.empty(phi.shape), np.zeros((nk, osys.M, osys.M))
+    for s in range(2):
+        Gam = np.zeros((osys.N, osys.NM))
+        for k in range(nk):
+            Gam[osys.rows(k), osys.cols(k)] = abs(g1) * np.abs(osys.A[k].conj().T @ osys.h[k])
+        Sinv, p = np.abs(np.linalg.inv(Ad.conj().T @ phi[s])), np.abs(phi[s])
+        bphi[s] = (Sinv @ (Gam + Gam @ p @ Sinv @ np.abs(Ad).T)).T
+        Gh = (p @ Sinv).T
+        for k in range(nk):
+            bh[k] += abs(g1) * np.abs(osys.A[k]) @ Gh[osys.rows(k), osys.cols(k)]
+    return bphi, bh
+
+
+GRAD = {"N16": ((2, 2, 2), 2, 8), "N65": ((5, 1, 1), 13, 15), "N108": ((3, 3, 3), 4, 8), "N108wide": ((3, 3, 3), 4, 26),
+        "N256": ((4, 4, 1), 16, 17)}
+# u per kind of walkers: dE/dphi, dE/dh
+#   near: S^-1 is near the identity, so one product of each sum outweighs the others and every running sum keeps its
+#   size: sqrt(2 k) roundings of 2^-49 in the mean, k <= 702, 19 2^-49 per product sum, twice: u = 2^-44.
+GRAD_U = {"near": (2.0**-44, 2.0**-44)}
+
+
+@pytest.mark.parametrize("kind", list(GRAD_U))
+@pytest.mark.parametrize("name", list(GRAD))
+def test_e1_gradient(name, kind):
+    """E1 alone: no part of its gradient passes through the 22-bit exchange or the fp32 Coulomb sum."""
+    sp = spec(*GRAD[name])
+    sys_, osys = make(sp, "mixed")
+    phis = walkers(sp, kind)
+    g = np.zeros((2, 3), dtype=np.complex128)
+    g[:, 0] = gen.upstream(sp)[:, 0]
+    gphi, gh1 = (host(t) for t in sys_.local_energy_backward(dev(phis), dev(g)))
+    ref = [ok.local_energy_vjp(osys, phis[w], g[w], two_body=lambda *a: None) for w in range(2)]
+    bounds = [gradient_bounds(osys, phis[w], g[w, 0]) for w in range(2)]
+    uphi, uh = GRAD_U[kind]
+    for w in range(2):
+        assert np.linalg.norm(gphi[w] - ref[w][0]) < uphi * np.linalg.norm(bounds[w][0])
+    assert np.linalg.norm(gh1 - sum(r[1] for r in ref)) < uh * np.linalg.norm(sum(b[1] for b in bounds))
+    only = host(sys_.local_energy_backward(dev(phis), dev(g), want_phi=False)[1])
+    assert np.array_equal(only, gh1)
+    sys_.close()
