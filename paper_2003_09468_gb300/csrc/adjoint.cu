@@ -187,11 +187,10 @@ __global__ void __launch_bounds__(128) gamma_kernel(const zc* LH, const zc* X, c
 // Gam[ws][i][(k,r)] -= sum_a P[ws][i][(k,a)] conj(A[k][r][a]) ; grid (ws, row chunks of 16).  One pass
 // over Gam; P's rows of the chunk and one k block of A at a time in shared memory.
 constexpr int PROWS = 16;
-__global__ void __launch_bounds__(256) gamma_project_kernel(float4* Gam, const float4* P, const zc* A,
-                                                            const int* sing, int* flags, int nk, int M, int n) {
+__global__ void __launch_bounds__(256) gamma_project_kernel(float4* Gam, const float4* P, const zc* A, int nk, int M,
+                                                            int n) {
   const int ws = blockIdx.x, i0 = blockIdx.y * PROWS, N = nk * n, NM = nk * M;
   const int rows = min(PROWS, N - i0);
-  if (sing && blockIdx.y == 0 && threadIdx.x == 0 && sing[ws]) atomicAdd(&flags[0], 1);
   extern __shared__ __align__(16) float4 ps[];   // [rows][n] of one k block, then A[k] as [n][M]
   float4* as = ps + PROWS * n;
   for (int k = 0; k < nk; ++k) {
@@ -294,7 +293,7 @@ cudaError_t gamma(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e, co
 }
 
 cudaError_t project(const zc* phi, float4* Gam, const float4* Sinv, const zc* A, float4* Y, float4* P,
-                    const int* sing, int* flags, zc* grad_phi, int WS, int nk, int M, int n, cudaStream_t st) {
+                    zc* grad_phi, int WS, int nk, int M, int n, cudaStream_t st) {
   const int N = nk * n, NM = nk * M;
   const long NN = (long)N * N, NNM = (long)N * NM;
   cudaError_t e;
@@ -303,7 +302,7 @@ cudaError_t project(const zc* phi, float4* Gam, const float4* Sinv, const zc* A,
   if ((e = gemm<0, 0>(Y, Sinv, P, Dims{N, N, N, N, N, N, NN, NN, NN}, WS, st)) != cudaSuccess) return e;
   const size_t smem = sizeof(float4) * ((size_t)PROWS * n + (size_t)M * n);
   if ((e = ensure_dyn_smem(reinterpret_cast<const void*>(gamma_project_kernel), smem)) != cudaSuccess) return e;
-  gamma_project_kernel<<<dim3(WS, (N + PROWS - 1) / PROWS), 256, smem, st>>>(Gam, P, A, sing, flags, nk, M, n);
+  gamma_project_kernel<<<dim3(WS, (N + PROWS - 1) / PROWS), 256, smem, st>>>(Gam, P, A, nk, M, n);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // grad_phi = Gam^H S^-H
   return gemm<2, 2>(Gam, Sinv, grad_phi, Dims{NM, N, N, NM, N, N, NNM, NN, NNM}, WS, st);

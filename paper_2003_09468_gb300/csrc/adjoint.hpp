@@ -20,10 +20,9 @@ cudaError_t gamma(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e, co
                   const int* kminus, const int* minus, int nk, int G, int M, int n, int Mp, int W, cudaStream_t st);
 
 // grad_phi[ws] = [S^-1 (Gam - (Gam phi S^-1) A^dag)]^H per walker-spin (Gh^T = phi S^-1).  Gam is
-// overwritten; Y and P are [WS][N][N] scratch.  Four launches.  sing (may be NULL) / flags: every
-// singular walker (S^-1 = 0, so its gradient is 0) is counted once more.
+// overwritten; Y and P are [WS][N][N] scratch.  Four launches.
 cudaError_t project(const zc* phi, float4* Gam, const float4* Sinv, const zc* A, float4* Y, float4* P,
-                    const int* sing, int* flags, zc* grad_phi, int WS, int nk, int M, int n, cudaStream_t st);
+                    zc* grad_phi, int WS, int nk, int M, int n, cudaStream_t st);
 
 // grad_h1[k][p][q] = sum_w g1[w] sum_s sum_a A[k][p][a] conj(Gh[w][s][(k,a)][(k,q)]), Gh^T = phi S^-1.
 // ghd: [WS][nk][n][M] scratch, part: scratch of part_cap elements.  Three launches.

@@ -492,8 +492,7 @@ struct GcPanel {          // what the owner tells every CTA about one panel
 
 template <int C, bool INV, int GC_THREADS, int LPR>
 __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
-    gjc_ff_kernel(float4* Sff, int N, int keep, zc* logdet, int* sing, int* flags, __half* out, int Np,
-                  float* s_out) {
+    gjc_ff_kernel(float4* Sff, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out) {
   namespace cg = cooperative_groups;
   // rows of a column that a thread updates together; in the next panel's eight columns, which everybody
   // waits for, two up to N = 128 (LPR 2), where four would leave half of the threads without any
@@ -886,7 +885,6 @@ __global__ void __launch_bounds__(GC_THREADS, 512 / GC_THREADS)
     const float4 v = singular ? ffa::czero() : a[r * lda + c];
     const int i = singular ? c0 + c : perm[c0 + c];
     mixed::put4f(o + mixed::sp_at(i, Np, r), v.x * sc, v.z * sc);
-    if (keep) Sff[(size_t)b * N * N + (size_t)r * N + i] = v;   // every CTA read its columns before the first panel
   }
   if (C > 1) cg::this_cluster().sync();
 }
@@ -900,7 +898,7 @@ size_t gj_smem_bytes(int N) { return (size_t)N * (sizeof(float4) + sizeof(double
 
 struct GjcArgs {
   float4* Sff;
-  int WS, N, keep;
+  int WS, N;
   zc* logdet;
   int *sing, *flags;
   __half* out;
@@ -926,7 +924,7 @@ cudaError_t gjc_launch(const GjcArgs& g, cudaStream_t st) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = C > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, fn, g.Sff, g.N, g.keep, g.logdet, g.sing, g.flags, g.out, g.Np, g.s_out);
+  return cudaLaunchKernelEx(&cfg, fn, g.Sff, g.N, g.logdet, g.sing, g.flags, g.out, g.Np, g.s_out);
 }
 
 // CTAs per matrix: the fewest whose shared memory holds it (0: none up to 8), doubled while every
@@ -969,7 +967,7 @@ cudaError_t gjc_invert(const GjcArgs& g, cudaStream_t st) {
   if (C == 0) return cudaErrorNotSupported;
   if (N > 128) C = C <= 4 ? 4 : 8;
   int dev = 0, sms = 0;
-  if (C > 1 && !g.keep && cudaGetDevice(&dev) == cudaSuccess &&
+  if (C > 1 && cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
       !cluster_pays(g.WS, C, INV, sms))
     return cudaErrorNotSupported;
@@ -1004,14 +1002,11 @@ cudaError_t overlap(const zc* A, const zc* phi, const zc* B, float4* Sff, float2
   return cudaGetLastError();
 }
 
-bool keeps_inverse(int N) { return gjc_cluster(1, N) > 0; }
-
 cudaError_t invert(float4* Sff, int WS, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out,
-                   cudaStream_t st, bool keep) {
-  const GjcArgs g = {Sff, WS, N, keep ? 1 : 0, logdet, sing, flags, out, Np, s_out};
+                   cudaStream_t st) {
+  const GjcArgs g = {Sff, WS, N, logdet, sing, flags, out, Np, s_out};
   const cudaError_t ec = out ? gjc_invert<true>(g, st) : gjc_invert<false>(g, st);
   if (ec != cudaErrorNotSupported) return ec;
-  if (keep) return cudaErrorNotSupported;
   cudaError_t e;
   if (out) {
     const size_t bytes = (size_t)GJB * N * sizeof(float4) + gj_smem_bytes(N);

@@ -2024,8 +2024,7 @@ static cudaError_t overlap_logdet(afqmc_kp* h, const zc* phi, zc* ld, int* sing,
 
 // The Green's function in three parts: the double-float overlap, inverse and log det and
 // the split of phi_perp (green_pre); the tensor-core GEMM; its max and split (green_post).
-// keep: S^-1 stays in s_ff in double-float (ffla::keeps_inverse).
-static cudaError_t green_pre(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st, bool keep = false) {
+static cudaError_t green_pre(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st) {
   MixedState* m = h->mixed;
   const int WS = m->WS;
   unsigned long long* mx_phi = m->mx;
@@ -2038,7 +2037,7 @@ static cudaError_t green_pre(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cuda
   MTRY(cudaMemsetAsync(m->mx, 0, sizeof(unsigned long long) * (2 * WS + 3 * h->W), st));
   MTRY(ffla::overlap(h->A, phi, m->bproj, m->s_ff, phi_perp, mx_phi, WS, h->nk, h->M, h->n, h->N, st));
   AFQMC_LAUNCHED(h);
-  MTRY(ffla::invert(m->s_ff, WS, h->N, ld, sing, h->flags, m->sinvt_sp, m->Np, m->s_sinv, st, keep));
+  MTRY(ffla::invert(m->s_ff, WS, h->N, ld, sing, h->flags, m->sinvt_sp, m->Np, m->s_sinv, st));
   AFQMC_LAUNCHED(h);
   split_rows32_kernel<<<dim3(WS, SPLIT_CHUNKS), 256, 0, st>>>(phi_perp, h->NM, h->N, m->Np, mx_phi, m->s_phi,
                                                                m->phi_sp);
@@ -2055,9 +2054,9 @@ static cudaError_t green_post(afqmc_kp* h, cudaStream_t st) {
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
 }
-static cudaError_t green(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st, bool keep = false) {
+static cudaError_t green(afqmc_kp* h, const zc* phi, zc* ld, int* sing, cudaStream_t st) {
   MixedState* m = h->mixed;
-  MTRY(green_pre(h, phi, ld, sing, st, keep));
+  MTRY(green_pre(h, phi, ld, sing, st));
   MTRY(run_gemm(h, m->m_sinvt, m->m_phi, green_params(h), h->flags + 1, st));
   AFQMC_LAUNCHED(h);
   return green_post(h, st);
@@ -2457,29 +2456,25 @@ static cudaError_t adjoint_exchange(afqmc_kp* h, cudaStream_t st) {
 // The adjoint: Gam = conj(grad_e)-weighted dE/dGh with the exchange part from the
 // tensor-core GEMM over the full precontracted tensor and the Coulomb and one-body parts in
 // fp32, then the projection onto dE/dphi through S^-1 and the walker, and dE/dh, in double-float
-// (adjoint.cu).  S^-1 is the Green's function's own, kept in double-float; matrices too large for
-// that form go through the FP64 LU.
+// (adjoint.cu) from the FP64 inverse.  (The Green's function's own inverse in double-float would save the
+// LU and the FP64 overlap, 3.3 of 12.5 ms at N = 108, but its elimination loses cond(S) of 48 bits: on random
+// walkers dE/dh went from 1e-13 to 5e-12 of its norm.)
 cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, zc* grad_phi, zc* grad_h1,
                                   cudaStream_t st) {
   MixedState* m = h->mixed;
-  const bool keep = ffla::keeps_inverse(h->N);
   float4* Gam = reinterpret_cast<float4*>(h->Gam);
   if (grad_phi) {
-    MSTAGE(AFQMC_STAGE_GREEN, green(h, phi, h->ld_old, h->sing_old, st, keep));
+    MSTAGE(AFQMC_STAGE_GREEN, green(h, phi, h->ld_old, h->sing_old, st));
     MSTAGE(AFQMC_STAGE_FORCE_BIAS, cholesky_trace(h, st));
     MSTAGE(AFQMC_STAGE_ADJOINT_GEMM, adjoint_exchange(h, st));
     AFQMC_LAUNCHED(h);
     MSTAGE(AFQMC_STAGE_BACKWARD, adjoint::gamma(h->LH, h->X, h->AhH, grad_e, m->gam32, Gam, h->kminus, h->minus,
                                                 h->nk, h->G, h->M, h->n, m->Mp, h->W, st));
     AFQMC_LAUNCHED(h);
-  } else if (keep) {
-    MSTAGE(AFQMC_STAGE_GREEN, green_pre(h, phi, h->ld_old, h->sing_old, st, true));
   }
-  if (!keep) {
-    MSTAGE(AFQMC_STAGE_GREEN, fp64::overlap_lu(h, phi, h->ld_old, h->sing_old, 1, st));
-    MTRY(adjoint::to_ff(h->Sinv, m->s_ff, (size_t)m->WS * h->N * h->N, st));
-    AFQMC_LAUNCHED(h);
-  }
+  MSTAGE(AFQMC_STAGE_GREEN, fp64::overlap_lu(h, phi, h->ld_old, h->sing_old, 1, st));
+  MTRY(adjoint::to_ff(h->Sinv, m->s_ff, (size_t)m->WS * h->N * h->N, st));
+  AFQMC_LAUNCHED(h);
   if (grad_h1) {
     MSTAGE(AFQMC_STAGE_BACKWARD, adjoint::grad_h1(phi, m->s_ff, h->A, grad_e, h->Gh, h->P,
                                                   (size_t)m->WS * h->N * h->N, grad_h1, h->W, h->nk, h->M, h->n, st));
@@ -2488,7 +2483,7 @@ cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, 
   if (grad_phi) {
     MSTAGE(AFQMC_STAGE_BACKWARD,
            adjoint::project(phi, Gam, m->s_ff, h->A, reinterpret_cast<float4*>(h->P), reinterpret_cast<float4*>(h->S),
-                            keep ? h->sing_old : nullptr, h->flags, grad_phi, m->WS, h->nk, h->M, h->n, st));
+                            grad_phi, m->WS, h->nk, h->M, h->n, st));
     h->launches += 4;
   }
   return cudaSuccess;

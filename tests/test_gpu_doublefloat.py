@@ -136,7 +136,10 @@ GRAD = {"N16": ((2, 2, 2), 2, 8), "N65": ((5, 1, 1), 13, 15), "N108": ((3, 3, 3)
 # u per kind of walkers: dE/dphi, dE/dh
 #   near: S^-1 is near the identity, so one product of each sum outweighs the others and every running sum keeps its
 #   size: sqrt(2 k) roundings of 2^-49 in the mean, k <= 702, 19 2^-49 per product sum, twice: u = 2^-44.
-GRAD_U = {"near": (2.0**-44, 2.0**-44)}
+#   random: terms of random sign, running sums far below the sums of absolute values: the operands' own
+#   rounding to 48 bits (2^-48 at most, half of it in the mean, and cond(S) 2^-53 of the inverse): u = 2^-48 for
+#   dE/dphi, whose bound multiplies four such sums, 2^-47 for dE/dh.
+GRAD_U = {"near": (2.0**-44, 2.0**-44), "random": (2.0**-48, 2.0**-47)}
 
 
 @pytest.mark.parametrize("kind", list(GRAD_U))
