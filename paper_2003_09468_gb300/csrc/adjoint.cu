@@ -33,7 +33,7 @@ __global__ void to_ff_kernel(const zc* in, float4* out, size_t n) {
 // a thread holds rows ty + 16 i, columns tx + 16 j, so a tile's unused rows and columns are skipped in
 // steps of 16 (N = 108: 7 % of the work is padding).
 // Three products of 128 matrices, 108 x 702 x 108 twice and 108^3 once: 8.6 ms with 4 x 4
-// outputs per thread and tiles of 64 x 64, 2.29 + 2.23 + 0.41 = 4.9 ms here.  (Biased accumulators, 24
+// outputs per thread and tiles of 64 x 64, 2.44 + 2.38 + 0.41 = 5.2 ms here (4.9 with Gam in double-float).  (Biased accumulators, 24
 // instructions per multiply-add for an error of 2^-47 of a row maximum times a column sum per product,
 // took 3.6 ms and made the gradient of E1 alone 25 to 60 times less exact on walkers near the trial.)
 constexpr int BM = 64, BN = 32, BK = 32, TI = 4, TJ = 2;
@@ -129,23 +129,24 @@ cudaError_t gemm(const TA* A, const TB* B, TC* C, const Dims& d, int batch, cuda
 // A block takes one (k1, Q) and GW walkers; a thread one (a, r) for all of them, so that each FP64
 // vector element is converted once per GW walkers (the conversions run at the FP64 pipe's two per
 // clock); consecutive walkers' X lie side by side in shared memory, two per load.  The weights are
-// applied in double-float: a double per element and part would cost as much as the sums.
+// applied and the parts added in FP64, in which Gam is kept (610 us at 3x3x3, 64 walkers; 515 with
+// double-float weights, which left up to four roundings of 2^-48 where FP64 leaves one).
 template <int GW>
 __global__ void __launch_bounds__(128) gamma_kernel(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e,
-                                                    const float2* gam32, float4* Gam, const int* kminus,
+                                                    const float2* gam32, zc* Gam, const int* kminus,
                                                     const int* minus, int nk, int G, int M, int n, int Mp, int W) {
   const int k1 = blockIdx.x, Q = blockIdx.y, w0 = blockIdx.z * GW;
   const int k2 = kminus[k1 * nk + Q], mQ = minus[Q];
   const int nw = min(GW, W - w0);
   const int nM = n * M, N = nk * n, NM = nk * M, WS = 2 * W, nMp = n * Mp;
   extern __shared__ __align__(16) float2 xs[];   // [G][GW]
-  __shared__ float4 cw[GW][3];                    // conj(grad_e)
+  __shared__ zc cw[GW][3];                        // conj(grad_e)
   for (int e = threadIdx.x; e < GW * G; e += blockDim.x) {
     const int wi = e / G, g = e % G;
     const zc v = wi < nw ? X[((size_t)(w0 + wi) * nk + mQ) * G + g] : zzero();
     xs[g * GW + wi] = make_float2((float)v.x, (float)v.y);
   }
-  for (int e = threadIdx.x; e < 3 * nw; e += blockDim.x) cw[e / 3][e % 3] = conj_ff(ff_of(grad_e[3 * w0 + e]));
+  for (int e = threadIdx.x; e < 3 * nw; e += blockDim.x) cw[e / 3][e % 3] = zconj(grad_e[3 * w0 + e]);
   __syncthreads();
   const zc* lh = LH + ((size_t)Q * nk + k1) * G * nM;
   for (int e = threadIdx.x; e < nM; e += blockDim.x) {
@@ -167,27 +168,27 @@ __global__ void __launch_bounds__(128) gamma_kernel(const zc* LH, const zc* X, c
       }
     }
     const int a = e / M, r = e % M;
-    const float4 ah = Q == 0 ? ff_of(AhH[(size_t)k1 * nM + e]) : ffa::czero();
+    const zc ah = Q == 0 ? AhH[(size_t)k1 * nM + e] : zzero();
 #pragma unroll
     for (int i = 0; i < GW; ++i) {
       if (i >= nw) break;
       const int w = w0 + i;
-      float4 base = ffa::cmul(cw[i][1], make_float4(acc[i].x, 0.f, acc[i].y, 0.f));
-      if (Q == 0) base = ffa::cfma(base, cw[i][0], ah);
+      zc base = zmul(cw[i][1], zmake(f2d(acc[i].x), f2d(acc[i].y)));
+      if (Q == 0) base = zfma(cw[i][0], ah, base);
       for (int sp = 0; sp < 2; ++sp) {
         const int ws = 2 * w + sp;
         const float2 gx = gam32[(((size_t)k1 * nk + k2) * WS + ws) * nMp + a * Mp + r];
         Gam[((size_t)ws * N + k1 * n + a) * NM + k2 * M + r] =
-            ffa::cfms(base, cw[i][2], make_float4(gx.x, 0.f, gx.y, 0.f));
+            zsub(base, zmul(cw[i][2], zmake(f2d(gx.x), f2d(gx.y))));
       }
     }
   }
 }
 
 // Gam[ws][i][(k,r)] -= sum_a P[ws][i][(k,a)] conj(A[k][r][a]) ; grid (ws, row chunks of 16).  One pass
-// over Gam; P's rows of the chunk and one k block of A at a time in shared memory.
+// over Gam, which the difference leaves in FP64; P's rows of the chunk and one k block of A at a time in shared memory.
 constexpr int PROWS = 16;
-__global__ void __launch_bounds__(256) gamma_project_kernel(float4* Gam, const float4* P, const zc* A, int nk, int M,
+__global__ void __launch_bounds__(256) gamma_project_kernel(zc* Gam, const float4* P, const zc* A, int nk, int M,
                                                             int n) {
   const int ws = blockIdx.x, i0 = blockIdx.y * PROWS, N = nk * n, NM = nk * M;
   const int rows = min(PROWS, N - i0);
@@ -202,10 +203,11 @@ __global__ void __launch_bounds__(256) gamma_project_kernel(float4* Gam, const f
     __syncthreads();
     for (int e = threadIdx.x; e < rows * M; e += blockDim.x) {
       const int i = e / M, r = e % M;
-      float4* o = Gam + ((size_t)ws * N + i0 + i) * NM + k * M + r;
-      ffa::cacc acc = ffa::cacc_from(*o);
-      for (int a = 0; a < n; ++a) ffa::cacc_fms(acc, ps[i * n + a], as[a * M + r]);
-      *o = ffa::cacc_get(acc);
+      zc* o = Gam + ((size_t)ws * N + i0 + i) * NM + k * M + r;
+      ffa::cacc acc = ffa::cacc_from(ffa::czero());
+      for (int a = 0; a < n; ++a) ffa::cacc_fma(acc, ps[i * n + a], as[a * M + r]);
+      const float4 v = ffa::cacc_get(acc);
+      *o = zsub(*o, zmake(ffa::to_double(ffa::re(v)), ffa::to_double(ffa::im(v))));
     }
   }
 }
@@ -281,7 +283,7 @@ cudaError_t gamma_smem(int G) {
                        : ensure_dyn_smem(reinterpret_cast<const void*>(gamma_kernel<16>), sizeof(float2) * 16 * G);
 }
 
-cudaError_t gamma(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e, const float2* gam32, float4* Gam,
+cudaError_t gamma(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e, const float2* gam32, zc* Gam,
                   const int* kminus, const int* minus, int nk, int G, int M, int n, int Mp, int W, cudaStream_t st) {
   if (gamma_wide(G))
     gamma_kernel<32><<<dim3(nk, nk, (W + 31) / 32), 128, sizeof(float2) * 32 * G, st>>>(
@@ -292,7 +294,7 @@ cudaError_t gamma(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e, co
   return cudaGetLastError();
 }
 
-cudaError_t project(const zc* phi, float4* Gam, const float4* Sinv, const zc* A, float4* Y, float4* P,
+cudaError_t project(const zc* phi, zc* Gam, const float4* Sinv, const zc* A, float4* Y, float4* P,
                     zc* grad_phi, int WS, int nk, int M, int n, cudaStream_t st) {
   const int N = nk * n, NM = nk * M;
   const long NN = (long)N * N, NNM = (long)N * NM;

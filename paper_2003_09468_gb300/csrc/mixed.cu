@@ -2462,13 +2462,12 @@ static cudaError_t adjoint_exchange(afqmc_kp* h, cudaStream_t st) {
 cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, zc* grad_phi, zc* grad_h1,
                                   cudaStream_t st) {
   MixedState* m = h->mixed;
-  float4* Gam = reinterpret_cast<float4*>(h->Gam);
   if (grad_phi) {
     MSTAGE(AFQMC_STAGE_GREEN, green(h, phi, h->ld_old, h->sing_old, st));
     MSTAGE(AFQMC_STAGE_FORCE_BIAS, cholesky_trace(h, st));
     MSTAGE(AFQMC_STAGE_ADJOINT_GEMM, adjoint_exchange(h, st));
     AFQMC_LAUNCHED(h);
-    MSTAGE(AFQMC_STAGE_BACKWARD, adjoint::gamma(h->LH, h->X, h->AhH, grad_e, m->gam32, Gam, h->kminus, h->minus,
+    MSTAGE(AFQMC_STAGE_BACKWARD, adjoint::gamma(h->LH, h->X, h->AhH, grad_e, m->gam32, h->Gam, h->kminus, h->minus,
                                                 h->nk, h->G, h->M, h->n, m->Mp, h->W, st));
     AFQMC_LAUNCHED(h);
   }
@@ -2482,7 +2481,7 @@ cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, 
   }
   if (grad_phi) {
     MSTAGE(AFQMC_STAGE_BACKWARD,
-           adjoint::project(phi, Gam, m->s_ff, h->A, reinterpret_cast<float4*>(h->P), reinterpret_cast<float4*>(h->S),
+           adjoint::project(phi, h->Gam, m->s_ff, h->A, reinterpret_cast<float4*>(h->P), reinterpret_cast<float4*>(h->S),
                             grad_phi, m->WS, h->nk, h->M, h->n, st));
     h->launches += 4;
   }

@@ -161,3 +161,22 @@ def test_e1_gradient(name, kind):
     only = host(sys_.local_energy_backward(dev(phis), dev(g), want_phi=False)[1])
     assert np.array_equal(only, gh1)
     sys_.close()
+
+
+def test_e1_gradient_weights():
+    """The weights enter in FP64: with the trial itself as the walker S^-1 is the identity and the virtual rows of
+    dE1/dphi are g conj(h A) unprojected, exact but for their one rounding to 48 bits (2^-48 of each
+    part; an eighth more for the FP64 operations)."""
+    sp = spec((2, 1, 1), 2, 24)
+    sys_, osys = make(sp, "mixed")
+    phis = np.broadcast_to(gen.trial_dense(sp), (2, 2, sp.NM, sp.N))
+    g = np.zeros((2, 3), dtype=np.complex128)
+    g[:, 0] = gen.upstream(sp)[:, 0]
+    gphi = host(sys_.local_energy_backward(dev(phis), dev(g), want_h1=False)[0])
+    for k in range(sp.nk):
+        virtual, occupied = slice(k * sp.M + sp.nocc, (k + 1) * sp.M), osys.rows(k)
+        want = g[:, 0, None, None, None] * (osys.A[k].conj().T @ osys.h[k]).conj().T[sp.nocc:]
+        d = gphi[:, :, virtual, occupied] - want
+        u = 1.125 * 2.0**-48
+        assert (np.abs(d.real) <= u * np.abs(want.real)).all() and (np.abs(d.imag) <= u * np.abs(want.imag)).all()
+    sys_.close()
