@@ -114,13 +114,14 @@ __global__ void __launch_bounds__(256, 2) gemm_ff_kernel(const TA* Ab, const TB*
 }
 
 template <int OPA, int OPB, class TA, class TB, class TC>
-cudaError_t gemm(const TA* A, const TB* B, TC* C, const Dims& d, int batch, cudaStream_t st) {
+cudaError_t gemm(const TA* A, const TB* B, TC* C, const Dims& d, int batch, int& launches, cudaStream_t st) {
   auto fn = gemm_ff_kernel<OPA, OPB, TA, TB, TC>;
   cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(fn), GEMM_SMEM);
   if (e != cudaSuccess) return e;
   for (int b0 = 0; b0 < batch; b0 += 65535) {
     const dim3 grid((d.n + BN - 1) / BN, (d.m + BM - 1) / BM, std::min(batch - b0, 65535));
     fn<<<grid, 256, GEMM_SMEM, st>>>(A + (size_t)b0 * d.sa, B + (size_t)b0 * d.sb, C + (size_t)b0 * d.sc, d);
+    ++launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -295,34 +296,38 @@ cudaError_t gamma(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e, co
 }
 
 cudaError_t project(const zc* phi, zc* Gam, const float4* Sinv, const zc* A, float4* Y, float4* P,
-                    zc* grad_phi, int WS, int nk, int M, int n, cudaStream_t st) {
+                    zc* grad_phi, int WS, int nk, int M, int n, int& launches, cudaStream_t st) {
   const int N = nk * n, NM = nk * M;
   const long NN = (long)N * N, NNM = (long)N * NM;
   cudaError_t e;
   // Y = Gam phi, P = Y S^-1
-  if ((e = gemm<0, 0>(Gam, phi, Y, Dims{N, N, NM, NM, N, N, NNM, NNM, NN}, WS, st)) != cudaSuccess) return e;
-  if ((e = gemm<0, 0>(Y, Sinv, P, Dims{N, N, N, N, N, N, NN, NN, NN}, WS, st)) != cudaSuccess) return e;
+  if ((e = gemm<0, 0>(Gam, phi, Y, Dims{N, N, NM, NM, N, N, NNM, NNM, NN}, WS, launches, st)) != cudaSuccess) return e;
+  if ((e = gemm<0, 0>(Y, Sinv, P, Dims{N, N, N, N, N, N, NN, NN, NN}, WS, launches, st)) != cudaSuccess) return e;
   const size_t smem = sizeof(float4) * ((size_t)PROWS * n + (size_t)M * n);
   if ((e = ensure_dyn_smem(reinterpret_cast<const void*>(gamma_project_kernel), smem)) != cudaSuccess) return e;
   gamma_project_kernel<<<dim3(WS, (N + PROWS - 1) / PROWS), 256, smem, st>>>(Gam, P, A, nk, M, n);
+  ++launches;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // grad_phi = Gam^H S^-H
-  return gemm<2, 2>(Gam, Sinv, grad_phi, Dims{NM, N, N, NM, N, N, NNM, NN, NNM}, WS, st);
+  return gemm<2, 2>(Gam, Sinv, grad_phi, Dims{NM, N, N, NM, N, N, NNM, NN, NNM}, WS, launches, st);
 }
 
 cudaError_t grad_h1(const zc* phi, const float4* Sinv, const zc* A, const zc* grad_e, zc* ghd, zc* part,
-                    size_t part_cap, zc* gh1, int W, int nk, int M, int n, cudaStream_t st) {
+                    size_t part_cap, zc* gh1, int W, int nk, int M, int n, int& launches, cudaStream_t st) {
   const size_t smem = sizeof(float4) * ((size_t)M * (GD_J + 1) + (size_t)GD_J * n);
   cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(green_diag_kernel), smem);
   if (e != cudaSuccess) return e;
   green_diag_kernel<<<dim3(2 * W, nk), std::min(256, (n * M + 31) / 32 * 32), smem, st>>>(phi, Sinv, ghd, nk, M, n);
+  ++launches;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const size_t per = (size_t)nk * M * M;
   const int chunks = (int)std::max<size_t>(1, std::min<size_t>({(size_t)16, (size_t)W, part_cap / per}));
   zc* dst = chunks == 1 ? gh1 : part;
   grad_h1_part_kernel<<<dim3(nk, chunks), 256, 0, st>>>(A, ghd, grad_e, dst, nk, M, n, W);
+  ++launches;
   if ((e = cudaGetLastError()) != cudaSuccess || chunks == 1) return e;
   grad_h1_sum_kernel<<<(int)std::min<size_t>((per + 255) / 256, 4096), 256, 0, st>>>(part, gh1, chunks, per);
+  ++launches;
   return cudaGetLastError();
 }
 

@@ -20,13 +20,14 @@ cudaError_t gamma(const zc* LH, const zc* X, const zc* AhH, const zc* grad_e, co
                   const int* kminus, const int* minus, int nk, int G, int M, int n, int Mp, int W, cudaStream_t st);
 
 // grad_phi[ws] = [S^-1 (Gam - (Gam phi S^-1) A^dag)]^H per walker-spin (Gh^T = phi S^-1).  Gam is
-// overwritten; Y and P are [WS][N][N] scratch.  Four launches.
+// overwritten; Y and P are [WS][N][N] scratch.
+// launches: incremented by every kernel launch.
 cudaError_t project(const zc* phi, zc* Gam, const float4* Sinv, const zc* A, float4* Y, float4* P,
-                    zc* grad_phi, int WS, int nk, int M, int n, cudaStream_t st);
+                    zc* grad_phi, int WS, int nk, int M, int n, int& launches, cudaStream_t st);
 
 // grad_h1[k][p][q] = sum_w g1[w] sum_s sum_a A[k][p][a] conj(Gh[w][s][(k,a)][(k,q)]), Gh^T = phi S^-1.
-// ghd: [WS][nk][n][M] scratch, part: scratch of part_cap elements.  Three launches.
+// ghd: [WS][nk][n][M] scratch, part: scratch of part_cap elements. 
 cudaError_t grad_h1(const zc* phi, const float4* Sinv, const zc* A, const zc* grad_e, zc* ghd, zc* part,
-                    size_t part_cap, zc* gh1, int W, int nk, int M, int n, cudaStream_t st);
+                    size_t part_cap, zc* gh1, int W, int nk, int M, int n, int& launches, cudaStream_t st);
 
 }  // namespace adjoint

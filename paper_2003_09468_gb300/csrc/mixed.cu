@@ -2476,14 +2476,13 @@ cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, 
   AFQMC_LAUNCHED(h);
   if (grad_h1) {
     MSTAGE(AFQMC_STAGE_BACKWARD, adjoint::grad_h1(phi, m->s_ff, h->A, grad_e, h->Gh, h->P,
-                                                  (size_t)m->WS * h->N * h->N, grad_h1, h->W, h->nk, h->M, h->n, st));
-    h->launches += 3;
+                                                  (size_t)m->WS * h->N * h->N, grad_h1, h->W, h->nk, h->M, h->n,
+                                                  h->launches, st));
   }
   if (grad_phi) {
     MSTAGE(AFQMC_STAGE_BACKWARD,
            adjoint::project(phi, h->Gam, m->s_ff, h->A, reinterpret_cast<float4*>(h->P), reinterpret_cast<float4*>(h->S),
-                            grad_phi, m->WS, h->nk, h->M, h->n, st));
-    h->launches += 4;
+                            grad_phi, m->WS, h->nk, h->M, h->n, h->launches, st));
   }
   return cudaSuccess;
 }
