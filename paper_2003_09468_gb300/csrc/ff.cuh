@@ -137,12 +137,6 @@ __device__ __forceinline__ float4 czero() { return make_float4(0.f, 0.f, 0.f, 0.
 __device__ __forceinline__ float4 cneg(float4 v) { return make_float4(-v.x, -v.y, -v.z, -v.w); }
 __device__ __forceinline__ float4 cfrom(double2 v) { return pack(from_double(v.x), from_double(v.y)); }
 
-// a + x y
-__device__ __forceinline__ float4 cfma(float4 a, float4 x, float4 y) {
-  const f2 r = fma(fma(re(a), re(x), re(y)), neg(im(x)), im(y));
-  const f2 i = fma(fma(im(a), re(x), im(y)), im(x), re(y));
-  return pack(r, i);
-}
 // a - x y
 __device__ __forceinline__ float4 cfms(float4 a, float4 x, float4 y) {
   const f2 r = fma(fma(re(a), neg(re(x)), re(y)), im(x), im(y));
@@ -176,12 +170,6 @@ __device__ __forceinline__ void cacc_fms(cacc& a, float4 x, float4 y) {
 }
 __device__ __forceinline__ float4 cacc_get(cacc a) { return pack(acc_get(a.r), acc_get(a.i)); }
 
-// a + conj(x) y
-__device__ __forceinline__ float4 cfma_conj(float4 a, float4 x, float4 y) {
-  const f2 r = fma(fma(re(a), re(x), re(y)), im(x), im(y));
-  const f2 i = fma(fma(im(a), re(x), im(y)), neg(im(x)), re(y));
-  return pack(r, i);
-}
 __device__ __forceinline__ float4 cmul(float4 x, float4 y) {
   const f2 r = fma(mul(re(x), re(y)), neg(im(x)), im(y));
   const f2 i = fma(mul(re(x), im(y)), im(x), re(y));

@@ -946,7 +946,8 @@ int gjc_cluster(int WS, int N) {
 // Whether a cluster of C CTAs per matrix beats one CTA per matrix in the global form.  Of the clusters
 // only 76 / 36 / 15 (C = 2 / 4 / 8) run at once on 152 SMs, so many matrices take many waves; `gain` is
 // what one wave of the global form costs in waves of clusters (a little less beyond one wave, when its
-// CTAs no longer move in step).  Measured, cluster | global, ms:
+// CTAs no longer move in step).  It takes the GPU to be free; members of a group on their own streams share it, and
+// then either form may be the slower one, with the same bits.  Measured, cluster | global, ms:
 //   inverse  N = 256: 64 matrices 4.63 | 6.55, 128 8.33 | 7.08, 304 19.4 | 12.7, 512 32.3 | 24.2
 //            N = 160: 64 1.05 | 1.84, 128 2.09 | 1.85, 512 7.80 | 6.46;  N = 120: 128 0.73 | 0.89, 512 2.58 | 2.99
 //   log det  N = 256: 64 3.19 | 4.81, 128 5.75 | 7.09, 304 13.4 | 11.4, 512 22.3 | 20.4

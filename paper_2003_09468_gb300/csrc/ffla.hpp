@@ -19,7 +19,8 @@ cudaError_t overlap(const zc* A, const zc* phi, const zc* B, float4* Sff, float2
 
 // log det of every Sff matrix into logdet[WS] (sing[ws] = 1 and flags[0] incremented for a
 // singular one).  With out != nullptr also S^-T as fp16 split planes out[WS][N][Np] (split.cuh)
-// with per-matrix scale s_out[ws].  Sff is overwritten.
+// with per-matrix scale s_out[ws].  Sff is overwritten.  The log det of the two forms (with and
+// without the inverse) differs in its last bits; each depends on the matrix alone, not on WS.
 cudaError_t invert(float4* Sff, int WS, int N, zc* logdet, int* sing, int* flags, __half* out, int Np, float* s_out,
                    cudaStream_t st);
 

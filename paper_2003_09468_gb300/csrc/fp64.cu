@@ -799,12 +799,6 @@ static cudaError_t one_body(afqmc_kp* h, const zc* in, zc* out, cudaStream_t st)
   return gemm_launch(h, g, st);
 }
 
-// The two halves of overlap_lu, for callers that use S before it is factorised.
-cudaError_t overlap_only(afqmc_kp* h, const zc* phi, cudaStream_t st) { return overlap(h, phi, st); }
-cudaError_t lu_only(afqmc_kp* h, zc* ld, int* sing, int want_inv, cudaStream_t st) {
-  return lu_launch(h, ld, sing, want_inv, st);
-}
-
 cudaError_t overlap_lu(afqmc_kp* h, const zc* phi, zc* ld, int* sing, int want_inv, cudaStream_t st) {
   cudaError_t e = overlap(h, phi, st);
   if (e != cudaSuccess) return e;
@@ -1153,7 +1147,7 @@ __global__ void grad_h1_kernel(const zc* A, const zc* Gh, const zc* grad_e, zc* 
   }
 }
 
-cudaError_t grad_h1(afqmc_kp* h, const zc* grad_e, zc* gh1, cudaStream_t st) {
+static cudaError_t grad_h1(afqmc_kp* h, const zc* grad_e, zc* gh1, cudaStream_t st) {
   grad_h1_kernel<<<h->nk, 256, 0, st>>>(h->A, h->Gh, grad_e, gh1, h->nk, h->M, h->n, h->W);
   AFQMC_LAUNCHED(h);
   return cudaGetLastError();
@@ -1162,9 +1156,8 @@ cudaError_t grad_h1(afqmc_kp* h, const zc* grad_e, zc* gh1, cudaStream_t st) {
 // dE/dphi from Gam = conj(grad_e)-weighted dE/dGh: with Gh = S^-T phi^T and S = A^dag phi,
 // dGh = S^-T dphi^T (I - A* Gh), so grad_phi = [S^-1 (Gam - (Gam Gh^T) A^dag)]^H in the
 // conjugate convention of the binding.
-cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st) {
+static cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st) {
   cudaError_t e;
-  auto launch = [&](const ZGemm& g) { return gemm_launch(h, g, st); };
   const int nk = h->nk, M = h->M, n = h->n, N = h->N, NM = h->NM, W = h->W;
   {  // P = Gam Gh^T  (N x N)
     ZGemm g = gemm_init(N, N, NM, 0, 1);
@@ -1172,7 +1165,7 @@ cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st) {
     g.B = h->Gh; g.ldb = NM; g.sB[0] = (long)N * NM;
     g.C = h->P; g.ldc = N; g.sC[0] = (long)N * N;
     g.nb[0] = 2 * W;
-    if ((e = launch(g)) != cudaSuccess) return e;
+    if ((e = gemm_launch(h, g, st)) != cudaSuccess) return e;
   }
   {  // Gam[:, k-block] -= P[:, k-block of n] A[k]^dagger
     ZGemm g = gemm_init(N, M, n, 0, 2);
@@ -1182,7 +1175,7 @@ cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st) {
     g.nb[0] = 2 * W; g.nb[1] = nk;
     g.alpha = zmake(-1.0, 0.0);
     g.beta = zmake(1.0, 0.0);
-    if ((e = launch(g)) != cudaSuccess) return e;
+    if ((e = gemm_launch(h, g, st)) != cudaSuccess) return e;
   }
   {  // grad_phi = Gam^H Sinv^H  (NM x N)
     ZGemm g = gemm_init(NM, N, N, 2, 2);
@@ -1190,7 +1183,7 @@ cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st) {
     g.B = h->Sinv; g.ldb = N; g.sB[0] = (long)N * N;
     g.C = grad_phi; g.ldc = N; g.sC[0] = (long)NM * N;
     g.nb[0] = 2 * W;
-    if ((e = launch(g)) != cudaSuccess) return e;
+    if ((e = gemm_launch(h, g, st)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

@@ -112,11 +112,7 @@ cudaError_t local_energy(afqmc_kp* h, const zc* phi, zc* eloc, cudaStream_t st);
 cudaError_t local_energy_backward(afqmc_kp* h, const zc* phi, const zc* grad_e, zc* grad_phi,
                                   zc* grad_h1, cudaStream_t st);
 // pieces shared with the mixed path
-cudaError_t grad_h1(afqmc_kp* h, const zc* grad_e, zc* grad_h1, cudaStream_t st);   // from Gh
-cudaError_t project_gamma(afqmc_kp* h, zc* grad_phi, cudaStream_t st);      // Gam, Gh, Sinv
 cudaError_t overlap_lu(afqmc_kp* h, const zc* phi, zc* ld, int* sing, int want_inv, cudaStream_t st);
-cudaError_t overlap_only(afqmc_kp* h, const zc* phi, cudaStream_t st);
-cudaError_t lu_only(afqmc_kp* h, zc* ld, int* sing, int want_inv, cudaStream_t st);
 cudaError_t weights(afqmc_kp* h, const zc* phi, const double* x, double* w, zc* logdet, cudaStream_t st);
 cudaError_t qr_with(afqmc_kp* h, zc* phi, zc* scratch, cudaStream_t st);
 cudaError_t qr_launch(zc* phi, zc* scratch, int rows, int cols, int nmat, cudaStream_t st);

@@ -939,8 +939,8 @@ __global__ void onebody_in_kernel(const zc* phi, const float2* dhalf, float2* co
   if (threadIdx.x == 0) atomic_max_pos(mx + w, (double)m);
 }
 
-// Second half step: with corr = d = phi'' - phi and p32 = phi'' (fp32) after the Taylor series, phi <- phi + d + D phi'' (the sum of fp32 corrections is added to the
-// FP64 walker once).  grid (k, ws, j-chunk of 64).  STAGE_D: both are staged in
+// Second half step: with corr = d = phi'' - phi and p32 = phi'' (fp32) after the Taylor series,
+// phi <- phi + d + D phi'' (the sum of fp32 corrections is added to the FP64 walker once).  grid (k, ws, j-chunk of 64).  STAGE_D: both are staged in
 // shared memory by one coalesced pass (rows j, orbitals contiguous), and the FP64 walker
 // (orbital rows, columns j contiguous) is updated with sixteen consecutive threads on sixteen
 // consecutive columns; without it (M too large for the second staging buffer) the threads

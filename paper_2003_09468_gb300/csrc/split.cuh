@@ -1,8 +1,8 @@
 // fp16 hi/lo operand split shared by the tensor-core GEMM operands (tc_gemm.cuh).
 //
-// A matrix enters a GEMM as four fp16 planes (hi and lo of the real and imaginary parts) of x*s, with s a power of two chosen per matrix so that the
-// largest |x*s| sits near SCALE_TARGET: far from the fp16 overflow, and high enough
-// that lo keeps its full 11 bits.
+// A matrix enters a GEMM as four fp16 planes (hi and lo of the real and imaginary parts) of x*s, with
+// s a power of two chosen per matrix so that the largest |x*s| sits near SCALE_TARGET: far from the
+// fp16 overflow, and high enough that lo keeps its full 11 bits.
 #pragma once
 
 #include <cuda_fp16.h>
