@@ -75,12 +75,13 @@ def reference(Ad, phi):
     return mag + 1j * np.angle(sign), np.sum(np.abs(np.linalg.inv(S)).T * terms)
 
 
-@pytest.mark.parametrize("kind", ["near", "random", "graded"])
-@pytest.mark.parametrize("name", list(SIZES))
+CASES = [(name, kind) for name, (_, nocc, M) in SIZES.items() for kind in ("near", "random", "graded")
+         if kind != "graded" or M >= 2 * nocc]
+
+
+@pytest.mark.parametrize("name,kind", CASES)
 def test_log_det(name, kind):
     sp = spec(*SIZES[name])
-    if kind == "graded" and sp.M < 2 * sp.nocc:
-        pytest.skip("the graded rows leave fewer rows than columns")
     sys_, osys = make(sp, "mixed")
     Ad = osys.A_dense()
     for call, (phi, ld) in calls(sys_, walkers(sp, kind), kind).items():
